@@ -41,7 +41,7 @@ def listed():
         {"name": "molecules_ri", "kind": "molecules", "algo": RI, "targets": 200, "pats": 1000},
         {"name": "molecules_sifc", "kind": "molecules", "algo": SIFC, "targets": 121, "pats": 601},
         # a batch of queries of 8 to 128 vertices on one large interaction network
-        {"name": "network_ri", "kind": "network", "algo": RI, "n": 100000, "degree": 16, "labels": 64, "pats": 256,
+        {"name": "network_ri", "kind": "network", "algo": RI, "n": 100000, "degree": 16, "labels": 64, "pats": 160,
          "k_lo": 8, "k_hi": 128, "serve": False},
         {"name": "network_sifc", "kind": "network", "algo": SIFC, "n": 70001, "degree": 16, "labels": 64, "pats": 64,
          "k_lo": 8, "k_hi": 96, "serve": False},
@@ -231,7 +231,7 @@ def _admit(E, tid, algo, make, lo, hi, tries, key="states"):
     for _ in range(tries):
         g = make()
         pid = E.load_pattern(g)
-        res = E.count(tid, pid, check=False, algo=algo, state_budget=4 * max(hi, 1 << 24))
+        res = E.count(tid, pid, check=False, algo=algo, state_budget=2 * max(hi, 1 << 20))
         size = res[key] if res["rc"] == 0 else hi + 1
         if size <= hi and (best is None or size > best[0]):
             if best is not None:
@@ -293,7 +293,7 @@ def prepare(case, seed):
         f = (i + 0.5) / case["pats"]   # sizes spread over the range, log-uniformly
         k = int(round(case["k_lo"] * (case["k_hi"] / case["k_lo"]) ** f))
         make = _walk_pattern if kind == "directed" else _dense_pattern
-        p, pid = _admit(E, tid, algo, lambda: make(r, g, rows, k), lo, hi, 40 if kind == "dense" else 12)
+        p, pid = _admit(E, tid, algo, lambda: make(r, g, rows, k), lo, hi, 40 if kind == "dense" else 8)
         pats.append(p)
         pids.append(pid)
     if kind == "dense" and case["load"]:   # the job starts from host arrays
