@@ -43,7 +43,7 @@ constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device 
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
 constexpr int POOL_CELLS = 1 << 15;
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
-constexpr int ROOT_CHUNK = 1024;                 // root candidates per root range frame
+constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
 constexpr int BLOCK_FIXPOINT_MAX_N = 16384;      // auto domain mode: in-block fixpoint for targets up to this
 constexpr long long LABEL_TABLE_MAX = 1ll << 26; // most (vertex, label) entries of a target's degree table
 constexpr int LIST_FIXPOINT_MIN_JOBS = 32;      // auto domain mode, small targets: in-block fixpoint over lists from
@@ -285,10 +285,13 @@ struct TargetRec {
     DevBuf rowptr, col, elab, irowptr, icol, ielab, vld, indeg, adj, hub_slot, hub_bits, hub_list;
     DevBuf ltab;           // distinct labels, then the per-(label, vertex) largest neighbour degree
     int nlab = 0, ltab_off = 0;
+    long long labs_at = 0;         // directed targets with runs: the distinct labels' place in `runs`
     int maxdeg = 0;                // longest out- or in-row
     std::vector<int32_t> labs_h;   // host copy of the distinct labels (ascending)
     DevBuf lbk;            // large targets: label buckets (vertices, their degrees, bucket starts)
     DevBuf ldm;            // small undirected targets: label-degree masks
+    DevBuf runs;           // label-grouped rows: a LabelRuns record, then its arrays
+    int maxrun = 0;        // longest label run
     TargetView view() const {
         TargetView v;
         v.n = n;
@@ -305,24 +308,25 @@ struct TargetRec {
         v.adj = adj.p ? adj.as<uint64_t>() : nullptr;
         v.hub_slot = hub_slot.p ? hub_slot.as<int32_t>() : nullptr;
         v.hub_bits = hub_bits.p ? hub_bits.as<uint64_t>() : nullptr;
-        v.labs = ltab.p ? ltab.as<int32_t>() : nullptr;
+        v.labs = ltab.p ? ltab.as<int32_t>() : runs.p ? runs.as<int32_t>() + labs_at : nullptr;
         v.nbmax = ltab.p ? ltab.as<int32_t>() + ltab_off : nullptr;
-        v.nlab = ltab.p ? nlab : 0;
+        v.nlab = v.labs ? nlab : 0;
         v.maxdeg = maxdeg;
         v.lbuck = lbk.p ? lbk.as<int32_t>() : nullptr;
         v.lbdeg = lbk.p ? lbk.as<int32_t>() + n : nullptr;
         v.lbstart = lbk.p ? lbk.as<int32_t>() + 2 * (size_t)n : nullptr;
         v.ldm = ldm.p ? ldm.as<uint64_t>() : nullptr;
+        v.runs = runs.p ? runs.as<LabelRuns>() : nullptr;
         return v;
     }
     void use_cache(BlockCache *c) {
         for (DevBuf *b : {&rowptr, &col, &elab, &irowptr, &icol, &ielab, &vld, &indeg, &adj, &hub_slot, &hub_bits,
-                          &hub_list, &ltab, &lbk, &ldm})
+                          &hub_list, &ltab, &lbk, &ldm, &runs})
             b->cache = c;
     }
     void release() {
         for (DevBuf *b : {&rowptr, &col, &elab, &irowptr, &icol, &ielab, &vld, &indeg, &adj, &hub_slot, &hub_bits,
-                          &hub_list, &ltab, &lbk, &ldm})
+                          &hub_list, &ltab, &lbk, &ldm, &runs})
             b->release();
     }
     ~TargetRec() { release(); }
@@ -598,9 +602,11 @@ void gcf_order(const PatternRec &P, int algo, const long long *dsize, std::vecto
 
 // Position tables of one search from its ordering (rules 2-4 per position),
 // written to caller-provided arrays: pos[k] and back[] (at most k(k-1)/2
-// entries).  Returns the number of back edges.
+// entries, twice that for a directed pattern: one per arc).  Returns the number of
+// back edges.  `loop_free`: the target is known to have no self-loop, so a candidate
+// next to an image cannot be that image and rule 1 skips such positions.
 int build_positions_into(const PatView &P, const int *mu, const int *par, int algo, const long long *dsize, int n,
-                         PosInfo *pos, BackEdge *back) {
+                         PosInfo *pos, BackEdge *back, bool loop_free) {
     const int k = P.k;
     int nb = 0;
     for (int i = 0; i < k; ++i) {
@@ -625,7 +631,8 @@ int build_positions_into(const PatView &P, const int *mu, const int *par, int al
             p.ucnt = algo == SGE_RI ? n : (int)dsize[v];
         }
         for (int j = 0; j < i; ++j)
-            if (P.lab[mu[j]] == p.lab) p.same[j >> 6] |= 1ull << (j & 63);
+            if (P.lab[mu[j]] == p.lab && !(loop_free && ((P.nb[2 * (size_t)v + (mu[j] >> 6)] >> (mu[j] & 63)) & 1ull)))
+                p.same[j >> 6] |= 1ull << (j & 63);
         p.bbeg = nb;
         for (int j = 0; j < i; ++j) {
             const int w = mu[j];
@@ -637,11 +644,8 @@ int build_positions_into(const PatView &P, const int *mu, const int *par, int al
                 if (p.flags & POS_IN_ROW) need_out = false; else need_in = false;
                 if (!need_out && !need_in) continue;
             }
-            BackEdge &be = back[nb++];
-            be.pos = j;
-            be.dir = P.directed ? ((need_out ? 1 : 0) | (need_in ? 2 : 0)) : 1;
-            be.lab_out = need_out ? lo : 0;
-            be.lab_in = need_in ? li : 0;
+            if (need_out || !P.directed) back[nb++] = BackEdge{j, 1, lo, 0};
+            if (need_in && P.directed) back[nb++] = BackEdge{j, 2, 0, li};
         }
         p.bcnt = nb - p.bbeg;
     }
@@ -652,8 +656,8 @@ void build_positions(const PatternRec &P, const std::vector<int> &mu, const std:
                      const long long *dsize, int n, std::vector<PosInfo> &pos, std::vector<BackEdge> &back) {
     const int k = P.k;
     pos.resize(k);
-    back.resize((size_t)k * (k > 0 ? k - 1 : 0) / 2 + 1);
-    const int nb = build_positions_into(P.core(), mu.data(), par.data(), algo, dsize, n, pos.data(), back.data());
+    back.resize((size_t)k * (k > 0 ? k - 1 : 0) / (P.directed ? 1 : 2) + 1);
+    const int nb = build_positions_into(P.core(), mu.data(), par.data(), algo, dsize, n, pos.data(), back.data(), true);
     back.resize(nb);
 }
 
@@ -809,11 +813,11 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     const int nj = (int)idx.size();
     std::vector<Job> &jobs = W.hjobs;   // kept across calls (no fresh pages)
     if (jobs.size() < (size_t)nj) jobs.resize((size_t)nj);
-    bool directed = false, any_elab = false;
+    bool directed = false, any_elab = false, any_runs = false;
     int kmax = 1, nmax = 1, max_pid = 0;
     std::mutex red;   // merges the threads' partial maxima
     parallel_for(nj, [&](int q0, int q1) {
-        bool el = false;
+        bool el = false, rn = false;
         int km = 1, nm = 1, mp = 0;
         for (int q = q0; q < q1; ++q) {
             Job &J = jobs[q];
@@ -835,6 +839,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                 km = std::max(km, J.p->k);
                 nm = std::max(nm, J.t->n);
                 el = el || J.t->any_elab || J.p->any_elab;
+                rn = rn || J.t->cached.runs != nullptr;
             }
         }
         std::lock_guard<std::mutex> g(red);
@@ -842,6 +847,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         nmax = std::max(nmax, nm);
         max_pid = std::max(max_pid, mp);
         any_elab = any_elab || el;
+        any_runs = any_runs || rn;
     });
     if (nj > 0) directed = jobs[0].t->directed;   // (a group holds pairs of one directedness)
     // kernel family: the bitset kernel needs undirected, unlabelled edges, an
@@ -908,25 +914,27 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     std::vector<int> fjobs;  // jobs with a filter block, in order
     for (int q = 0; q < nj; ++q)
         if (jobs[q].active && jobs[q].filt_off >= 0) fjobs.push_back(q);
-    // RI-DS jobs on targets with a label-degree table (undirected, no edge labels in the batch):
-    // their pattern vertices' label indices among the target's labels, written on the device
-    // below into one array indexed like the domain sizes (job's vertex offset + vertex)
+    // jobs on targets with label runs, and RI-DS jobs on targets with a label-degree table
+    // (undirected, no edge labels in the batch): their pattern vertices' label indices among
+    // the target's labels, written on the device below
     bool any_plidx = false;
-    if (!any_elab && !directed) {
+    const bool table = algo != SGE_RI && !any_elab && !directed;
+    if (any_runs || table) {
+        auto wants = [&](const Job &J) {
+            return J.active && (J.t->cached.runs != nullptr || (table && !J.t->labs_h.empty()));
+        };
         long long g = 0;
-        for (int q : fjobs) {
-            const Job &J = jobs[q];
-            if (J.algo != SGE_RI && !J.t->labs_h.empty()) any_plidx = true;
-            g += J.p->k;
-        }
-        if (any_plidx) {
-            CK(W.plidx.ensure((size_t)std::max<long long>(g, 1) * 4), "alloc label indices");
+        for (int q = 0; q < nj; ++q)
+            if (wants(jobs[q])) g += jobs[q].p->k;
+        if (g > 0) {
+            any_plidx = true;
+            CK(W.plidx.ensure((size_t)g * 4), "alloc label indices");
             g = 0;
-            for (int q : fjobs) {
-                const Job &J = jobs[q];
-                if (J.algo != SGE_RI && !J.t->labs_h.empty()) desc[q].plidx = W.plidx.as<int32_t>() + g;
-                g += J.p->k;
-            }
+            for (int q = 0; q < nj; ++q)
+                if (wants(jobs[q])) {
+                    desc[q].plidx = W.plidx.as<int32_t>() + g;
+                    g += jobs[q].p->k;
+                }
         }
     }
     bool any_buckets = false;
@@ -957,7 +965,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         CK(upload(W.unit_off, unit_off, st), "upload unit offsets");
         CK(upload(W.vert_off, vert_off, st), "upload vertex offsets");
         if (any_plidx) {
-            CK(launch_label_index(W.fjobs.as<JobDesc>(), W.vert_off.as<long long>(), nf, nverts, st), "label indices");
+            CK(launch_label_index(W.fjobs.as<JobDesc>(), nf, st), "label indices");
             ++launches;
         }
         CK(W.sizes.ensure((size_t)nverts * 8), "alloc sizes");
@@ -1316,7 +1324,8 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             D.back = W.back.as<BackEdge>() + back_off[q];
             if (jobs[q].active) {
                 // can a position after the first have more than SPLIT_RANGE candidates?
-                bool longl = jobs[q].t->maxdeg == 0 || jobs[q].t->maxdeg > SPLIT_RANGE;
+                const TargetRec &T = *jobs[q].t;
+                bool longl = T.cached.runs ? T.maxrun > SPLIT_RUN_RANGE : T.maxdeg == 0 || T.maxdeg > SPLIT_RANGE;
                 for (int i = 1; i < D.k && !longl; ++i) {
                     const PosInfo &P = pos[(size_t)pos_off[q] + i];
                     longl = P.par < 0 && ((D.flags & JOB_RIDS) ? (long long)P.ucnt : jobs[q].t->n) > SPLIT_RANGE;
@@ -1332,6 +1341,10 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     });
     const double t_up = now_ms();
     CK(upload(W.jobs, desc, st), "upload jobs");
+    if (any_plidx && nf == 0) {   // (with domains they are there already)
+        CK(launch_label_index(W.jobs.as<JobDesc>(), nj, st), "label indices");
+        ++launches;
+    }
     const double t_pre = now_ms();
     if (trace_on()) std::fprintf(stderr, "[sge] job records uploaded in %.3f ms\n", t_pre - t_up);
 
@@ -1345,20 +1358,25 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     const long long resident_warps = (long long)ctx->sms * occ * search_warps_per_block();
     const long long fpw = o.frames_per_warp > 0 ? o.frames_per_warp : 8;
     const long long target_frames = fpw * resident_warps * shard_count;
-    // roots: one frame per active job, cut into ranges of ROOT_CHUNK candidates
-    // when the root has more (a range frame counts the node's states only if it
-    // starts at candidate 0)
+    // roots: one frame per active job, cut into ranges when the root has more candidates
+    // (a range frame counts the node's states only if it starts at candidate 0): of as
+    // few as spread the call's root candidates over the resident warps, 32 to ROOT_CHUNK (a
+    // single 1,000-vertex root scanned by one warp took 40 us, the first level's whole time)
     std::vector<std::array<int32_t, 4>> roots;
     roots.reserve((size_t)nj);
+    long long nroot = 0;
+    for (int q = 0; q < nj; ++q)
+        if (const Job &J = jobs[q]; J.active) nroot += J.algo == SGE_RI ? J.t->n : pos[pos_off[q]].ucnt;
+    const long long chunk = std::min<long long>(ROOT_CHUNK, std::max<long long>(32, (nroot / resident_warps + 31) & ~31ll));
     for (int q = 0; q < nj; ++q) {
         const Job &J = jobs[q];
         if (!J.active) continue;
         const long long len = J.algo == SGE_RI ? J.t->n : pos[pos_off[q]].ucnt;
-        if (len <= ROOT_CHUNK) {
+        if (len <= chunk) {
             roots.push_back({q, 0, -1, -1});
         } else {
-            for (long long b = 0; b < len; b += ROOT_CHUNK)
-                roots.push_back({q, 0, (int32_t)b, (int32_t)std::min<long long>(b + ROOT_CHUNK, len)});
+            for (long long b = 0; b < len; b += chunk)
+                roots.push_back({q, 0, (int32_t)b, (int32_t)std::min<long long>(b + chunk, len)});
         }
     }
     long long F0 = (long long)roots.size();
@@ -1666,6 +1684,12 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             CK(take(C.ckpt, (long long)nd, cs, cs), "read checkpoint frames");
             // frontier frames of this shard never taken (frame i of the shard is frame i*count+index)
             const long long taken = std::min<long long>((long long)hc[0], nfront);
+            // (ranges of label runs become row ranges first, in the frontier and in the queue)
+            int32_t *rest = W.front[cur].as<int32_t>() + (taken * shard_count + shard_index) * (long long)fstride;
+            CK(launch_frames_to_rows(W.jobs.as<JobDesc>(), rest, nfront - taken, (long long)fstride * shard_count,
+                                     nullptr, directed ? 1 : 0, st), "frontier ranges");
+            CK(launch_frames_to_rows(W.jobs.as<JobDesc>(), W.pool.as<int32_t>(), POOL_CELLS, POOL_STRIDE,
+                                     W.pseq.as<unsigned long long>(), directed ? 1 : 0, st), "queue ranges");
             CK(take(C.front + (taken * shard_count + shard_index) * (long long)fstride, nfront - taken, fstride,
                     (long long)fstride * shard_count), "read frontier");
             // queued frames never taken: the cells left published (sequence word = ticket + 1)
@@ -2183,17 +2207,69 @@ sge_status sge_load_target(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *sr
     int32_t *d_maxdeg = I.small.as<int32_t>() + 3;   // (zeroed with the ingest flags)
     CK(launch_ingest_maxdeg(T->rowptr.as<int32_t>(), n, d_maxdeg, st), "longest row");
     if (directed) CK(launch_ingest_maxdeg(T->irowptr.as<int32_t>(), n, d_maxdeg, st), "longest row");
+    const bool want_runs = n > 0 && (directed ? m : arcs) >= (long long)RUNS_MIN_MEAN_ROW * n;
+    int32_t *d_maxrun = I.small.as<int32_t>() + 4;   // (zeroed with the ingest flags)
+    // label runs: the rows regrouped by neighbour label (lidx: label indices on the device)
+    auto build_runs = [&](const std::vector<int32_t> &labs, const int32_t *d_lidx) -> cudaError_t {
+        const long long L = (long long)labs.size(), rows = (long long)n * (L + 1);
+        if (!want_runs || rows > LABEL_TABLE_MAX) return cudaSuccess;
+        const long long cap[2] = {std::max<long long>(directed ? m : arcs, 1), directed ? std::max<long long>(m, 1) : 0};
+        auto pad = [](long long ints) { return (ints + 3) & ~3ll; };
+        // the record (32 ints), the labels when no label table holds them, then run, col, elab per direction
+        long long at = 32, labs_at = 0, part[2][3];
+        if (directed) {
+            labs_at = at;
+            at += pad(L);
+        }
+        for (int d = 0; d < (directed ? 2 : 1); ++d) {
+            part[d][0] = at;
+            part[d][1] = part[d][0] + pad(rows);
+            part[d][2] = part[d][1] + 2 * pad(cap[d]);
+            at = part[d][2] + pad(cap[d]);
+        }
+        cudaError_t e = T->runs.ensure((size_t)at * 4);
+        if (e != cudaSuccess) return e;
+        int32_t *b = T->runs.as<int32_t>();
+        LabelRuns R;
+        std::memset(&R, 0, sizeof(R));
+        const int di = directed ? 1 : 0;
+        R.run = b + part[0][0]; R.col = reinterpret_cast<int2 *>(b + part[0][1]); R.elab = b + part[0][2];
+        R.irun = b + part[di][0]; R.icol = reinterpret_cast<int2 *>(b + part[di][1]); R.ielab = b + part[di][2];
+        R.stride = (int32_t)L + 1;
+        static_assert(sizeof(LabelRuns) <= 128, "the record's place holds it");
+        e = cudaMemcpyAsync(b, &R, sizeof(R), cudaMemcpyHostToDevice, st);
+        if (directed) {
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(b + labs_at, labs.data(), (size_t)L * 4, cudaMemcpyHostToDevice, st);
+            T->labs_at = labs_at;
+            T->nlab = (int)L;
+        }
+        for (int d = 0; d < (directed ? 2 : 1) && e == cudaSuccess; ++d)
+            e = launch_label_runs((d ? T->irowptr : T->rowptr).as<int32_t>(), (d ? T->icol : T->col).as<int32_t>(),
+                                  (d ? T->ielab : T->elab).as<int32_t>(), T->vld.as<int2>(), d_lidx, n, (int)L,
+                                  b + part[d][0], reinterpret_cast<int2 *>(b + part[d][1]), b + part[d][2], d_maxrun,
+                                  st);
+        return e;
+    };
+    std::vector<int32_t> labs, lidx;
+    if (n > 0 && (!directed || want_runs)) {
+        labs.assign(vlabel, vlabel + n);
+        std::sort(labs.begin(), labs.end());
+        labs.erase(std::unique(labs.begin(), labs.end()), labs.end());
+        lidx.resize((size_t)n);
+        for (int v = 0; v < n; ++v)
+            lidx[(size_t)v] = (int32_t)(std::lower_bound(labs.begin(), labs.end(), vlabel[v]) - labs.begin());
+    }
+    if (directed && want_runs) {
+        CK(cudaMemcpyAsync(I.fill_out.p, lidx.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st),
+           "upload label indices");
+        CK(build_runs(labs, I.fill_out.as<int32_t>()), "label runs");
+    }
     if (!directed && n > 0) {
         // the largest neighbour degree per (vertex, label): domain initialisation reads it to
         // drop, at once, the candidates that have no neighbour able to carry some pattern edge
-        std::vector<int32_t> labs(vlabel, vlabel + n);
-        std::sort(labs.begin(), labs.end());
-        labs.erase(std::unique(labs.begin(), labs.end()), labs.end());
         const long long L = (long long)labs.size();
         if ((long long)n * L <= LABEL_TABLE_MAX) {
-            std::vector<int32_t> lidx((size_t)n);
-            for (int v = 0; v < n; ++v)
-                lidx[(size_t)v] = (int32_t)(std::lower_bound(labs.begin(), labs.end(), vlabel[v]) - labs.begin());
             T->nlab = (int)L;
             T->labs_h = labs;
             T->ltab_off = (int)((L + 3) & ~3LL);
@@ -2204,6 +2280,7 @@ sge_status sge_load_target(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *sr
             CK(launch_label_nbmax(T->rowptr.as<int32_t>(), T->col.as<int32_t>(), T->vld.as<int2>(),
                                   I.fill_out.as<int32_t>(), n, (int)L, T->ltab.as<int32_t>() + T->ltab_off, st),
                "label table");
+            CK(build_runs(labs, I.fill_out.as<int32_t>()), "label runs");
             const long long ldm_words = L * LDM_DEGREES * T->dw;
             if (n <= LDM_MAX_N && ldm_words <= LDM_MAX_WORDS) {
                 CK(T->ldm.ensure((size_t)ldm_words * 8), "alloc label-degree masks");
@@ -2245,11 +2322,12 @@ sge_status sge_load_target(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *sr
         CK(launch_ingest_bits(T->rowptr.as<int32_t>(), T->col.as<int32_t>(), n, T->dw, T->adj.as<uint64_t>(), st),
            "adjacency bitset");
     }
-    int32_t hsmall[4] = {0, 0, 0, 0};   // flags, long out-rows, long in-rows, longest row
+    int32_t hsmall[5] = {0, 0, 0, 0, 0};   // flags, long out-rows, long in-rows, longest row, longest run
     CK(cudaMemcpyAsync(hsmall, flags, sizeof(hsmall), cudaMemcpyDeviceToHost, st), "read ingest flags");
     CK(cudaStreamSynchronize(st), "target ingest");
     const int hflags = hsmall[0];
     T->maxdeg = hsmall[3];
+    T->maxrun = hsmall[4];
     const char *bad = (hflags & ING_RANGE) ? "edge endpoint out of range"
                       : (hflags & ING_LOOP) ? "self-loop"
                       : (hflags & ING_LABEL) ? "repeated edge with a different label" : nullptr;
@@ -2571,7 +2649,7 @@ sge_status sge_count_noalloc(int32_t n, const int32_t *d_rowptr, const int32_t *
     gcf_order_into(P, SGE_RI, nullptr, mu, par);
     PosInfo *pos = hbuf->pos;
     BackEdge *back = hbuf->back;
-    const int nb = build_positions_into(P, mu, par, SGE_RI, nullptr, n, pos, back);
+    const int nb = build_positions_into(P, mu, par, SGE_RI, nullptr, n, pos, back, false);
 
     void *base = nullptr;
     size_t cap = 0;

@@ -233,6 +233,65 @@ __global__ void __launch_bounds__(IB) k_label_nbmax(const int32_t *rowptr, const
         }
 }
 
+// Label runs: one warp per vertex regroups its row by the neighbours' label index, ids
+// ascending within a label -- a counting sort whose counters are the vertex's own slots of
+// the run table: count, scan to the runs' ends, then place the row from its last entry
+// back, each slot counting down to its run's start.  Bound by the row's reads and the
+// serial 32-entry steps of the longest row (a 1,256-neighbour hub: 40 steps twice).
+__global__ void __launch_bounds__(IB) k_label_runs(const int32_t *rowptr, const int32_t *col, const int32_t *elab,
+                                                   const int2 *vld, const int32_t *lidx, int n, int nlab, int32_t *run,
+                                                   int2 *rcol, int32_t *relab, int32_t *maxrun) {
+    const int lane = threadIdx.x & 31;
+    const long long w0 = (blockIdx.x * (long long)IB + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * IB) >> 5;
+    int longest = 0;
+    for (long long v = w0; v < n; v += nw) {
+        volatile int32_t *slot = run + (size_t)v * (nlab + 1);
+        const int b = rowptr[v], e = rowptr[v + 1];
+        for (int l = lane; l <= nlab; l += 32) slot[l] = l == nlab ? e : 0;
+        __syncwarp();
+        for (int x0 = b; x0 < e; x0 += 32) {
+            const int x = x0 + lane;
+            const int l = x < e ? lidx[col[x]] : -1;
+            const unsigned peers = __match_any_sync(FULLMASK, l);
+            if (l >= 0 && (peers >> lane) == 1u) slot[l] = slot[l] + __popc(peers);
+            __syncwarp();
+        }
+        int before = b;
+        for (int l0 = 0; l0 < nlab; l0 += 32) {
+            const int l = l0 + lane;
+            const int c = l < nlab ? slot[l] : 0;
+            longest = max(longest, c);
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULLMASK, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (l < nlab) slot[l] = before + incl;
+            before += __shfl_sync(FULLMASK, incl, 31);
+        }
+        __syncwarp();
+        for (int x1 = e; x1 > b; x1 -= 32) {   // entries (x1 - 32, x1], the last ones first
+            const int x = x1 - 1 - lane;
+            const int y = x >= b ? col[x] : -1;
+            const int l = y >= 0 ? lidx[y] : -1;
+            const unsigned peers = __match_any_sync(FULLMASK, l);
+            const int end = l >= 0 ? slot[l] : 0;
+            __syncwarp();
+            if (l >= 0) {
+                const int at = end - 1 - __popc(peers & ((1u << lane) - 1u));
+                rcol[at] = make_int2(y, vld[y].y);
+                relab[at] = elab[x];
+                if ((peers >> lane) == 1u) slot[l] = at;   // the peers' lowest place
+            }
+            __syncwarp();
+        }
+    }
+    longest = (int)__reduce_max_sync(FULLMASK, (unsigned)longest);
+    if (lane == 0 && longest > 0) atomicMax(maxrun, longest);
+}
+
 // Label-degree masks: one warp per (label index, degree threshold, 64-vertex word), two
 // ballots over the word's vertices.
 __global__ void __launch_bounds__(IB) k_label_degree_masks(const int2 *vld, int n, const int32_t *labs, long long units,
@@ -265,6 +324,15 @@ cudaError_t launch_label_degree_masks(const int2 *vld, int n, const int32_t *lab
     const long long units = (long long)nlab * LDM_DEGREES * dw;
     if (units <= 0) return cudaSuccess;
     k_label_degree_masks<<<blocks_for(units * 32, IB), IB, 0, st>>>(vld, n, labs, units, dw, ldm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_label_runs(const int32_t *rowptr, const int32_t *col, const int32_t *elab, const int2 *vld,
+                              const int32_t *lidx, int n, int nlab, int32_t *run, int2 *rcol, int32_t *relab, int32_t *maxrun,
+                              cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_label_runs<<<blocks_for((long long)n * 32, IB), IB, 0, st>>>(rowptr, col, elab, vld, lidx, n, nlab, run, rcol,
+                                                                   relab, maxrun);
     return cudaGetLastError();
 }
 

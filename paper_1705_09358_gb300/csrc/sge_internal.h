@@ -29,6 +29,10 @@ constexpr int POOL_STRIDE = FRAME_HDR + KMAX;
 // the survivors to search below them.  Checkpoints write such frames.
 constexpr int FRAME_COUNTED = 1 << 16;
 constexpr int FRAME_DEPTH_MASK = FRAME_COUNTED - 1;
+// Flag in a frame's depth word, inside one launch sequence only: [begin, end) counts
+// in the node's chosen label run (see LabelRuns), not in the parent's row.  Checkpoints
+// hold row ranges: k_frames_to_rows and the dump code translate.
+constexpr int FRAME_RUN = 1 << 17;
 
 // PosInfo.flags
 constexpr int POS_IN_ROW = 1;        // candidates come from the parent's in-row (directed)
@@ -47,6 +51,7 @@ constexpr int JOB_LONG_LISTS = 16;   // some position after the first may have m
 // The breadth-first split writes a child whose candidate list is longer than
 // this as range frames of this many candidates each.
 constexpr int SPLIT_RANGE = 256;
+constexpr int SPLIT_RUN_RANGE = 1024;   // ... or as this many entries of a label run
 
 // One search position i of a job: pattern vertex mu_i and its constraints.
 struct PosInfo {
@@ -72,6 +77,21 @@ struct BackEdge {
     int32_t dir;      // bit 0: arc mu_i -> mu_j needed; bit 1: arc mu_j -> mu_i needed
     int32_t lab_out;  // label of mu_i -> mu_j (undirected: the edge label)
     int32_t lab_in;   // label of mu_j -> mu_i
+};
+
+// The rows of a target grouped by neighbour label: row v's neighbours with label
+// index l, ascending by id, are entries run[v * stride + l] .. run[v * stride + l + 1].
+// A search node's candidates are then the shortest such run among the rows of all
+// its earlier neighbours' images instead of the parent's whole row: rule 2 holds by
+// construction and most of rule 4 by starting from the shortest list.
+struct LabelRuns {
+    // out-rows (undirected: all neighbours): run starts, then per entry {neighbour, its out-degree}
+    // (one load gives what rules 2 and 3 need) and the edge's label; in-rows likewise
+    // (undirected: the same arrays)
+    const int32_t *run, *elab, *irun, *ielab;
+    const int2 *col, *icol;
+    int32_t stride;                       // distinct labels + 1
+    int32_t pad;
 };
 
 struct TargetView {
@@ -105,7 +125,13 @@ struct TargetView {
     // mask of the vertices with label l and degree at least d, at ldm[(l * LDM_DEGREES + d) * dw];
     // null otherwise.  Domain initialisation without the neighbour-label test copies a row.
     const uint64_t *ldm;
+    const LabelRuns *runs;      // label-grouped rows, or null (short rows, or too many labels)
 };
+
+// Targets get label runs when their mean stored row has at least this many entries: on the
+// molecule shape (rows of 1-4) a run saves nothing over the row and costs a table look-up
+// (and the table itself: 8 bytes per arc more, 4 (labels + 1) per vertex).
+constexpr int RUNS_MIN_MEAN_ROW = 4;
 
 constexpr int LDM_DEGREES = 17;          // degree thresholds 0..16 in a target's label-degree masks
 constexpr int LDM_MAX_N = 4096;          // targets up to this many vertices get the masks ...
@@ -132,8 +158,8 @@ struct JobDesc {
     const BackEdge *back;
     uint64_t *filt;             // k x t.dw words: D(v) / label-degree filter, or null
     const int32_t *ulist;       // candidate lists of unparented RI-DS positions
-    const int32_t *plidx;       // RI-DS on a target with nbmax: each pattern vertex's label index among
-                                // the target's labels (-1: absent), else null
+    const int32_t *plidx;       // on a target with label runs, or RI-DS on one with nbmax: each pattern
+                                // vertex's label index among the target's labels (-1: absent), else null
     int32_t k;
     int32_t flags;
     unsigned long long *ctr;    // [4]: matches, states, nodes, hash
@@ -200,9 +226,8 @@ inline void bind_control(SearchCtl &C, void *block) {
 // ------------------------------------------------------------ launchers
 // (implemented in sge_kernels.cu; all launch on `st`)
 
-// plidx of every job that has one: its pattern vertices' label indices (thread per vertex).
-cudaError_t launch_label_index(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
-                               cudaStream_t st);
+// plidx of every job that has one: its pattern vertices' label indices (block per job).
+cudaError_t launch_label_index(const JobDesc *jobs, int njobs, cudaStream_t st);
 // Initial domains of the jobs whose targets have label buckets (their filter words already
 // zeroed): one warp per (job, pattern vertex), setting the bits of the bucket prefix.
 cudaError_t launch_domain_init_buckets(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
@@ -258,6 +283,12 @@ size_t search_smem_bytes(int kernel, int kmax, int nwl);
 // Global scratch the search kernel needs for a grid of `grid` blocks.
 size_t search_slab_bytes(int kernel, int kmax, int nwl, long long grid);
 
+// Checkpoint frames in place: label-run ranges (FRAME_RUN) become ranges of the parent's row.
+// Frames 0, 1, .. of `frames`, `pitch` ints apart; with `seq` non-null only the published
+// queue cells (sequence word = ticket + 1) of a queue of n cells.
+cudaError_t launch_frames_to_rows(const JobDesc *jobs, int32_t *frames, long long n, long long pitch,
+                                  const unsigned long long *seq, int directed, cudaStream_t st);
+
 // Adjacency bitset rows of the hub vertices `hubs[0..h)` (rows zeroed first).
 cudaError_t launch_build_hubs(const int32_t *rowptr, const int32_t *col, const int32_t *hubs, int h, int dw,
                               uint64_t *bits, cudaStream_t st);
@@ -292,5 +323,11 @@ cudaError_t launch_label_degree_masks(const int2 *vld, int n, const int32_t *lab
 // nbmax[lidx[y] * n + t] = max deg(y) over the neighbours y of t (nbmax zeroed first).
 cudaError_t launch_label_nbmax(const int32_t *rowptr, const int32_t *col, const int2 *vld, const int32_t *lidx, int n,
                                int nlab, int32_t *nbmax, cudaStream_t st);
+
+// Label runs of one direction (see LabelRuns): run[v * (nlab + 1) + l], col, elab and degrees
+// grouped by the label index lidx[] of the neighbour; *maxrun is raised to the longest run.
+cudaError_t launch_label_runs(const int32_t *rowptr, const int32_t *col, const int32_t *elab, const int2 *vld,
+                              const int32_t *lidx, int n, int nlab, int32_t *run, int2 *rcol, int32_t *relab, int32_t *maxrun,
+                              cudaStream_t st);
 
 }  // namespace sge

@@ -8,11 +8,12 @@
 // GPU design (not the paper's CPU work-stealing runtime):
 //  * domain kernels: one warp per 64-target bitset word; arc consistency and
 //    forward checking iterate to their joint fixpoint under a host loop;
-//  * split: breadth-first expansion of the search tree, one warp per frame,
-//    until the frontier holds enough frames for every resident warp;
+//  * split: breadth-first expansion of the search tree, up to 32 frames per
+//    warp at once, until the frontier holds enough frames for every resident warp;
 //  * persistent search: one warp owns one depth-first search.  The CSR kernel
-//    scans the candidate row 32 candidates at a time (one per lane), tests
-//    rules 1-4 per lane and compacts survivors with a ballot; the bitset kernel
+//    scans the candidate list (on targets with label runs the shortest run among
+//    the earlier neighbours' rows) 32 candidates at a time, one per lane, spreads the
+//    back-edge tests over the lanes and compacts survivors with a ballot; the bitset kernel
 //    computes a whole candidate set as the AND of the parent's adjacency row,
 //    the back-neighbours' rows and the filter D(mu_i), one 64-bit word per
 //    lane.  Idle warps take frames from the frontier, then from a bounded
@@ -189,6 +190,376 @@ __device__ __forceinline__ int find_job(const long long *off, int njobs, long lo
     return lo;
 }
 
+// ------------------------------------------------- candidates of a node
+//
+// Position i's earlier neighbours give its constraints: number 0 is the arc to
+// the parent, 1 + b back edge b (rule 4; a directed back edge names one arc).
+// Each says "the candidate is in the out- or in-row of an image".  On a target
+// with label runs a node's candidates are the shortest of its constraints'
+// runs of lab(mu_i) -- with ties the lowest-numbered constraint's, so that every
+// kernel picks the same list and a range of it means the same everywhere --
+// and the other constraints are tested; without runs they are the parent's row.
+// (On the 100k-vertex network a query's parent row holds 16 to 1,250 entries,
+// the shortest run mostly 0 to 4.)  The node's states stay the parent's row
+// length, its accepted candidates are the same set.
+
+// One position's constants in registers.
+struct PosV {
+    int pv, par, lab, odeg, ideg, pel, bb, bc, flags;
+};
+
+__device__ __forceinline__ PosV load_pos(const PosInfo *p) {
+    const int4 a = __ldg(reinterpret_cast<const int4 *>(p)), b = __ldg(reinterpret_cast<const int4 *>(p) + 1);
+    return PosV{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, __ldg(&p->flags)};
+}
+static_assert(sizeof(PosInfo) == 64 && sizeof(BackEdge) == 16, "position tables are read as 16-byte words");
+
+// A job's fields as the candidate functions read them: through its record here,
+// from registers in the CSR search (CsrJob).
+struct JobRef {
+    const JobDesc *J;
+    __device__ __forceinline__ const int32_t *rowptr() const { return J->t.rowptr; }
+    __device__ __forceinline__ const int32_t *col() const { return J->t.col; }
+    __device__ __forceinline__ const int32_t *elab() const { return J->t.elab; }
+    __device__ __forceinline__ const int32_t *irowptr() const { return J->t.irowptr; }
+    __device__ __forceinline__ const int32_t *icol() const { return J->t.icol; }
+    __device__ __forceinline__ const int32_t *ielab() const { return J->t.ielab; }
+    __device__ __forceinline__ const int32_t *hub_slot() const { return J->t.hub_slot; }
+    __device__ __forceinline__ const uint64_t *hub_bits() const { return J->t.hub_bits; }
+    __device__ __forceinline__ const uint64_t *adj() const { return J->t.adj; }
+    __device__ __forceinline__ const LabelRuns *runs() const { return J->t.runs; }
+    __device__ __forceinline__ const BackEdge *back() const { return J->back; }
+    __device__ __forceinline__ const int32_t *ulist() const { return J->ulist; }
+    __device__ __forceinline__ const int32_t *plidx() const { return J->plidx; }
+    __device__ __forceinline__ int n() const { return J->t.n; }
+    __device__ __forceinline__ int dw() const { return J->t.dw; }
+    __device__ __forceinline__ int flags() const { return J->flags; }
+};
+
+struct Con {
+    int x, in, lab;   // the candidate is in x's in-row (in != 0) or out-row, by an arc with this label
+};
+
+template <bool DIR, class V>
+__device__ __forceinline__ Con constraint(const V &v, const PosV &p, int q, const int *M) {
+    if (q == 0) return Con{M[p.par], DIR ? p.flags & POS_IN_ROW : 0, p.pel};
+    const int4 be = __ldg(reinterpret_cast<const int4 *>(v.back() + p.bb + q - 1));
+    // arc mu_i -> mu_j: the candidate is in the in-row of M_j; mu_j -> mu_i: in its out-row
+    return Con{M[be.x], DIR ? be.y & 1 : 0, DIR && (be.y & 2) ? be.w : be.z};
+}
+
+struct Cand {
+    const int32_t *ids;    // candidate e of the list is ids[base + e] (a run's, see li: the first of
+                           // {id, degree} pair base + e); null: vertex base + e
+    const int32_t *elab;   // labels beside ids (read only when edge labels are compared)
+    int base, len;
+    int raw;               // the node's raw candidates: the parent's row (its states)
+    int skip;              // constraint the list itself satisfies, -1 for an unparented position
+    int lab;               // ... and that arc's label
+    int next;              // constraint with the next shortest run, -1 if there is none
+    int li;                // label index of the position when the list is a run, else -1
+};
+
+// The unparented case (V_t, or D(mu_i) for RI-DS), and the parent's row on a target without runs.
+template <bool DIR, class V>
+__device__ __forceinline__ Cand plain_list(const V &v, const PosV &p, const PosInfo *P, const int *M) {
+    Cand S;
+    S.elab = nullptr;
+    S.li = -1;
+    S.next = -1;
+    S.lab = p.pel;
+    if (p.par < 0) {
+        S.skip = -1;
+        if (v.flags() & JOB_RIDS) {
+            S.ids = v.ulist(); S.base = __ldg(&P->uoff); S.len = __ldg(&P->ucnt);
+        } else {
+            S.ids = nullptr; S.base = 0; S.len = v.n();
+        }
+    } else {
+        const bool in = DIR && (p.flags & POS_IN_ROW);
+        const int32_t *rp = in ? v.irowptr() : v.rowptr();
+        const int a = M[p.par];
+        S.skip = 0;
+        S.ids = in ? v.icol() : v.col();
+        S.elab = in ? v.ielab() : v.elab();
+        S.base = __ldg(rp + a);
+        S.len = __ldg(rp + a + 1) - S.base;
+    }
+    S.raw = S.len;
+    return S;
+}
+
+// Start and length of constraint q's run of label index li.
+template <bool DIR, class V>
+__device__ __forceinline__ int run_of(const V &v, const LabelRuns *R, const PosV &p, int q, int li, const int *M,
+                                      int &len) {
+    const Con k = constraint<DIR>(v, p, q, M);
+    const int32_t *r = (DIR && k.in ? R->irun : R->run) + (size_t)k.x * R->stride + li;
+    const int b = __ldg(r);
+    len = __ldg(r + 1) - b;
+    return b;
+}
+
+// Candidate e of list S.
+__device__ __forceinline__ int cand_id(const Cand &S, int e) {
+    if (S.ids == nullptr) return S.base + e;
+    return __ldg(S.ids + ((size_t)(S.base + e) << (S.li >= 0 ? 1 : 0)));
+}
+
+// First entry of ascending ids[0..n) (every other word for a run) that is at least x.
+__device__ __forceinline__ int lower_bound_ids(const int32_t *ids, int n, int x, bool run = false) {
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(ids + ((size_t)mid << (run ? 1 : 0))) < x) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// The parent's row of a parented position: its entries are what a checkpoint's ranges count.
+template <bool DIR, class V>
+__device__ __forceinline__ const int32_t *parent_row(const V &v, const PosV &p, const int *M, int &len) {
+    const bool in = DIR && (p.flags & POS_IN_ROW);
+    const int32_t *rp = (in ? v.irowptr() : v.rowptr()) + M[p.par];
+    const int b = __ldg(rp);
+    len = __ldg(rp + 1) - b;
+    return (in ? v.icol() : v.col()) + b;
+}
+
+// Makes S constraint q's run.
+template <bool DIR, class V>
+__device__ __forceinline__ void set_run(const V &v, const LabelRuns *R, const PosV &p, const int *M, int q, int b,
+                                        int len, Cand &S) {
+    const Con k = constraint<DIR>(v, p, q, M);
+    S.ids = reinterpret_cast<const int32_t *>(DIR && k.in ? R->icol : R->col);
+    S.elab = DIR && k.in ? R->ielab : R->elab;
+    S.base = b;
+    S.len = len;
+    S.skip = q;
+    S.lab = k.lab;
+}
+
+// Entries of run S below the parent row's first: none of them is a candidate.  A range of a
+// run starts at or after this one, and the part that holds it counts the node's states; so
+// a later part starts later in the row too, which is how a checkpoint's row ranges tell.
+template <bool DIR, class V>
+__device__ __forceinline__ int run_drop(const V &v, const PosV &p, const Cand &S, const int *M) {
+    int n;
+    const int32_t *row = parent_row<DIR>(v, p, M, n);
+    return n > 0 ? lower_bound_ids(S.ids + 2 * (size_t)S.base, S.len, __ldg(row), true) : S.len;
+}
+
+// The candidate list of position P of a node with images M[0..], found by a group of G lanes (a
+// power of two; every lane of the warp calls, `sub` its lane within the group): the group's lanes
+// look up the constraints' runs side by side, then agree on the shortest and the next.
+template <bool DIR, class V>
+__device__ __forceinline__ Cand pick_group(const V &v, const PosV &p, const PosInfo *P, const int *M, int G, int sub) {
+    Cand S = plain_list<DIR>(v, p, P, M);
+    const LabelRuns *R = v.runs();
+    const bool runs = R != nullptr && p.par >= 0;
+    constexpr unsigned long long NONE = ~0ull;
+    unsigned long long k1 = NONE, k2 = NONE;   // (length, constraint) of the shortest and next run
+    int b1 = 0;
+    if (runs) {
+        S.li = v.plidx()[p.pv];
+        if (S.li >= 0) {
+#pragma unroll 4
+            for (int q = sub; q <= p.bc; q += G) {
+                int len;
+                const int b = run_of<DIR>(v, R, p, q, S.li, M, len);
+                const unsigned long long k = (unsigned long long)len << 32 | (unsigned)q;
+                if (k < k1) { k2 = k1; k1 = k; b1 = b; }
+                else if (k < k2) k2 = k;
+            }
+        }
+    }
+    for (int o = G >> 1; o >= 1; o >>= 1) {
+        const unsigned long long o1 = __shfl_xor_sync(FULL, k1, o), o2 = __shfl_xor_sync(FULL, k2, o);
+        const int ob = __shfl_xor_sync(FULL, b1, o);
+        k2 = min(max(k1, o1), min(k2, o2));
+        if (o1 < k1) { k1 = o1; b1 = ob; }
+    }
+    if (runs) {
+        if (S.li < 0) {
+            S.len = 0;
+        } else {
+            set_run<DIR>(v, R, p, M, (int)(unsigned)k1, b1, (int)(k1 >> 32), S);
+            S.next = k2 == NONE ? -1 : (int)(unsigned)k2;
+        }
+    }
+    return S;
+}
+
+template <bool DIR, class V>
+__device__ __forceinline__ Cand pick_warp(const V &v, const PosV &p, const PosInfo *P, const int *M) {
+    return pick_group<DIR>(v, p, P, M, 32, threadIdx.x & 31);
+}
+
+// The bitset row of constraint q's image, when the target keeps one and edge labels do not matter.
+template <bool DIR, class V>
+__device__ __forceinline__ const uint64_t *con_row(const V &v, const PosV &p, int q, const int *M) {
+    if (DIR || q < 0 || (v.flags() & JOB_ELAB)) return nullptr;
+    const Con k = constraint<DIR>(v, p, q, M);
+    if (v.adj() != nullptr) return v.adj() + (size_t)k.x * v.dw();
+    if (v.hub_slot() == nullptr) return nullptr;
+    const int h = __ldg(v.hub_slot() + k.x);
+    return h >= 0 ? v.hub_bits() + (size_t)h * v.dw() : nullptr;
+}
+
+// Rules 2 and 3, the domain bit and the list's own edge label for candidate c, entry e of its list.
+template <bool DIR, class V>
+__device__ __forceinline__ bool cand_local(const V &v, const PosV &p, const Cand &S, int c, int e) {
+    if (S.li >= 0) {                                                          // rules 2 (the run's label), 3
+        if (__ldg(S.ids + 2 * (size_t)(S.base + e) + 1) < p.odeg) return false;
+    } else {
+        const int2 r = __ldg(v.vld() + c);
+        if (r.x != p.lab || r.y < p.odeg) return false;
+    }
+    if (DIR && __ldg(v.indeg() + c) < p.ideg) return false;                  // rule 3 (in)
+    if (v.flags() & JOB_RIDS) {                                               // v_t in D(mu_i)
+        const uint64_t w = v.filt()[(size_t)p.pv * v.dw() + (c >> 6)];
+        if (!((w >> (c & 63)) & 1ull)) return false;
+    }
+    return !(v.flags() & JOB_ELAB) || S.skip < 0 || __ldg(S.elab + S.base + e) == S.lab;
+}
+
+// Is candidate c where constraint q wants it (rule 4)?
+template <bool DIR, class V>
+__device__ __forceinline__ bool con_holds(const V &v, const PosV &p, int q, int li, int c, const int *M) {
+    const Con k = constraint<DIR>(v, p, q, M);
+    const bool chk = (v.flags() & JOB_ELAB) != 0;
+    if (!DIR && !chk) {
+        if (v.adj() != nullptr) return (__ldg(v.adj() + (size_t)k.x * v.dw() + (c >> 6)) >> (c & 63)) & 1ull;
+        if (v.hub_slot() != nullptr) {
+            const int h = __ldg(v.hub_slot() + k.x);
+            if (h >= 0) return (__ldg(v.hub_bits() + (size_t)h * v.dw() + (c >> 6)) >> (c & 63)) & 1ull;
+        }
+    }
+    // binary search in x's run of the position's label, else in its whole row
+    const LabelRuns *R = v.runs();
+    const bool in = DIR && k.in, run = R != nullptr && li >= 0;
+    const int32_t *at = run ? (in ? R->irun : R->run) + (size_t)k.x * R->stride + li
+                            : (in ? v.irowptr() : v.rowptr()) + k.x;
+    const int32_t *col = run ? reinterpret_cast<const int32_t *>(in ? R->icol : R->col) : (in ? v.icol() : v.col());
+    const int step = run ? 1 : 0;   // (a run's ids are every other word)
+    int lo = __ldg(at), hi = __ldg(at + 1);
+    const int end = hi;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(col + ((size_t)mid << step)) < c) lo = mid + 1; else hi = mid;
+    }
+    if (lo >= end || __ldg(col + ((size_t)lo << step)) != c) return false;
+    return !chk || __ldg((run ? (in ? R->ielab : R->elab) : (in ? v.ielab() : v.elab())) + lo) == k.lab;
+}
+
+// Rule 1 against the positions named in `same`.
+__device__ __forceinline__ bool unused(const PosInfo *P, int c, const int *M) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        for (uint64_t m = __ldg(&P->same[h]); m; m &= m - 1)
+            if (M[64 * h + __ffsll((long long)m) - 1] == c) return false;
+    return true;
+}
+
+// All rules for candidate c, entry e of list S, by one lane.
+template <bool DIR, class V>
+__device__ __forceinline__ bool cand_lane(const V &v, const PosV &p, const PosInfo *P, const Cand &S, int c, int e,
+                                          const int *M) {
+    if (!cand_local<DIR>(v, p, S, c, e)) return false;
+    if (p.par >= 0)
+        for (int q = 0; q <= p.bc; ++q)
+            if (q != S.skip && !con_holds<DIR>(v, p, q, S.li, c, M)) return false;
+    return unused(P, c, M);
+}
+
+// Up to this many (candidate, constraint) tests of a chunk are spread over the warp's lanes.
+constexpr int SPREAD_TESTS = 128;
+
+// Warp-collective: the candidates of entries [x0, x0 + 32) below `end` of list S that pass all
+// rules, as a ballot; `c` receives this lane's candidate (-1 beyond the list).  Each lane makes
+// its candidate's local tests; the few that remain are tested against the constraints with the
+// lanes spread over (candidate, constraint) pairs, so that a node costs a handful of dependent
+// loads however many earlier neighbours it has; a chunk with many left tests them lane by lane,
+// leaving at the first that fails.  Cs: 32 ints of shared memory of this warp.
+template <bool DIR, class V>
+__device__ __forceinline__ unsigned cand_chunk(const V &v, const PosV &p, const PosInfo *P, const Cand &S, int x0,
+                                               int end, const int *M, int *Cs, int &c) {
+    const int lane = threadIdx.x & 31;
+    const int e = x0 + lane;
+    bool ok = false;
+    c = -1;
+    if (e < end) {
+        c = cand_id(S, e);
+        ok = cand_local<DIR>(v, p, S, c, e);
+    }
+    const unsigned loc = __ballot_sync(FULL, ok);
+    const int nq = p.par >= 0 ? p.bc : 0;   // constraints left to test (the list satisfies one)
+    if (loc && nq) {
+        const int left = __popc(loc);
+        if (left * nq <= SPREAD_TESTS) {
+            const int r = __popc(loc & ((1u << lane) - 1u));
+            if (ok) Cs[r] = c;
+            __syncwarp();
+            unsigned bad = 0;
+            for (int t = lane; t < left * nq; t += 32) {
+                const int q = t / left, x = t - q * left;
+                if (!con_holds<DIR>(v, p, q + (q >= S.skip ? 1 : 0), S.li, Cs[x], M)) bad |= 1u << x;
+            }
+            bad = __reduce_or_sync(FULL, bad);
+            if (ok) ok = !((bad >> r) & 1u);
+        } else if (ok) {
+            for (int q = 0; ok && q <= p.bc; ++q) ok = q == S.skip || con_holds<DIR>(v, p, q, S.li, c, M);
+        }
+    }
+    if (ok) ok = unused(P, c, M);
+    return __ballot_sync(FULL, ok);
+}
+
+// A frame's range [beg, end) (beg < 0: everything) as entries [lo, hi) of list S: as it stands
+// (clipped) unless S is a run and the range counts in the parent's row -- both ascend, so the
+// row range is an interval of ids.  Returns whether this part counts the node's states.
+template <bool DIR, class V>
+__device__ __forceinline__ bool list_range(const V &v, const PosV &p, const Cand &S, const int *M, int beg, int end,
+                                           bool in_run, int &lo, int &hi) {
+    lo = beg >= 0 ? beg : 0;
+    hi = beg >= 0 ? min(end, S.len) : S.len;   // (S is never longer than the parent's row)
+    if (beg < 0) return true;
+    if (in_run) {
+        if (S.li < 0) {   // the label is absent: no entry
+            lo = hi = 0;
+            return beg == 0;
+        }
+        const int drop = run_drop<DIR>(v, p, S, M);
+        lo = max(beg, drop);
+        return beg <= drop && drop < end;
+    }
+    if (S.li < 0 || (beg == 0 && end >= S.raw)) return beg == 0;
+    int len;
+    const int32_t *row = parent_row<DIR>(v, p, M, len);
+    const int e = min(end, len);
+    if (beg >= e) {
+        lo = hi = 0;
+    } else {
+        lo = lower_bound_ids(S.ids + 2 * (size_t)S.base, S.len, __ldg(row + beg), true);
+        hi = lower_bound_ids(S.ids + 2 * (size_t)S.base, S.len, __ldg(row + e - 1) + 1, true);
+    }
+    return beg == 0;
+}
+
+// The other way: entries [lo, hi) of list S (lo < hi) as a range of the parent's row.
+template <bool DIR, class V>
+__device__ __forceinline__ void row_range(const V &v, const PosV &p, const Cand &S, const int *M, int lo, int hi,
+                                          int &beg, int &end) {
+    beg = lo;
+    end = hi;
+    if (S.li < 0) return;
+    int len;
+    const int32_t *row = parent_row<DIR>(v, p, M, len);
+    // (an entry of another constraint's run need not be in the parent's row: bounds by id)
+    beg = lower_bound_ids(row, len, cand_id(S, lo));
+    end = lower_bound_ids(row, len, cand_id(S, hi - 1) + 1);
+}
+
 // Write one match row (images of pattern vertices 0..k-1) for enumeration.
 __device__ __forceinline__ void emit_match(const JobDesc &J, const int *M, int last_pos, int c) {
     unsigned long long slot = atomicAdd(J.mlen, 1ull);
@@ -200,18 +571,12 @@ __device__ __forceinline__ void emit_match(const JobDesc &J, const int *M, int l
 
 // ================================================================ domains
 
-// D(v) initialisation (Section 4): equal label, in/out-degree at least v's.
-// For RI it is exactly the rule 2-3 filter.  One warp per 32 consecutive 64-bit words.
 // Each pattern vertex's label index among its job's target labels (-1: absent),
-// for the jobs that read the label-degree table; one thread per (job, vertex).
-__global__ void __launch_bounds__(BLOCK) k_label_index(const JobDesc *jobs, const long long *vert_off, int njobs,
-                                                       long long nverts) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= nverts) return;
-    const int j = find_job(vert_off, njobs, g);
-    const JobDesc &J = jobs[j];
-    if (J.plidx == nullptr) return;
-    const int u = (int)(g - vert_off[j]);
+// for the jobs that keep one: one block per job, one thread per vertex.
+__global__ void __launch_bounds__(KMAX) k_label_index(const JobDesc *jobs) {
+    const JobDesc &J = jobs[blockIdx.x];
+    const int u = threadIdx.x;
+    if (J.plidx == nullptr || u >= J.p.k) return;
     const int lab = J.p.lab[u];
     int lo = 0, hi = J.t.nlab;
     while (lo < hi) {
@@ -262,6 +627,8 @@ __global__ void __launch_bounds__(BLOCK) k_domain_init_buckets(const JobDesc *jo
     }
 }
 
+// D(v) initialisation (Section 4): equal label, in/out-degree at least v's.
+// For RI it is exactly the rule 2-3 filter.  One warp per 32 consecutive 64-bit words.
 constexpr int INIT_WORDS_PER_WARP = 32;   // most consecutive filter words one warp of k_domain_init writes
 static_assert(INIT_WORDS_PER_WARP <= 32, "k_domain_init copies a warp's words one per lane");
 
@@ -1350,292 +1717,436 @@ __global__ void __launch_bounds__(BLOCK) k_split_coop(const JobDesc *jobs, long 
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 7), globaltimer());
 }
 
-// Counters of the single-pass split, summed per warp while consecutive frames
-// belong to one job and added to the job's counters on a job change or at the
-// end of the warp's slice (lane 0), so a level of many frames does not queue
-// thousands of atomics on one job's four words.
-struct SplitAcc {
-    int job;
-    unsigned long long st, nd, mt, hs;
-};
-
-// (lane 0 only; the warp's SplitAcc lives in shared memory)
-__device__ __forceinline__ void split_acc_flush(const JobDesc *jobs, SplitAcc &A) {
-    if (A.job >= 0) {
-        unsigned long long *ctr = jobs[A.job].ctr;
-        if (A.st) atomicAdd(ctr + 1, A.st);
-        if (A.nd) atomicAdd(ctr + 2, A.nd);
-        if (A.mt) atomicAdd(ctr + 0, A.mt);
-        if (A.hs) atomicAdd(ctr + 3, A.hs);
-    }
-    A.job = -1;
-    A.st = A.nd = A.mt = A.hs = 0;
-}
-
-// One frame of a single-pass split level: test its candidates once, add its
-// counters to A, and append the children of each chunk at offsets reserved on
-// the level's child counter `lvl_ctr`.  A reservation that ends past
-// `cap_frames` raises `full` and writes nothing (the level is then abandoned,
-// see below).  Returns the frame's candidate range length.
+// Frames a child of `depth` images plus c takes: one, or one per SPLIT_RANGE candidates
+// of its list when that is longer (JOB_LONG_LISTS pairs only).
 template <bool DIR>
-__device__ __forceinline__ int split_frame_once(const JobDesc *jobs, const int32_t *fr, int *M, int32_t *fout,
-                                                int stride, long long cap_frames, unsigned long long *lvl_ctr,
-                                                long long *full, SplitAcc &A) {
-    const int lane = threadIdx.x & 31;
-    const int j = fr[0], depth = fr[1], rbeg = fr[2], rend = fr[3];
-    const JobDesc &J = jobs[j];
-    const bool leaf = depth + 1 == J.k;
-    for (int t = lane; t < depth; t += 32) M[t] = fr[FRAME_HDR + t];
-    __syncwarp();
-    const PosInfo &P = J.pos[depth];
-    const Src src = cand_source(J, P, M);
-    const int c_lo = rbeg >= 0 ? rbeg : 0, c_hi = rbeg >= 0 ? min(rend, src.len) : src.len;
-    unsigned long long psum = 0, nodes = 0, hs = 0;
-    if (leaf) {
-        for (int t = lane; t < depth; t += 32) psum += gterm(J.pos[t].pv, M[t]);
-        psum = warp_sum(psum);
-    }
-    // the children's position: where its candidates come from
-    // a child whose own candidate list is longer than SPLIT_RANGE is written as range
-    // frames, so that no warp of the next level scans a hub's whole row while the
-    // others wait at the level's barrier (JOB_LONG_LISTS: such a list can occur)
-    PosInfo Q;
-    const int32_t *qrow = nullptr;
-    bool ranges = false;
-    if (!leaf && (J.flags & JOB_LONG_LISTS)) {
-        Q = J.pos[depth + 1];
-        if (Q.par >= 0) {
-            qrow = (Q.flags & POS_IN_ROW) ? J.t.irowptr : J.t.rowptr;
-            ranges = J.t.maxdeg == 0 || J.t.maxdeg > SPLIT_RANGE;
-        } else {
-            ranges = ((J.flags & JOB_RIDS) ? Q.ucnt : J.t.n) > SPLIT_RANGE;
-        }
-    }
-    for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
-        const int idx = c0 + lane;
-        bool ok = false;
-        int c = -1;
-        if (idx < c_hi) {
-            c = src.ptr ? __ldg(src.ptr + src.base + idx) : idx;
-            ok = feasible<DIR>(J, P, depth, c, (src.ptr && P.par >= 0) ? src.base + idx : -1, M);
-        }
-        const unsigned bal = __ballot_sync(FULL, ok);
-        const int cnt = __popc(bal);
-        nodes += cnt;
-        if (leaf) {
-            if (ok) {
-                hs += fmix64(psum + gterm(P.pv, c));
-                if (J.mbuf) emit_match(J, M, depth, c);
-            }
-        } else if (cnt > 0) {
-            // frames per child: one, or one per SPLIT_RANGE candidates of a long list
-            int r = ok ? 1 : 0;
-            if (ok && ranges) {
-                int len;
-                if (qrow) {
-                    const int a = Q.par == depth ? c : M[Q.par];
-                    len = __ldg(qrow + a + 1) - __ldg(qrow + a);
-                } else {
-                    len = (J.flags & JOB_RIDS) ? Q.ucnt : J.t.n;
-                }
-                r = len > SPLIT_RANGE ? (len + SPLIT_RANGE - 1) / SPLIT_RANGE : 1;
-            }
-            int incl, total;
-            if (ranges) {
-                incl = r;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                total = __shfl_sync(FULL, incl, 31);
-            } else {
-                incl = __popc(bal & (0xffffffffu >> (31 - lane)));   // survivors up to this lane
-                total = cnt;
-            }
-            unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(lvl_ctr, (unsigned long long)total);
-            at = __shfl_sync(FULL, at, 0);
-            if ((long long)(at + total) <= cap_frames) {
-                for (int q = 0; q < r; ++q) {
-                    int32_t *dst = fout + (long long)(at + incl - r + q) * stride;
-                    dst[0] = j;
-                    dst[1] = depth + 1;
-                    dst[2] = r == 1 ? -1 : q * SPLIT_RANGE;
-                    dst[3] = r == 1 ? -1 : (q + 1 == r ? 0x7fffffff : (q + 1) * SPLIT_RANGE);
-                    for (int t = 0; t < depth; ++t) dst[FRAME_HDR + t] = M[t];
-                    dst[FRAME_HDR + depth] = c;
-                }
-            } else if (lane == 0) {
-                *(volatile long long *)full = 1;
-            }
-        }
-    }
-    hs = warp_sum(hs);
-    if (lane == 0) {
-        if (A.job != j) {
-            split_acc_flush(jobs, A);
-            A.job = j;
-        }
-        if (rbeg <= 0) A.st += (unsigned long long)src.len;
-        A.nd += nodes;
-        if (leaf) {
-            A.mt += nodes;
-            A.hs += hs;
-        }
-    }
-    __syncwarp();
-    return c_hi - c_lo;
-}
-
-// A split frame with at most this many candidates is expanded by one lane.
-constexpr int SPLIT_LANE_MAX = 8;
-static_assert(SPLIT_LANE_MAX <= 32, "a lane keeps its frame's survivors in one 32-bit mask");
-
-// Frames of candidates a child of position depth + 1 takes: one, or one per
-// SPLIT_RANGE candidates when its list is longer (JOB_LONG_LISTS pairs only).
 __device__ __forceinline__ int split_child_frames(const JobDesc &J, int depth, int c, const int *M) {
     if (!(J.flags & JOB_LONG_LISTS)) return 1;
-    const PosInfo &Q = J.pos[depth + 1];
+    const PosInfo *Q = J.pos + depth + 1;
+    const PosV q = load_pos(Q);
     long long len;
-    if (Q.par >= 0) {
+    int range = SPLIT_RANGE;
+    if (q.par >= 0) {
         if (J.t.maxdeg != 0 && J.t.maxdeg <= SPLIT_RANGE) return 1;
-        const int32_t *rp = (Q.flags & POS_IN_ROW) ? J.t.irowptr : J.t.rowptr;
-        const int a = Q.par == depth ? c : M[Q.par];
-        len = __ldg(rp + a + 1) - __ldg(rp + a);
+        const LabelRuns *R = J.t.runs;
+        const JobRef v{&J};
+        const int li = R ? J.plidx[q.pv] : -1;
+        if (R && li < 0) return 1;
+        // the shortest constraint's list, as pick_lane will find it; any short one settles it
+        if (R) range = SPLIT_RUN_RANGE;
+        len = 0x7fffffff;
+        for (int x = 0; x <= (R ? q.bc : 0); ++x) {
+            int pos = q.par, in = DIR ? q.flags & POS_IN_ROW : 0;
+            if (x > 0) {
+                const int4 be = __ldg(reinterpret_cast<const int4 *>(J.back + q.bb + x - 1));
+                pos = be.x;
+                in = DIR ? be.y & 1 : 0;
+            }
+            const int a = pos == depth ? c : M[pos];
+            const int32_t *at = R ? (in ? R->irun : R->run) + (size_t)a * R->stride + li
+                                  : (in ? v.irowptr() : v.rowptr()) + a;
+            len = min(len, (long long)(__ldg(at + 1) - __ldg(at)));
+            if (len <= range) return 1;
+        }
     } else {
-        len = (J.flags & JOB_RIDS) ? Q.ucnt : J.t.n;
+        len = (J.flags & JOB_RIDS) ? Q->ucnt : J.t.n;
     }
-    return len > SPLIT_RANGE ? (int)((len + SPLIT_RANGE - 1) / SPLIT_RANGE) : 1;
+    return (int)((len + range - 1) / range);
 }
 
-// The next 32 frames of a warp's slice [f0, hi) of a single-pass split level,
-// one per lane where a frame has at most 32 candidates: the lane tests them in
-// turn (a warp on such a frame would leave most lanes idle), reading the
-// frame's images straight from the frontier.  Children are appended at offsets
-// from one fetch-and-add per warp; counters are summed over runs of lanes with
-// the same job and added with one atomic per run.  Returns the lanes whose
-// frames have longer ranges (the caller expands them a warp at a time) and
-// raises `longest` to the longest range seen.
+// Header words of range q of r of a child frame.
+__device__ __forceinline__ void split_child_header(int32_t *dst, const JobDesc &J, int j, int depth, int r, int q) {
+    const bool run = r > 1 && J.t.runs != nullptr && J.pos[depth].par >= 0;   // (its range counts in a run)
+    dst[0] = j;
+    dst[1] = depth | (run ? FRAME_RUN : 0);
+    const int range = run ? SPLIT_RUN_RANGE : SPLIT_RANGE;
+    dst[2] = r == 1 ? -1 : q * range;
+    dst[3] = r == 1 ? -1 : (q + 1 == r ? 0x7fffffff : (q + 1) * range);
+}
+
+// The single-pass split expands up to 32 frames of a level per warp at once.  The frames'
+// candidate lists laid end to end are tested by the whole warp, SPLIT_STEPS x 32 candidates at
+// a time whichever frames they belong to, so that lanes are busy whatever the mix of list lengths
+// and several loads per lane are in flight; the candidates that pass their local tests queue up
+// for the constraint tests, one per lane (spread over (candidate, constraint) pairs where few are
+// left, as on narrow levels).  The shared block is kept small: what it takes is L1 that the frames
+// and records are read through (5.9 KB per warp made the widest levels 1.6x slower than 3.4 KB).
+constexpr int SPLIT_STEPS = 2;
+constexpr int SPLIT_QUEUE = 32 * SPLIT_STEPS + 32;
+// A child with at least this many images is written by the whole warp, consecutive words at a time.
+constexpr int SPLIT_COOP_DEPTH = 8;
+// Of a longer list, each candidate's local tests include the constraints whose images have a
+// bitset row, the next shortest run's first: their row pointers are looked up once per frame
+// (at most SPLIT_ROWS for the batch), so a test is one load instead of a chain of four
+// (a power-law network's hubs form a near-clique: long lists there pass most constraints).
+constexpr int SPLIT_ROW_MIN = 4;
+constexpr int SPLIT_ROWS = 64;
+
+struct SplitWarp {   // one warp's shared memory: the batch's frames, then its waiting candidates
+    uint64_t ids[32];          // address of the first candidate's id (a run: {id, degree}); below 2^32: that vertex
+    const int32_t *elab[32];   // first candidate's label in the list, null when not compared
+    const int2 *vld[32];       // null: the list is a run (its label is right, its degrees beside the ids)
+    const uint64_t *filt[32];  // D(mu_i), or null
+    const uint64_t *row[SPLIT_ROWS];   // the frames' constraint rows (null: that image has none)
+    int start[33];             // first of the frame's candidates among the batch's
+    int job[32], lab[32], odeg[32], slab[32], li[32], nd[32];
+    int qc[SPLIT_QUEUE];
+    unsigned char ql[SPLIT_QUEUE];
+    unsigned char alive[32];   // split_accept: waiting candidates still in the running
+    unsigned char rbeg[33];    // first of the frame's rows in `row`
+    unsigned char skip[32], next[32], nq[32];   // nq: constraints split_accept has to test
+};
+
+// Tests the n <= 32 waiting candidates from `at` on against their frames' constraints and rule 1,
+// counts and hashes the accepted ones (hs: of frame `lane`), and appends their child frames at
+// offsets reserved on the level's child counter `lvl_ctr`.  A reservation that ends past
+// `cap_frames` raises `full` and writes nothing (the level is then abandoned, see k_split_once).
 template <bool DIR>
-__device__ unsigned split_lane_frames(const JobDesc *jobs, const int32_t *fin, long long f0, long long hi, int depth,
-                                      int32_t *fout, long long cap_frames, unsigned long long *lvl_ctr,
-                                      long long *full, int &longest) {
+__device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t *fin, long long f0, int depth,
+                                             int32_t *fout, long long cap_frames, unsigned long long *lvl_ctr,
+                                             long long *full, SplitWarp &W, int at, int n, unsigned long long &hs) {
     const int lane = threadIdx.x & 31;
     const int sin = FRAME_HDR + depth, sout = sin + 1;
-    const long long f = f0 + lane;
-    const bool have = f < hi;
-    const int32_t *fr = fin + (have ? f : f0) * sin;
-    const int *Mg = fr + FRAME_HDR;
-    int j = 0, rbeg = -1, c_lo = 0, c_hi = 0;
-    Src src;
-    src.ptr = nullptr; src.base = 0; src.len = 0;
-    if (have) {
-        j = fr[0];
-        rbeg = fr[2];
-        const int rend = fr[3];
-        src = cand_source(jobs[j], jobs[j].pos[depth], Mg);
-        c_lo = rbeg >= 0 ? rbeg : 0;
-        c_hi = rbeg >= 0 ? min(rend, src.len) : src.len;
-        longest = max(longest, c_hi - c_lo);
-    }
-    const bool mine = have && c_hi - c_lo <= SPLIT_LANE_MAX;
-    const unsigned longm = __ballot_sync(FULL, have && !mine);
-    if (!__any_sync(FULL, mine)) return longm;
-    const JobDesc &J = jobs[j];
-    const PosInfo &P = J.pos[depth];   // (read where used: a copy would hold 16 registers)
-    const bool leaf = depth + 1 == J.k;
-    unsigned mask = 0;   // the lane's survivors, bit i for candidate c_lo + i
-    int nch = 0;         // frames its children take
-    unsigned long long st = 0, nd = 0, mt = 0, hs = 0;
-    if (mine) {
-        for (int i = 0; i < c_hi - c_lo; ++i) {
-            const int idx = c_lo + i;
-            const int c = src.ptr ? __ldg(src.ptr + src.base + idx) : idx;
-            if (feasible<DIR>(J, P, depth, c, (src.ptr && P.par >= 0) ? src.base + idx : -1, Mg)) mask |= 1u << i;
-        }
-        nd = __popc(mask);
-        if (rbeg <= 0) st = (unsigned long long)src.len;
-        if (leaf) {
-            mt = nd;
-            if (mask) {
-                unsigned long long psum = 0;
-                for (int t = 0; t < depth; ++t) psum += gterm(J.pos[t].pv, Mg[t]);
-                for (unsigned m = mask; m; m &= m - 1) {
-                    const int idx = c_lo + __ffs(m) - 1;
-                    const int c = src.ptr ? __ldg(src.ptr + src.base + idx) : idx;
-                    hs += fmix64(psum + gterm(P.pv, c));
-                    if (J.mbuf) emit_match(J, Mg, depth, c);
-                }
-            }
+    bool ok = lane < n;
+    const int L = W.ql[at + (ok ? lane : 0)], c = W.qc[at + (ok ? lane : 0)];
+    const JobDesc &J = jobs[W.job[L]];
+    const PosInfo *P = J.pos + depth;
+    const int *Mg = fin + (f0 + L) * sin + FRAME_HDR;
+    const int nq = ok ? W.nq[L] : 0;
+    const int mq = (int)__reduce_max_sync(FULL, (unsigned)nq);
+    if (mq > 0) {
+        int left = n, q0 = 0;   // candidates with constraints to test, and those from which on
+        if (n * mq > SPREAD_TESTS) {
+            // many: each lane tries two constraints of its own candidate first, which most fail
+            const JobRef v{&J};
+            const PosV p = load_pos(P);
+            for (int q = 0; ok && q < 2 && q < nq; ++q)
+                ok = con_holds<DIR>(v, p, q + (q >= W.skip[L] ? 1 : 0), W.li[L], c, Mg);
+            const unsigned m = __ballot_sync(FULL, ok && nq > 2);
+            if ((m >> lane) & 1u) W.alive[__popc(m & ((1u << lane) - 1u))] = (unsigned char)lane;
+            left = __popc(m);
+            q0 = 2;
         } else {
-            for (unsigned m = mask; m; m &= m - 1) {
-                const int idx = c_lo + __ffs(m) - 1;
-                const int c = src.ptr ? __ldg(src.ptr + src.base + idx) : idx;
-                nch += split_child_frames(J, depth, c, Mg);
+            W.alive[lane] = (unsigned char)lane;
+        }
+        __syncwarp();
+        if (left > 0) {   // the (candidate, constraint) tests that remain, spread over the lanes
+            const int tests = left * (mq - q0);
+            unsigned bad = 0;
+            for (int t = lane; t < tests; t += 32) {
+                const int q = q0 + t / left, x = W.alive[t % left], Lx = W.ql[at + x];
+                const JobDesc &Jx = jobs[W.job[Lx]];
+                if (q < W.nq[Lx] &&
+                    !con_holds<DIR>(JobRef{&Jx}, load_pos(Jx.pos + depth), q + (q >= W.skip[Lx] ? 1 : 0), W.li[Lx],
+                                    W.qc[at + x], fin + (f0 + Lx) * sin + FRAME_HDR))
+                    bad |= 1u << x;
             }
+            bad = __reduce_or_sync(FULL, bad);
+            ok = ok && !((bad >> lane) & 1u);
         }
     }
-    // children: one reservation for the warp
-    int incl = nch;
+    ok = ok && unused(P, c, Mg);
+    if (!__any_sync(FULL, ok)) return;
+    if (ok) atomicAdd(&W.nd[L], 1);
+    const bool leaf = depth + 1 == J.k;
+    for (unsigned m = __ballot_sync(FULL, ok && leaf); m;) {   // matches, one frame's at a time
+        const int L0 = __shfl_sync(FULL, L, __ffs(m) - 1);
+        const int32_t *M0 = fin + (f0 + L0) * sin + FRAME_HDR;
+        const PosInfo *P0 = jobs[W.job[L0]].pos;
+        unsigned long long psum = 0;
+        for (int t = lane; t < depth; t += 32) psum += gterm(P0[t].pv, M0[t]);
+        psum = warp_sum(psum);
+        const bool here = ok && leaf && L == L0;
+        unsigned long long h = 0;
+        if (here) {
+            h = fmix64(psum + gterm(P->pv, c));
+            if (J.mbuf) emit_match(J, Mg, depth, c);
+        }
+        h = warp_sum(h);
+        if (lane == L0) hs += h;
+        m &= ~__ballot_sync(FULL, here);
+    }
+    // frames per child: one, or one per part of a long list, so that no warp of the next level
+    // scans a hub's whole row while the others wait at the barrier
+    const int r = ok && !leaf ? split_child_frames<DIR>(J, depth, c, Mg) : 0;
+    int incl = r;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(FULL, incl, o);
         if (lane >= o) incl += y;
     }
     const int total = __shfl_sync(FULL, incl, 31);
-    if (total > 0) {
-        unsigned long long at = 0;
-        if (lane == 0) at = atomicAdd(lvl_ctr, (unsigned long long)total);
-        at = __shfl_sync(FULL, at, 0);
-        if ((long long)(at + total) <= cap_frames) {
-            long long o = (long long)at + incl - nch;
-            for (unsigned m = nch ? mask : 0u; m; m &= m - 1) {
-                const int idx = c_lo + __ffs(m) - 1;
-                const int c = src.ptr ? __ldg(src.ptr + src.base + idx) : idx;
-                const int r = split_child_frames(J, depth, c, Mg);
-                for (int q = 0; q < r; ++q, ++o) {
-                    int32_t *dst = fout + o * sout;
-                    dst[0] = j;
-                    dst[1] = depth + 1;
-                    dst[2] = r == 1 ? -1 : q * SPLIT_RANGE;
-                    dst[3] = r == 1 ? -1 : (q + 1 == r ? 0x7fffffff : (q + 1) * SPLIT_RANGE);
-                    for (int t = 0; t < depth; ++t) dst[FRAME_HDR + t] = Mg[t];
-                    dst[FRAME_HDR + depth] = c;
-                }
+    if (total == 0) return;
+    unsigned long long to = 0;
+    if (lane == 0) to = atomicAdd(lvl_ctr, (unsigned long long)total);
+    to = __shfl_sync(FULL, to, 0);
+    if ((long long)(to + total) > cap_frames) {
+        if (lane == 0) *(volatile long long *)full = 1;
+        return;
+    }
+    const bool coop = depth >= SPLIT_COOP_DEPTH;
+    for (int q = 0; q < r; ++q) {
+        int32_t *dst = fout + (long long)(to + incl - r + q) * sout;
+        split_child_header(dst, J, W.job[L], depth + 1, r, q);
+        for (int t = 0; t < depth && !coop; ++t) dst[FRAME_HDR + t] = Mg[t];
+        dst[FRAME_HDR + depth] = c;
+    }
+    if (coop)
+        for (unsigned m = __ballot_sync(FULL, r > 0); m; m &= m - 1) {
+            const int x = __ffs(m) - 1;
+            const int rx = __shfl_sync(FULL, r, x), Lx = __shfl_sync(FULL, L, x);
+            const int32_t *from = fin + (f0 + Lx) * sin + FRAME_HDR;
+            int32_t *dst = fout + ((long long)to + __shfl_sync(FULL, incl, x) - rx) * sout + FRAME_HDR;
+            for (int t = lane; t < depth; t += 32) {
+                const int y = from[t];
+                for (int q = 0; q < rx; ++q) dst[(long long)q * sout + t] = y;
             }
-        } else if (lane == 0) {
-            *(volatile long long *)full = 1;
+        }
+}
+
+// Frames [f0, f0 + nf) of a split level (nf <= 32), by one warp.  Returns the longest list.
+template <bool DIR>
+__device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *fin, long long f0, int nf, int depth,
+                                           int32_t *fout, long long cap_frames, unsigned long long *lvl_ctr,
+                                           long long *full, SplitWarp &W) {
+    const int lane = threadIdx.x & 31;
+    const int sin = FRAME_HDR + depth;
+    // the frames' lists: few frames share the warp's lanes out among them
+    int G = 32;
+    while (G > 1 && 32 / G < nf) G >>= 1;
+    int j = -1, len = 0, rows = 0;
+    unsigned long long st = 0;
+    {
+        const int sub = lane & (G - 1), x = lane / G;
+        const bool have = x < nf;
+        const int32_t *fr = fin + (f0 + (have ? x : 0)) * sin;
+        const int jx = fr[0];
+        const JobDesc &J = jobs[jx];
+        const JobRef v{&J};
+        const PosInfo *P = J.pos + depth;
+        const PosV p = load_pos(P);
+        const int *Mg = fr + FRAME_HDR;
+        const Cand S = pick_group<DIR>(v, p, P, Mg, G, sub);
+        int n = 0, nr = 0, raw = 0;
+        if (have && sub == 0) {
+            int lo, hi;
+            raw = list_range<DIR>(v, p, S, Mg, fr[2], fr[3], (fr[1] & FRAME_RUN) != 0, lo, hi) ? S.raw : 0;
+            n = max(hi - lo, 0);
+            // (rows are of use: the list is long and the target keeps bitset rows)
+            if (!DIR && n > SPLIT_ROW_MIN && S.next >= 0 && !(J.flags & JOB_ELAB) &&
+                (J.t.adj != nullptr || J.t.hub_slot != nullptr))
+                nr = p.bc;
+            const bool run = S.li >= 0;
+            W.ids[x] = run       ? reinterpret_cast<uint64_t>(reinterpret_cast<const int2 *>(S.ids) + S.base + lo)
+                       : S.ids   ? reinterpret_cast<uint64_t>(S.ids + S.base + lo)
+                                 : (uint64_t)(S.base + lo);
+            W.elab[x] = (J.flags & JOB_ELAB) && S.skip >= 0 ? S.elab + S.base + lo : nullptr;
+            W.vld[x] = run ? nullptr : J.t.vld;
+            W.filt[x] = (J.flags & JOB_RIDS) ? J.filt + (size_t)p.pv * J.t.dw : nullptr;
+            W.lab[x] = p.lab;
+            W.odeg[x] = p.odeg;
+            W.slab[x] = S.lab;
+            W.li[x] = S.li;
+            W.skip[x] = (unsigned char)S.skip;   // (unparented: no constraint is tested)
+            W.next[x] = (unsigned char)S.next;
+            W.nq[x] = (unsigned char)(p.par >= 0 ? p.bc : 0);
+            W.job[x] = jx;
+            W.nd[x] = 0;
+        }
+        // frame x's numbers to lane x
+        const int from = min(lane * G, 31);
+        n = __shfl_sync(FULL, n, from);
+        nr = __shfl_sync(FULL, nr, from);
+        raw = __shfl_sync(FULL, raw, from);
+        const int jl = __shfl_sync(FULL, jx, from);
+        if (lane < nf) {
+            j = jl;
+            len = n;
+            rows = nr;
+            st = (unsigned long long)raw;
         }
     }
-    // counters: segmented sums over runs of consecutive lanes with the same job
-    const int key = mine ? j : -1;
-    const int prev = __shfl_up_sync(FULL, key, 1);
-    const unsigned heads = __ballot_sync(FULL, lane == 0 || key != prev);
-    const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    int incl = len;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long a = __shfl_up_sync(FULL, st, o), b = __shfl_up_sync(FULL, nd, o),
-                                 c = __shfl_up_sync(FULL, mt, o), d = __shfl_up_sync(FULL, hs, o);
-        if (lane - o >= head) {
-            st += a;
-            nd += b;
-            mt += c;
-            hs += d;
+        const int y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    W.start[lane + 1] = incl;
+    if (lane == 0) W.start[0] = 0;
+    const int total = __shfl_sync(FULL, incl, 31);
+    const bool any_rows = !DIR && __any_sync(FULL, rows > 0);
+    __syncwarp();
+    if (any_rows) {
+        const int want = rows;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, rows, o);
+            if (lane >= o) rows += y;
+        }
+        const int from = min(rows - want, SPLIT_ROWS), to = min(rows, SPLIT_ROWS);
+        W.rbeg[lane + 1] = (unsigned char)to;
+        if (lane == 0) W.rbeg[0] = 0;
+        const int bc = lane < nf ? W.nq[lane] : 0;
+        __syncwarp();
+        if (want > 0 && to - from == want) W.nq[lane] = 0;   // (unless a row is missing, below)
+        __syncwarp();
+        const int nrow = __shfl_sync(FULL, to, 31);
+        for (int e0 = 0; e0 < nrow; e0 += 32) {
+            const int e = e0 + lane;
+            int x = 0;
+#pragma unroll
+            for (int h = 16; h >= 1; h >>= 1)
+                if (W.rbeg[x + h] <= e) x += h;
+            const int bx = __shfl_sync(FULL, bc, x);
+            if (e < nrow) {
+                const JobDesc &J = jobs[W.job[x]];
+                // the frame's constraints but the list's own, with `next` first
+                const int skip = W.skip[x], first = W.next[x] - (W.next[x] > skip ? 1 : 0), i = e - W.rbeg[x];
+                const int y = i == 0 ? first : i == first ? 0 : i;
+                const uint64_t *row = con_row<DIR>(JobRef{&J}, load_pos(J.pos + depth), y + (y >= skip ? 1 : 0),
+                                                   fin + (f0 + x) * sin + FRAME_HDR);
+                W.row[e] = row;
+                if (row == nullptr) W.nq[x] = (unsigned char)bx;
+            }
+        }
+        __syncwarp();
+    }
+    int n = 0;   // waiting candidates
+    unsigned long long hs = 0;
+    for (int t0 = 0; t0 < total; t0 += 32 * SPLIT_STEPS) {
+        int L[SPLIT_STEPS], c[SPLIT_STEPS];
+        bool ok[SPLIT_STEPS];
+        int e[SPLIT_STEPS], dg[SPLIT_STEPS];
+#pragma unroll
+        for (int u = 0; u < SPLIT_STEPS; ++u) {
+            const int t = t0 + 32 * u + lane;
+            c[u] = -1;
+            dg[u] = 0;
+            L[u] = e[u] = 0;
+            if (t < total) {
+                int x = 0;   // the last frame with start[x] <= t
+#pragma unroll
+                for (int h = 16; h >= 1; h >>= 1)
+                    if (W.start[x + h] <= t) x += h;
+                L[u] = x;
+                e[u] = t - W.start[x];
+                const uint64_t ids = W.ids[x];
+                if (W.vld[x] == nullptr) {
+                    const int2 y = __ldg(reinterpret_cast<const int2 *>(ids) + e[u]);
+                    c[u] = y.x;
+                    dg[u] = y.y;
+                } else {
+                    c[u] = ids >> 32 ? __ldg(reinterpret_cast<const int32_t *>(ids) + e[u]) : (int)ids + e[u];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < SPLIT_STEPS; ++u) {
+            ok[u] = c[u] >= 0;
+            if (ok[u]) {
+                const int x = L[u];
+                const int2 *vld = W.vld[x];
+                int lab = W.lab[x];
+                if (vld != nullptr) {
+                    const int2 r = __ldg(vld + c[u]);
+                    dg[u] = r.y;
+                    ok[u] = r.x == lab;                                            // rule 2
+                }
+                ok[u] = ok[u] && dg[u] >= W.odeg[x];                               // rule 3
+                if (DIR && ok[u]) {
+                    const JobDesc &J = jobs[W.job[x]];
+                    ok[u] = __ldg(J.t.indeg + c[u]) >= __ldg(&J.pos[depth].ideg);
+                }
+                if (ok[u] && W.filt[x]) ok[u] = (W.filt[x][c[u] >> 6] >> (c[u] & 63)) & 1ull;
+                if (ok[u] && W.elab[x]) ok[u] = __ldg(W.elab[x] + e[u]) == W.slab[x];
+            }
+        }
+        if (any_rows) {   // two rows of each candidate at a time
+            int r0[SPLIT_STEPS], r1[SPLIT_STEPS];
+#pragma unroll
+            for (int u = 0; u < SPLIT_STEPS; ++u) {
+                r0[u] = W.rbeg[L[u]];
+                r1[u] = ok[u] ? W.rbeg[L[u] + 1] : 0;
+            }
+            for (bool more = true; more;) {
+                uint64_t wa[SPLIT_STEPS], wb[SPLIT_STEPS];
+#pragma unroll
+                for (int u = 0; u < SPLIT_STEPS; ++u) {
+                    const uint64_t *ra = r0[u] < r1[u] ? W.row[r0[u]] : nullptr;
+                    const uint64_t *rb = r0[u] + 1 < r1[u] ? W.row[r0[u] + 1] : nullptr;
+                    wa[u] = ra ? __ldg(ra + (c[u] >> 6)) : ~0ull;
+                    wb[u] = rb ? __ldg(rb + (c[u] >> 6)) : ~0ull;
+                }
+                more = false;
+#pragma unroll
+                for (int u = 0; u < SPLIT_STEPS; ++u) {
+                    if (!(((wa[u] & wb[u]) >> (c[u] & 63)) & 1ull)) {
+                        ok[u] = false;
+                        r1[u] = 0;
+                    }
+                    r0[u] += 2;
+                    more = more || r0[u] < r1[u];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < SPLIT_STEPS; ++u) {
+            const unsigned bal = __ballot_sync(FULL, ok[u]);
+            if (ok[u]) {
+                const int y = n + __popc(bal & ((1u << lane) - 1u));
+                W.qc[y] = c[u];
+                W.ql[y] = (unsigned char)L[u];
+            }
+            n += __popc(bal);
+        }
+        __syncwarp();
+        while (n >= 32) {   // full warps of them, from the end
+            n -= 32;
+            split_accept<DIR>(jobs, fin, f0, depth, fout, cap_frames, lvl_ctr, full, W, n, 32, hs);
+            __syncwarp();
+        }
+    }
+    if (n > 0) split_accept<DIR>(jobs, fin, f0, depth, fout, cap_frames, lvl_ctr, full, W, 0, n, hs);
+    __syncwarp();
+    // counters: segmented sums over runs of consecutive lanes with the same job, one atomic per run
+    const bool leaf = j >= 0 && depth + 1 == jobs[j].k;
+    unsigned long long nd = j >= 0 ? (unsigned long long)W.nd[lane] : 0, mt = leaf ? nd : 0;
+    const int prev = __shfl_up_sync(FULL, j, 1);
+    const unsigned heads = __ballot_sync(FULL, lane == 0 || j != prev);
+    const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    if (nf > 1) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long a = __shfl_up_sync(FULL, st, o), b = __shfl_up_sync(FULL, nd, o),
+                                     c = __shfl_up_sync(FULL, mt, o), d = __shfl_up_sync(FULL, hs, o);
+            if (lane - o >= head) {
+                st += a;
+                nd += b;
+                mt += c;
+                hs += d;
+            }
         }
     }
     const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
-    if (tail && key >= 0) {
-        unsigned long long *ctr = J.ctr;
+    if (tail && j >= 0) {
+        unsigned long long *ctr = jobs[j].ctr;
         if (st) atomicAdd(ctr + 1, st);
         if (nd) atomicAdd(ctr + 2, nd);
         if (mt) atomicAdd(ctr + 0, mt);
         if (hs) atomicAdd(ctr + 3, hs);
     }
-    return longm;
+    __syncwarp();
+    return warp_max(len);
 }
 
 // Single-pass split (unsharded runs; the caller's shard counts the levels).
+// Bound by the gathers of the wide levels (id and degree streamed, one bitset word per
+// constraint tested) and, on narrow ones, by the dependent loads of one frame and the barrier.
+// Per call, against lists that were the parent's rows, tested by a warp or a lane per frame:
+// 160 queries on the 100k-vertex network 9.0 -> 5.7 ms, 24 directed edge-labelled patterns
+// 1.45 -> 0.66 ms, 96 served queries on 50k vertices 6.0 -> 4.1 ms end to end; 200,000
+// molecule pairs (no runs: short rows) 5.4 -> 5.2 ms.
 // The children of level L are counted on wtot[L] (zeroed by the host).  A
 // level whose children do not all fit is abandoned after its barrier: its
 // frames stay the frontier, rewritten so that the search does not count the
@@ -1645,20 +2156,14 @@ __device__ unsigned split_lane_frames(const JobDesc *jobs, const int32_t *fin, l
 // the empty range [1, 1).
 template <bool DIR>
 __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, long long f0, SplitCtl S) {
-    __shared__ int Msh[WARPS_PER_BLOCK][KMAX];
-    __shared__ SplitAcc Ash[WARPS_PER_BLOCK];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int *M = Msh[wib];
-    SplitAcc &A = Ash[wib];
+    __shared__ SplitWarp Wsh[WARPS_PER_BLOCK];
+    const int lane = threadIdx.x & 31;
+    SplitWarp &W = Wsh[threadIdx.x >> 5];
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     unsigned long long *lvl_ctr = reinterpret_cast<unsigned long long *>(S.wtot);
     long long F = f0;
     int cur = 0, level = 0;
-    if (lane == 0) {
-        A.job = -1;
-        A.st = A.nd = A.mt = A.hs = 0;
-    }
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 6), ~globaltimer());
     for (; level < S.max_levels; ++level) {
         if (F == 0 || F >= S.target) break;
@@ -1667,19 +2172,9 @@ __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, lo
         const int sin = FRAME_HDR + level, sout = FRAME_HDR + level + 1;
         const long long lo = F * w / nw, hi = F * (w + 1) / nw;
         int longest = 0;
-        for (long long f0 = lo; f0 < hi; f0 += 32) {
-            // frames of at most 32 candidates one per lane, longer ones a warp at a time
-            unsigned longm = split_lane_frames<DIR>(jobs, fin, f0, hi, level, fout, S.cap_ints / sout,
-                                                    lvl_ctr + level, S.result + 5, longest);
-            while (longm) {
-                const int L = __ffs(longm) - 1;
-                longm &= longm - 1;
-                longest = max(longest, split_frame_once<DIR>(jobs, fin + (f0 + L) * sin, M, fout, sout,
-                                                             S.cap_ints / sout, lvl_ctr + level, S.result + 5, A));
-            }
-        }
-        longest = warp_max(longest);
-        if (lane == 0) split_acc_flush(jobs, A);
+        for (long long f = lo; f < hi; f += 32)
+            longest = max(longest, split_batch<DIR>(jobs, fin, f, (int)min(32ll, hi - f), level, fout,
+                                                    S.cap_ints / sout, lvl_ctr + level, S.result + 5, W));
         if (S.trace && lane == 0 && longest > 0)
             atomicMax(reinterpret_cast<unsigned long long *>(S.trace + KMAX + level), (unsigned long long)longest);
         grid_barrier(S.bar, S.bar + 1, S.status);
@@ -1688,7 +2183,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, lo
             for (long long f = lo; f < hi; ++f) {
                 int32_t *fr = fin + f * sin;
                 if (lane == 0) {
-                    const bool leaf = fr[1] + 1 == jobs[fr[0]].k;
+                    const bool leaf = (fr[1] & FRAME_DEPTH_MASK) + 1 == jobs[fr[0]].k;
                     if (leaf) { fr[2] = 1; fr[3] = 1; }
                     else {
                         fr[1] |= FRAME_COUNTED;
@@ -1873,6 +2368,7 @@ __device__ bool push_frame(const SearchCtl &C, int j, int depth, int beg, int en
 struct Frame {
     int job, depth, beg, end;
     bool counted;   // FRAME_COUNTED: the range's accepted nodes and states are already counted
+    bool in_run;    // FRAME_RUN: the range counts in the node's label run
 };
 
 // Optional per-warp timing, kept in the warp's own trace record (no registers):
@@ -2027,6 +2523,7 @@ __device__ bool acquire_frame(const SearchCtl &C, int *M, Frame &fr, unsigned lo
     }
     const int dw = src[1];
     fr.job = src[0]; fr.depth = dw & FRAME_DEPTH_MASK; fr.counted = (dw & FRAME_COUNTED) != 0;
+    fr.in_run = (dw & FRAME_RUN) != 0;
     fr.beg = src[2]; fr.end = src[3];
     for (int i = lane; i < fr.depth; i += 32) M[i] = src[FRAME_HDR + i];
     __syncwarp();
@@ -2088,12 +2585,13 @@ __device__ __forceinline__ void donation_done(const SearchCtl &C) {
 
 // ===================================================== search: CSR kernel
 //
-// One warp owns one depth-first search.  A level's candidates are the row of
-// M(P(mu_i)) (or V_t / D(mu_i) when mu_i is unparented), scanned 32 at a time,
-// one candidate per lane; each lane tests rules 1-4 and the domain bit, and a
-// ballot compacts the chunk's survivors.  Per warp, shared memory holds M,
-// the level records and a compact copy of the job's position table; the
-// job's pointers stay in registers.
+// One warp owns one depth-first search.  A level's candidates are its shortest
+// label run, on targets without runs the row of M(P(mu_i)) (or V_t / D(mu_i)
+// when mu_i is unparented), scanned 32 at a time, one candidate per lane; each
+// lane makes its candidate's local tests, the constraints are tested spread over
+// the warp (cand_chunk), and a ballot compacts the chunk's survivors.  Per warp,
+// shared memory holds M, the level records and a compact copy of the job's
+// position table; the job's pointers stay in registers.
 
 __host__ __device__ __forceinline__ size_t round16(size_t x) { return (x + 15) & ~(size_t)15; }
 
@@ -2102,83 +2600,92 @@ struct PosC {                // hot fields of one position
     int32_t lab, odeg, ideg, pel, flags;
 };
 
+// What a level's candidates are entries of.
+enum : int16_t { LIST_VERTICES = 0, LIST_DOMAIN, LIST_ROW, LIST_IN_ROW, LIST_RUN, LIST_IN_RUN };
+
 struct LvCsr {
     int base;                // offset of the level's candidate list in its array
     int cur, end;            // unscanned candidates [cur, end)
     unsigned mask;           // survivors of the last scanned chunk, not yet descended
     int cbase;               // index of that chunk's first candidate
-    int len;                 // the node's raw candidate count (its states, counted at index 0)
+    int raw;                 // the node's raw candidate count (its states)
+    int len;                 // length of the list
+    int16_t kind, skip;      // LIST_*, and the constraint the list itself satisfies
 };
 
 __host__ __device__ __forceinline__ size_t csr_smem_per_warp(int kmax) {
-    return round16((size_t)kmax * sizeof(LvCsr) + (size_t)kmax * sizeof(int) + (size_t)kmax * sizeof(PosC));
+    return round16((size_t)kmax * sizeof(LvCsr) + ((size_t)kmax + 32) * sizeof(int) + (size_t)kmax * sizeof(PosC));
 }
 
+// A job's pointers in registers, read like JobRef.
 struct CsrJob {
-    const int32_t *rowptr, *col, *elab, *irowptr, *icol, *ielab, *indeg, *ulist, *hub_slot;
-    const int2 *vld;
-    const uint64_t *filt, *adj, *hub_bits;
-    const BackEdge *back;
+    const int32_t *rowptr_, *col_, *elab_, *irowptr_, *icol_, *ielab_, *indeg_, *ulist_, *hub_slot_, *plidx_;
+    const int2 *vld_;
+    const uint64_t *filt_, *adj_, *hub_bits_;
+    const BackEdge *back_;
     const PosInfo *pos;
-    int n, dw, k, flags;
+    const LabelRuns *runs_;
+    int n_, dw_, k, flags_;
+    __device__ __forceinline__ const int32_t *rowptr() const { return rowptr_; }
+    __device__ __forceinline__ const int32_t *col() const { return col_; }
+    __device__ __forceinline__ const int32_t *elab() const { return elab_; }
+    __device__ __forceinline__ const int32_t *irowptr() const { return irowptr_; }
+    __device__ __forceinline__ const int32_t *icol() const { return icol_; }
+    __device__ __forceinline__ const int32_t *ielab() const { return ielab_; }
+    __device__ __forceinline__ const int32_t *indeg() const { return indeg_; }
+    __device__ __forceinline__ const int32_t *hub_slot() const { return hub_slot_; }
+    __device__ __forceinline__ const uint64_t *hub_bits() const { return hub_bits_; }
+    __device__ __forceinline__ const uint64_t *adj() const { return adj_; }
+    __device__ __forceinline__ const int2 *vld() const { return vld_; }
+    __device__ __forceinline__ const LabelRuns *runs() const { return runs_; }
+    __device__ __forceinline__ const uint64_t *filt() const { return filt_; }
+    __device__ __forceinline__ const BackEdge *back() const { return back_; }
+    __device__ __forceinline__ const int32_t *ulist() const { return ulist_; }
+    __device__ __forceinline__ const int32_t *plidx() const { return plidx_; }
+    __device__ __forceinline__ int n() const { return n_; }
+    __device__ __forceinline__ int dw() const { return dw_; }
+    __device__ __forceinline__ int flags() const { return flags_; }
 };
 
-// Candidate array of a position: the parent's out- or in-row, D(mu_i), or
-// null for "candidate j is vertex j".
-__device__ __forceinline__ const int32_t *csr_src(const CsrJob &B, const PosC &p) {
-    if (p.par >= 0) return (p.flags & POS_IN_ROW) ? B.icol : B.col;
-    return (B.flags & JOB_RIDS) ? B.ulist : nullptr;
+__device__ __forceinline__ PosV csr_pos(const PosC &q) {
+    return PosV{q.pv, q.par, q.lab, q.odeg, q.ideg, q.pel, q.bb, q.bc, q.flags};
 }
 
-// Rules 1-4 (Section "RI") and the RI-DS domain test for candidate c of
-// position i; eidx is c's index in the parent's row (parent-arc label) or -1.
+// A level's list as cand_chunk reads it.
 template <bool DIR>
-__device__ __forceinline__ bool csr_feasible(const CsrJob &B, const PosC &p, int i, int c, int eidx, const int *M) {
-    const int2 v = __ldg(B.vld + c);
-    if (v.x != p.lab || v.y < p.odeg) return false;                           // rules 2, 3
-    if (DIR && __ldg(B.indeg + c) < p.ideg) return false;                    // rule 3 (in)
-    if (B.flags & JOB_RIDS) {                                                 // v_t in D(mu_i)
-        const uint64_t w = B.filt[(size_t)p.pv * B.dw + (c >> 6)];
-        if (!((w >> (c & 63)) & 1ull)) return false;
+__device__ __forceinline__ Cand csr_list(const CsrJob &B, const PosV &p, const LvCsr &L, const int *M) {
+    Cand S;
+    S.base = L.base;
+    S.len = L.len;
+    S.raw = L.raw;
+    S.skip = L.skip;
+    S.next = -1;
+    S.elab = nullptr;
+    S.li = -1;
+    S.lab = p.pel;
+    switch (L.kind) {
+        case LIST_VERTICES: S.ids = nullptr; break;
+        case LIST_DOMAIN: S.ids = B.ulist_; break;
+        case LIST_ROW: S.ids = B.col_; S.elab = B.elab_; break;
+        case LIST_IN_ROW: S.ids = B.icol_; S.elab = B.ielab_; break;
+        default:
+            S.ids = reinterpret_cast<const int32_t *>(DIR && L.kind == LIST_IN_RUN ? B.runs_->icol : B.runs_->col);
+            S.elab = DIR && L.kind == LIST_IN_RUN ? B.runs_->ielab : B.runs_->elab;
+            S.li = B.plidx_[p.pv];
+            if (L.skip > 0 && (B.flags_ & JOB_ELAB)) S.lab = constraint<DIR>(B, p, L.skip, M).lab;
     }
-    const bool chk = (B.flags & JOB_ELAB) != 0;
-    if (chk && eidx >= 0) {                                                   // parent arc label
-        const int l = (p.flags & POS_IN_ROW) ? __ldg(B.ielab + eidx) : __ldg(B.elab + eidx);
-        if (l != p.pel) return false;
-    }
-    for (int b = 0; b < p.bc; ++b) {                                          // rule 4
-        const BackEdge be = B.back[p.bb + b];
-        const int x = M[be.pos];
-        if (!DIR) {
-            if (B.adj != nullptr && !chk) {
-                const uint64_t w = __ldg(B.adj + (size_t)x * B.dw + (c >> 6));
-                if (!((w >> (c & 63)) & 1ull)) return false;
-            } else if (B.hub_slot != nullptr && !chk && __ldg(B.hub_slot + x) >= 0) {
-                const uint64_t w = __ldg(B.hub_bits + (size_t)__ldg(B.hub_slot + x) * B.dw + (c >> 6));
-                if (!((w >> (c & 63)) & 1ull)) return false;
-            } else if (!row_has(B.rowptr, B.col, B.elab, x, c, be.lab_out, chk)) {
-                return false;
-            }
-        } else {
-            if ((be.dir & 1) && !row_has(B.irowptr, B.icol, B.ielab, x, c, be.lab_out, chk)) return false;
-            if ((be.dir & 2) && !row_has(B.rowptr, B.col, B.elab, x, c, be.lab_in, chk)) return false;
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)                                               // rule 1 (same-label positions)
-        for (uint64_t m = B.pos[i].same[h]; m; m &= m - 1)
-            if (M[64 * h + __ffsll((long long)m) - 1] == c) return false;
-    return true;
+    return S;
 }
 
 template <bool DIR>
-__global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, SearchCtl C, int kmax) {
+__global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, SearchCtl C, int kmax) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned char *base = smem + wib * csr_smem_per_warp(kmax);
     LvCsr *lv = reinterpret_cast<LvCsr *>(base);
     int *M = reinterpret_cast<int *>(lv + kmax);
-    PosC *tab = reinterpret_cast<PosC *>(M + kmax);
+    int *Cs = M + kmax;
+    PosC *tab = reinterpret_cast<PosC *>(Cs + 32);
 
     const unsigned long long deadline = C.deadline_ns ? globaltimer() + C.deadline_ns : 0ull;
     Frame fr;
@@ -2193,11 +2700,11 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
         const JobDesc &J = jobs[fr.job];
         if (fr.job != cur_job) {
             cur_job = fr.job;
-            B.rowptr = J.t.rowptr; B.col = J.t.col; B.elab = J.t.elab;
-            B.irowptr = J.t.irowptr; B.icol = J.t.icol; B.ielab = J.t.ielab; B.indeg = J.t.indeg;
-            B.ulist = J.ulist; B.vld = J.t.vld; B.filt = J.filt; B.adj = J.t.adj; B.back = J.back; B.pos = J.pos;
-            B.hub_slot = J.t.hub_slot; B.hub_bits = J.t.hub_bits;
-            B.n = J.t.n; B.dw = J.t.dw; B.k = J.k; B.flags = J.flags;
+            B.rowptr_ = J.t.rowptr; B.col_ = J.t.col; B.elab_ = J.t.elab;
+            B.irowptr_ = J.t.irowptr; B.icol_ = J.t.icol; B.ielab_ = J.t.ielab; B.indeg_ = J.t.indeg;
+            B.ulist_ = J.ulist; B.vld_ = J.t.vld; B.filt_ = J.filt; B.adj_ = J.t.adj; B.back_ = J.back; B.pos = J.pos;
+            B.hub_slot_ = J.t.hub_slot; B.hub_bits_ = J.t.hub_bits; B.runs_ = J.t.runs; B.plidx_ = J.plidx;
+            B.n_ = J.t.n; B.dw_ = J.t.dw; B.k = J.k; B.flags_ = J.flags;
             for (int t = lane; t < B.k; t += 32) {
                 const PosInfo P = J.pos[t];
                 PosC q;
@@ -2214,34 +2721,41 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
         // since the last fold (every 64 iterations): an iteration adds at most 32 nodes and a
         // candidate list below 2^24 states (longer lists go straight to the 64-bit total)
         unsigned st32 = 0, nd32 = 0, mt32 = 0;
-        // set up level `l` (positions 0..l-1 assigned)
-        auto setup = [&](int l, int beg, int endv) {
-            const PosC p = tab[l];
-            int b0, len;
+        bool counts0 = true;   // the frame counted its first node's states
+        // set up level `l` (positions 0..l-1 assigned) and count the node's states: a range
+        // frame counts them if it starts the node, a counted frame not at all
+        auto setup = [&](int l, int beg, int endv, bool in_run) {
+            const PosV p = csr_pos(tab[l]);
+            const Cand S = pick_warp<DIR>(B, p, B.pos + l, M);
+            int cur, end;
+            const bool counts = list_range<DIR>(B, p, S, M, beg, endv, in_run, cur, end);
+            int kind = p.par < 0 ? (S.ids ? LIST_DOMAIN : LIST_VERTICES) : LIST_ROW;
             if (p.par >= 0) {
-                const int a = M[p.par];
-                const int32_t *rp = (p.flags & POS_IN_ROW) ? B.irowptr : B.rowptr;
-                b0 = __ldg(rp + a);
-                len = __ldg(rp + a + 1) - b0;
-            } else if (B.flags & JOB_RIDS) {
-                const PosInfo &P = J.pos[l];
-                b0 = P.uoff;
-                len = P.ucnt;
-            } else {
-                b0 = 0;
-                len = B.n;
+                if (B.runs_ != nullptr)
+                    kind = DIR && S.ids == reinterpret_cast<const int32_t *>(B.runs_->icol) ? LIST_IN_RUN : LIST_RUN;
+                else if (DIR && (p.flags & POS_IN_ROW)) kind = LIST_IN_ROW;
             }
-            int cur = 0, end = len;
-            if (beg >= 0) { cur = beg; end = min(endv, len); }
             __syncwarp();
             if (lane == 0) {
-                lv[l].base = b0; lv[l].cur = cur; lv[l].end = end; lv[l].mask = 0; lv[l].cbase = 0; lv[l].len = len;
+                lv[l].base = S.base; lv[l].cur = cur; lv[l].end = end; lv[l].mask = 0; lv[l].cbase = 0;
+                lv[l].raw = S.raw; lv[l].len = S.len; lv[l].kind = (int16_t)kind; lv[l].skip = (int16_t)S.skip;
             }
             __syncwarp();
+            if (l == d0) counts0 = counts;
+            if (counts && l != quiet) {
+                if (S.raw < (1 << 24)) st32 += (unsigned)S.raw;
+                else st += (unsigned long long)S.raw;
+            }
         };
-        // a node's states are counted when its candidate 0 is scanned, so every split of
-        // its candidate range (range frames, donations, checkpoints) counts them exactly once
-        setup(d0, fr.beg, fr.end);
+        // candidate of entry e of level l's list
+        auto entry = [&](const LvCsr &L, int e) {
+            if (L.kind >= LIST_RUN) return __ldg(&(DIR && L.kind == LIST_IN_RUN ? B.runs_->icol : B.runs_->col)[L.base + e]).x;
+            const int32_t *ids = L.kind == LIST_VERTICES ? nullptr
+                                 : L.kind == LIST_DOMAIN ? B.ulist_
+                                 : L.kind == LIST_ROW    ? B.col_ : B.icol_;
+            return ids ? __ldg(ids + L.base + e) : L.base + e;
+        };
+        setup(d0, fr.beg, fr.end, fr.in_run);
         int lvl = d0;
         bool stopped = false;
         for (;;) {
@@ -2265,10 +2779,19 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
                     last_don_ns = last_check;
                     for (int l = d0; l <= lvl && l + 1 + DONATE_MIN_LEVELS <= k; ++l) {
                         LvCsr &L = lv[l];
-                        const int rem = L.end - L.cur;
+                        int rem = L.end - L.cur;
+                        if (rem >= 64 && L.kind >= LIST_RUN) {   // past the entries no part may start in
+                            const PosV p = csr_pos(tab[l]);
+                            const int drop = run_drop<DIR>(B, p, csr_list<DIR>(B, p, L, M), M);
+                            __syncwarp();
+                            if (lane == 0 && L.cur < drop) L.cur = min(drop, L.end);
+                            __syncwarp();
+                            rem = L.end - L.cur;
+                        }
                         if (rem >= 64) {
                             const int mid = L.cur + ((rem / 2 + 31) & ~31);
-                            if (push_frame(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0), mid, L.end, M, l,
+                            const int run = L.kind >= LIST_RUN ? FRAME_RUN : 0;
+                            if (push_frame(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0) | run, mid, L.end, M, l,
                                            -1)) {
                                 __syncwarp();
                                 if (lane == 0) L.end = mid;
@@ -2277,12 +2800,10 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
                             break;
                         }
                         if (L.mask != 0) {
-                            const int32_t *src = csr_src(B, tab[l]);
                             int given = 0;
                             while (L.mask != 0 && given < C.gran) {
                                 const unsigned m = L.mask;
-                                const int b = __ffs(m) - 1;
-                                const int c = src ? __ldg(src + L.base + L.cbase + b) : L.cbase + b;
+                                const int c = entry(L, L.cbase + __ffs(m) - 1);
                                 if (!push_frame(C, fr.job, l + 1, -1, -1, M, l, c)) break;
                                 __syncwarp();
                                 if (lane == 0) L.mask = m & (m - 1);
@@ -2297,8 +2818,6 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
             }
             LvCsr &L = lv[lvl];
             const unsigned mask = L.mask;
-            const PosC p = tab[lvl];
-            const int32_t *src = csr_src(B, p);
             if (mask == 0) {
                 const int cur = L.cur, end = L.end;
                 if (cur >= end) {
@@ -2306,19 +2825,10 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
                     --lvl;
                     continue;
                 }
-                const int cnt = min(32, end - cur);
-                if (cur == 0 && lvl != quiet) {
-                    if (L.len < (1 << 24)) st32 += (unsigned)L.len;
-                    else st += (unsigned long long)L.len;
-                }
-                bool ok = false;
-                int c = -1;
-                if (lane < cnt) {
-                    const int e = L.base + cur + lane;
-                    c = src ? __ldg(src + e) : cur + lane;
-                    ok = csr_feasible<DIR>(B, p, lvl, c, (src && p.par >= 0) ? e : -1, M);
-                }
-                unsigned bal = __ballot_sync(FULL, ok);
+                const PosV p = csr_pos(tab[lvl]);
+                const Cand S = csr_list<DIR>(B, p, L, M);
+                int c;
+                unsigned bal = cand_chunk<DIR>(B, p, B.pos + lvl, S, cur, end, M, Cs, c);
                 if (lvl != quiet) nd32 += __popc(bal);
                 if (lvl == k - 1) {
                     mt32 += __popc(bal);
@@ -2327,7 +2837,7 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
                         unsigned long long ps = 0;
                         for (int t = lane; t < lvl; t += 32) ps += gterm(tab[t].pv, M[t]);
                         ps = warp_sum(ps);
-                        if (ok) {
+                        if ((bal >> lane) & 1u) {
                             hs += fmix64(ps + gterm(p.pv, c));
                             if (J.mbuf) emit_match(J, M, lvl, c);
                         }
@@ -2335,13 +2845,12 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
                     bal = 0;
                 }
                 __syncwarp();
-                if (lane == 0) { L.cur = cur + cnt; L.mask = bal; L.cbase = cur; }
+                if (lane == 0) { L.cur = min(cur + 32, end); L.mask = bal; L.cbase = cur; }
                 __syncwarp();
                 continue;
             }
             // descend into the lowest pending survivor
-            const int b = __ffs(mask) - 1;
-            const int c = src ? __ldg(src + L.base + L.cbase + b) : L.cbase + b;
+            const int c = entry(L, L.cbase + __ffs(mask) - 1);
             __syncwarp();
             if (lane == 0) {
                 L.mask = mask & (mask - 1);
@@ -2349,20 +2858,38 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
             }
             __syncwarp();
             ++lvl;
-            setup(lvl, -1, 0);
+            setup(lvl, -1, 0, false);
         }
         if (stopped && C.ckpt != nullptr) {
             // checkpoint, per level: the part of the current chunk from its lowest pending
             // survivor on (already counted; survivors are taken lowest first), then the
-            // unscanned rest of the range (counted only if the frame itself was)
+            // unscanned rest of the range (counted only if the frame itself was); both as ranges
+            // of the parent's row.  A part left from entry 0 on counts the node's states again
+            // when it is resumed: they are taken back here.
             for (int l = d0; l <= lvl; ++l) {
                 const LvCsr L = lv[l];
+                const PosV p = csr_pos(tab[l]);
+                const Cand S = csr_list<DIR>(B, p, L, M);
                 const int cb = L.mask ? L.cbase + __ffs(L.mask) - 1 : L.cur;
+                int beg, end;
                 if (l == quiet) {
-                    if (cb < L.end) ckpt_push(C, fr.job, l, true, cb, L.end, M);
+                    if (cb < L.end) {
+                        row_range<DIR>(B, p, S, M, cb, L.end, beg, end);
+                        ckpt_push(C, fr.job, l, true, beg, end, M);
+                    }
                 } else {
-                    if (cb < L.cur) ckpt_push(C, fr.job, l, true, cb, L.cur, M);
-                    if (L.cur < L.end) ckpt_push(C, fr.job, l, false, L.cur, L.end, M);
+                    if (cb < L.cur) {
+                        row_range<DIR>(B, p, S, M, cb, L.cur, beg, end);
+                        ckpt_push(C, fr.job, l, true, beg, end, M);
+                    }
+                    const int cur = L.cur < L.end && S.li >= 0 ? max(L.cur, run_drop<DIR>(B, p, S, M)) : L.cur;
+                    if (cur < L.end) {
+                        row_range<DIR>(B, p, S, M, cur, L.end, beg, end);
+                        const bool counted = l > d0 || counts0;
+                        if (counted && L.cur == 0) beg = 0;   // scan not begun: the whole node
+                        if (counted && beg == 0) st -= (unsigned long long)L.raw;
+                        ckpt_push(C, fr.job, l, false, beg, end, M);
+                    }
                 }
             }
         }
@@ -2381,6 +2908,40 @@ __global__ void __launch_bounds__(BLOCK) k_search_csr(const JobDesc *jobs, Searc
     }
     WarpClock::finish(C);
     if ((threadIdx.x & 31) == 0) atomicMax(C.span + 1, globaltimer());
+}
+
+// One warp per checkpoint frame: a label-run range becomes the same part of the parent's row.
+template <bool DIR>
+__global__ void __launch_bounds__(BLOCK) k_frames_to_rows(const JobDesc *jobs, int32_t *frames, long long n,
+                                                          long long pitch, const unsigned long long *seq) {
+    const long long f = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (f >= n) return;
+    if (seq != nullptr) {   // a queue cell that is not published holds no frame
+        const unsigned long long sv = seq[f];
+        if (sv == 0 || (sv & CELL_LOCK) || (sv - 1) % (unsigned long long)n != (unsigned long long)f) return;
+    }
+    int32_t *fr = frames + f * pitch;
+    const int dw = fr[1];
+    if (!(dw & FRAME_RUN)) return;
+    const JobDesc &J = jobs[fr[0]];
+    const JobRef v{&J};
+    const PosInfo *P = J.pos + (dw & FRAME_DEPTH_MASK);
+    const PosV p = load_pos(P);
+    const int *M = fr + FRAME_HDR;
+    const Cand S = pick_warp<DIR>(v, p, P, M);
+    int lo, hi, beg = 1, end = 1;   // (an empty part)
+    const bool counts = list_range<DIR>(v, p, S, M, fr[2], fr[3], true, lo, hi);
+    if (lo < hi) row_range<DIR>(v, p, S, M, lo, hi, beg, end);
+    if (counts) {
+        end = lo < hi ? end : 0;
+        beg = 0;
+    }
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        fr[1] = dw & ~FRAME_RUN;
+        fr[2] = beg;
+        fr[3] = end;
+    }
 }
 
 // ================================================== search: bitset kernel
@@ -2737,29 +3298,23 @@ __global__ void __launch_bounds__(BLOCK, 4) k_search_bits(const JobDesc *jobs, S
         // a range frame covers candidates [beg, end) of its node: as the candidate
         // lists are ascending, that is the vertex-id interval [first, last]
         int vlo = 0, vhi = 0x7fffffff;
+        bool counts = true;   // this part counts the node's states
         if (fr.beg >= 0) {
-            const PosB p = W.tab()[d0];
-            const int32_t *lst = nullptr;
-            int b0 = 0, len = 0;
-            if (p.par >= 0) {
-                const int a = M[p.par];
-                lst = J.t.col;
-                b0 = __ldg(J.t.rowptr + a);
-                len = __ldg(J.t.rowptr + a + 1) - b0;
-            } else if (J.flags & JOB_RIDS) {
-                lst = J.ulist;
-                b0 = J.pos[d0].uoff;
-                len = J.pos[d0].ucnt;
-            } else {
-                len = J.t.n;
-            }
-            const int e = min(fr.end, len);
-            if (fr.beg >= e) { vlo = 1; vhi = 0; }
-            else if (lst) { vlo = __ldg(lst + b0 + fr.beg); vhi = __ldg(lst + b0 + e - 1); }
-            else { vlo = fr.beg; vhi = e - 1; }
+            const JobRef v{&J};
+            const PosInfo *P = J.pos + d0;
+            const PosV p = load_pos(P);
+            // (a run's range as it stands; any other range counts in the plain list)
+            const Cand S = fr.in_run ? pick_warp<false>(v, p, P, M) : plain_list<false>(v, p, P, M);
+            int lo, hi, rb = 1, re = 1;
+            counts = list_range<false>(v, p, S, M, fr.beg, fr.end, fr.in_run, lo, hi);
+            if (lo < hi) row_range<false>(v, p, S, M, lo, hi, rb, re);
+            if (lane == 0) { W.frange()[0] = rb; W.frange()[1] = re; }   // read back only by a checkpoint
+            if (lo >= hi) { vlo = 1; vhi = 0; }
+            else { vlo = cand_id(S, lo); vhi = cand_id(S, hi - 1); }
+        } else if (lane == 0) {
+            W.frange()[0] = W.frange()[1] = -1;
         }
-        if (lane == 0) { W.frange()[0] = fr.beg; W.frange()[1] = fr.end; }   // read back only by a checkpoint
-        const bool count_len = fr.beg <= 0 && !fr.counted;
+        const bool count_len = counts && !fr.counted;
         const bool leaf0 = d0 == k - 1;
         int c0;
         {
@@ -2961,10 +3516,9 @@ cudaError_t launch_domain_init_buckets(const JobDesc *jobs, const long long *ver
     return cudaGetLastError();
 }
 
-cudaError_t launch_label_index(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
-                               cudaStream_t st) {
-    if (nverts <= 0) return cudaSuccess;
-    k_label_index<<<(unsigned)((nverts + BLOCK - 1) / BLOCK), BLOCK, 0, st>>>(jobs, vert_off, njobs, nverts);
+cudaError_t launch_label_index(const JobDesc *jobs, int njobs, cudaStream_t st) {
+    if (njobs <= 0) return cudaSuccess;
+    k_label_index<<<njobs, KMAX, 0, st>>>(jobs);
     return cudaGetLastError();
 }
 
@@ -3117,6 +3671,14 @@ __global__ void k_build_hubs(const int32_t *rowptr, const int32_t *col, const in
     }
 }
 }  // namespace
+
+cudaError_t launch_frames_to_rows(const JobDesc *jobs, int32_t *frames, long long n, long long pitch,
+                                  const unsigned long long *seq, int directed, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    if (directed) k_frames_to_rows<true><<<grid_for(n), BLOCK, 0, st>>>(jobs, frames, n, pitch, seq);
+    else k_frames_to_rows<false><<<grid_for(n), BLOCK, 0, st>>>(jobs, frames, n, pitch, seq);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_build_hubs(const int32_t *rowptr, const int32_t *col, const int32_t *hubs, int h, int dw,
                               uint64_t *bits, cudaStream_t st) {
