@@ -42,6 +42,7 @@ constexpr int HUB_MIN_DEGREE = 24;               // larger targets: bitset rows 
 constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device memory
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
 constexpr int POOL_CELLS = 1 << 15;
+constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
 constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
 constexpr int BLOCK_FIXPOINT_MAX_N = 16384;      // auto domain mode: in-block fixpoint for targets up to this
@@ -402,7 +403,8 @@ struct Workspace {
         ctask;
     DevBuf front[2], counts, offs, scan_tmp, total, splitctl;
     DevBuf pool, pseq, ctl, slab;
-    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart;
+    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft;
+    unsigned long long aepoch = 0;   // last launch's mark in aentry (0: the entries are to be cleared)
     std::vector<Job> hjobs;       // the call's pairs, reused (their vectors keep their capacity)
     std::vector<JobDesc> hdesc;   // host job records, reused
     std::vector<JobDesc> hfdesc;  // host records of the jobs with a filter block, reused
@@ -419,7 +421,7 @@ struct Workspace {
 #define SGE_WS_BUFFERS                                                                                             \
     &jobs, &fjobs, &ctr, &filt, &pos, &back, &ulist, &unit_off, &vert_off, &sizes, &task, &flag, &dent, &deoff, &vchg, \
         &cand, &ctask, &front[0], &front[1], &counts, &offs, &scan_tmp, &total, &splitctl, &pool, &pseq, &ctl, &slab, \
-        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart
+        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart, &aentry, &aleft
     // Every buffer of this workspace is used on `st` only: allocate them stream-ordered there.
     void bind(cudaStream_t st) {
         if (bound == st && st != nullptr) return;
@@ -1384,6 +1386,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     float split_ms = 0.f;   // device time of the cooperative split (CUDA events)
     float split_exec_ms = 0.f, search_exec_ms = 0.f;   // the kernels' own spans (device clock)
     int cur = 0, depth = 0, fstride = FRAME_HDR;
+    bool listed = false;   // the frontier is a list of frame addresses
     bool split_done = F0 == 0;
     if (resume != nullptr) {
         // continue from a checkpoint: its frames (mixed depths, stride FRAME_HDR + kmax) are the frontier
@@ -1397,7 +1400,11 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         }
         split_done = true;
     }
-    const int max_levels = std::max(0, std::min(o.split_depth > 0 ? o.split_depth : INT_MAX, kmax - 1));
+    const bool limited = o.state_budget > 0 || o.time_limit_ms > 0;
+    // the breadth-first run to the end of an unsharded CSR call takes the last position too (a wide
+    // last level is far cheaper there than frame by frame in the search kernel)
+    const bool to_the_end = o.split_depth <= 0 && kernel == SGE_KERNEL_CSR && !limited && shard_count == 1;
+    const int max_levels = std::max(0, std::min(o.split_depth > 0 ? o.split_depth : INT_MAX, to_the_end ? kmax : kmax - 1));
     const long long front_ints = o.frontier_kib > 0 ? 256ll * o.frontier_kib : FRONTIER_MAX_INTS;
     if (!split_done && resume == nullptr) {
         // the whole split as one cooperative launch.  Auto depth, CSR kernel: breadth-first
@@ -1407,7 +1414,6 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         // word-parallel expansion beats the split's per-candidate tests on dense targets.
         // A state budget or time limit is enforced by the search kernel, so with either
         // set the split also stops at the frame target and the search does the bulk.
-        const bool limited = o.state_budget > 0 || o.time_limit_ms > 0;
         const long long target = o.split_depth > 0 ? LLONG_MAX
                                  : (kernel == SGE_KERNEL_BITSET || limited) ? target_frames : (long long)INT_MAX;
         const long long cap_ints = std::max<long long>(F0 * FRAME_HDR, front_ints);
@@ -1419,7 +1425,9 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         CK(cudaMemcpyAsync(W.front[0].p, roots.data(), (size_t)F0 * sizeof(roots[0]), cudaMemcpyHostToDevice, st),
            "upload roots");
         const long long wcap = (long long)ctx->sms * 32 * search_warps_per_block();
-        const size_t ctl_words = (size_t)wcap + 16 + 2 * KMAX;   // (+ the level trace)
+        // (+ the level trace, + the asynchronous end's control lines)
+        const size_t async_at = ((size_t)wcap + 16 + 2 * KMAX + 15) & ~(size_t)15;
+        const size_t ctl_words = async_at + SPLIT_ASYNC_BYTES / 8;
         CK(W.splitctl.ensure(ctl_words * 8), "alloc split control");
         CK(cudaMemsetAsync(W.splitctl.p, 0, ctl_words * 8, st), "clear split control");
         long long *wtot = W.splitctl.as<long long>();
@@ -1429,6 +1437,25 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         constexpr long long SPLIT_MASKS = 1ll << 24;   // 64 MiB of replayed candidate ballots
         const bool have_masks = ordered && W.smask.ensure((size_t)SPLIT_MASKS * 4) == cudaSuccess;
         if (!have_masks) (void)cudaGetLastError();   // without the buffer the write pass tests again
+        // the asynchronous end of the split: not when the search may have to write a checkpoint, which
+        // reads untaken frames from the frontier buffer
+        SplitAsync async;
+        std::memset(&async, 0, sizeof(async));
+        if (to_the_end && !o.no_donation && ckpt_frames == nullptr) {
+            async.narrow = resident_warps;
+            async.ctl = wtot + async_at;
+            async.qcap = ASYNC_QUEUE;
+            const bool fresh = W.aentry.p == nullptr || W.aepoch + 1 >= (1ull << 24);
+            CK(W.aentry.ensure((size_t)ASYNC_QUEUE * 8), "alloc split queue");
+            CK(W.aleft.ensure((size_t)(ASYNC_QUEUE + 64 * wcap + async.narrow) * 8), "alloc split list");
+            if (fresh) {
+                CK(cudaMemsetAsync(W.aentry.p, 0, (size_t)ASYNC_QUEUE * 8, st), "clear split queue");
+                W.aepoch = 0;
+            }
+            async.epoch = ++W.aepoch;
+            async.entries = W.aentry.as<unsigned long long>();
+            async.left = W.aleft.as<const int32_t *>();
+        }
         if (!W.ev2) {
             CK(cudaEventCreate(&W.ev2), "event");
             CK(cudaEventCreate(&W.ev3), "event");
@@ -1439,12 +1466,17 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                                                  wcap, bar, res, sstat, count_ctr, directed ? 1 : 0,
                                                  serving ? 1 : 0, have_masks ? W.smask.as<uint32_t>() : nullptr,
                                                  SPLIT_MASKS, ordered ? 1 : 0,
+                                                 async,
                                                  trace_on() ? wtot + wcap + 16 : nullptr, st);
         if (le == cudaSuccess) {
             ++launches;
             CK(cudaEventRecord(W.ev3, st), "event record");
             long long r4[8] = {0, 0, 0, 0, 0, 0, 0, 0};
             int ss = 0;
+            unsigned long long nleft = 0;
+            if (async.narrow > 0)
+                CK(cudaMemcpyAsync(&nleft, static_cast<char *>(async.ctl) + SPLIT_ASYNC_LEFT, 8, cudaMemcpyDeviceToHost,
+                                   st), "read split list");
             CK(cudaMemcpyAsync(r4, res, sizeof(r4), cudaMemcpyDeviceToHost, st), "read split result");
             CK(cudaMemcpyAsync(&ss, sstat, sizeof(int), cudaMemcpyDeviceToHost, st), "read split status");
             CK(cudaStreamSynchronize(st), "split sync");
@@ -1452,6 +1484,10 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             split_exec_ms = span_ms((unsigned long long)r4[6], (unsigned long long)r4[7]);
             if (ss != 0) return fail(ctx, SGE_ERR_CUDA, "device split barrier timed out");
             F = r4[0];
+            if (F < 0) {   // ended asynchronously: what it left is listed frame by frame
+                listed = true;
+                F = (long long)nleft;
+            }
             cur = (int)r4[1];
             depth = (int)r4[2];
             fstride = FRAME_HDR + depth;
@@ -1465,7 +1501,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                     CK(cudaMemcpy(tr.data(), wtot + wcap + 16, tr.size() * 8, cudaMemcpyDeviceToHost), "read trace");
                     CK(cudaMemcpy(lv.data(), wtot, lv.size() * 8, cudaMemcpyDeviceToHost), "read trace");
                     long long prev = ~r4[6];
-                    for (int l = 0; l < depth; ++l) {
+                    for (int l = 0; l < depth && tr[(size_t)l] != 0; ++l) {
                         std::fprintf(stderr, "[sge]   level %d: %.1f us, %lld children, longest list %lld\n", l,
                                      (tr[(size_t)l] - prev) * 1e-3, lv[(size_t)l], tr[(size_t)KMAX + l]);
                         prev = tr[(size_t)l];
@@ -1529,6 +1565,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         std::memset(&C, 0, sizeof(C));
         bind_control(C, W.ctl.p);
         C.front = W.front[cur].as<int32_t>();
+        C.front_ptr = listed ? W.aleft.as<const int32_t *>() : nullptr;
         C.nfront = nfront;
         C.fstride = fstride;
         C.shard_index = shard_index;
@@ -1544,7 +1581,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         C.donate = o.no_donation ? 0 : 1;
         // a bitset-kernel donor hands out up to 16 of its shallowest pending survivors at once:
         // with few, large frontier frames the tail is split fastest that way
-        C.gran = o.steal_granularity > 0 ? o.steal_granularity : (kernel == SGE_KERNEL_BITSET ? 32 : 2);
+        C.gran = o.steal_granularity > 0 ? o.steal_granularity : 32;
         // donation cadence: a busy warp checks whether idle warps wait for work at most once
         // per this many iterations or this much device time.  Donating costs a few microseconds
         // (two fetch-and-adds and one cell write), so the bitset kernel checks every 50 us; the
@@ -1553,7 +1590,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         // (its deepest, heaviest subtrees) are shared before idle warps leave.
         const bool bits_k = kernel == SGE_KERNEL_BITSET;
         C.donate_iters = o.donate_every_iters > 0 ? o.donate_every_iters
-                         : (bits_k || serving ? (1 << 30) : 1024);
+                         : bits_k ? (1 << 30) : o.donate_every_us > 0 ? 1024 : 1;
         C.donate_ns = (unsigned long long)(o.donate_every_us > 0 ? o.donate_every_us
                                            : (bits_k ? 50 : (serving ? 20 : 500))) * 1000ull;
         // serving groups: a warp idle for 200 us (ten donation periods without a frame for it)

@@ -172,6 +172,7 @@ struct JobDesc {
 // Control block of one persistent search launch.
 struct SearchCtl {
     const int32_t *front;       // frontier frames, stride fstride
+    const int32_t *const *front_ptr;   // ... or, when not null, one by one
     long long nfront;           // frames of this shard
     int32_t fstride;
     int32_t shard_index, shard_count;
@@ -258,6 +259,18 @@ cudaError_t launch_domain_lists(const JobDesc *jobs, const int *task_job, const 
 cudaError_t launch_split(const JobDesc *jobs, const int32_t *fin, long long nf, int depth,
                          int32_t *counts, const long long *offs, int32_t *fout, int pass,
                          int count_ctr, int directed, cudaStream_t st);
+// The asynchronous end of the single-pass split (see split_async in sge_kernels.cu).
+struct SplitAsync {
+    long long narrow;              // 0: off
+    void *ctl;                     // SPLIT_ASYNC_BYTES of zeroed control words
+    unsigned long long *entries;   // [qcap]
+    long long qcap;
+    unsigned long long epoch;      // differs from every earlier launch's on `entries`, below 2^24, not 0
+    const int32_t **left;          // [split_left_cap]
+};
+constexpr size_t SPLIT_ASYNC_BYTES = 6 * 128;
+constexpr size_t SPLIT_ASYNC_LEFT = 4 * 128;   // ... of which this one, after the launch: frames left
+
 // The whole split as one cooperative launch (see k_split_coop): frames of
 // level L have stride FRAME_HDR + L in buffers of cap_ints ints; result[4] =
 // {final frame count, final buffer 0/1, levels done, last level's child count, -, -,
@@ -267,7 +280,7 @@ cudaError_t launch_split_coop(const JobDesc *jobs, long long f0, int32_t *buf0, 
                               long long target, int max_levels, long long *wtot, long long wtot_cap,
                               unsigned *bar, long long *result, int *status, int count_ctr, int directed,
                               int blocks_per_sm, uint32_t *masks, long long mask_total, int ordered,
-                              long long *trace, cudaStream_t st);
+                              const SplitAsync &async, long long *trace, cudaStream_t st);
 cudaError_t launch_scan(const int32_t *in, long long *out, long long n, long long *total,
                         void *tmp, size_t tmp_bytes, cudaStream_t st);
 size_t scan_tmp_bytes(long long n);

@@ -95,6 +95,13 @@ __device__ __forceinline__ int load_relaxed(const int *p) {
     return v;
 }
 
+// (unordered: a poll that orders nothing must not cost its SM the L1 an acquire drops)
+__device__ __forceinline__ unsigned long long load_relaxed(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, 0, code); }
 
 // Is `c` in the sorted row of `x` (with edge label `lab` when `chk`)?
@@ -1554,6 +1561,18 @@ struct SplitCtl {
     int32_t *buf0, *buf1;       // frame buffers of `cap_ints` ints each; a level-L frame has stride FRAME_HDR + L
     long long cap_ints;
     long long target;           // stop once the frontier has this many frames
+    // single-pass split: a level of fewer frames than `narrow` that does not grow ends the
+    // level-by-level expansion; the rest runs without barriers (see split_async).  0: never
+    long long narrow;
+    unsigned long long *qhead, *qtail;   // frame queue: tickets drawn, frames pushed
+    unsigned long long *qentry;          // [qcap]: epoch << 40 | frame's offset in the arena
+    long long qcap;
+    unsigned long long epoch;            // marks this launch's entries (24 bits)
+    long long *pend;                     // frames not finished, less the first level's
+    unsigned long long *top;             // arena ints handed out
+    int *stop;                           // out of arena or queue: what is left goes to `left`
+    unsigned long long *nleft;
+    const int32_t **left;                // [qcap + 64 per warp + the first level's frames]
     int max_levels;
     long long *wtot;            // [blocks]: children per block, then the blocks' exclusive offsets
     unsigned *bar;              // [2]: barrier count, generation (zeroed by the host)
@@ -1788,6 +1807,7 @@ struct SplitWarp {   // one warp's shared memory: the batch's frames, then its w
     const int2 *vld[32];       // null: the list is a run (its label is right, its degrees beside the ids)
     const uint64_t *filt[32];  // D(mu_i), or null
     const uint64_t *row[SPLIT_ROWS];   // the frames' constraint rows (null: that image has none)
+    int32_t *fr[32];           // split_async: the batch's frames
     int start[33];             // first of the frame's candidates among the batch's
     int job[32], lab[32], odeg[32], slab[32], li[32], nd[32];
     int qc[SPLIT_QUEUE];
@@ -1797,21 +1817,44 @@ struct SplitWarp {   // one warp's shared memory: the batch's frames, then its w
     unsigned char skip[32], next[32], nq[32];   // nq: constraints split_accept has to test
 };
 
+// A level's frames [f0, ..) and its children's buffer; places are reserved on the level's child
+// counter.  A reservation that ends past `cap_frames` raises `full` and writes nothing (the
+// level is then abandoned, see k_split_once).
+struct LevelOut {
+    const int32_t *fin;
+    long long f0;
+    int sin;
+    int32_t *fout;
+    long long cap_frames;
+    unsigned long long *lvl_ctr;
+    long long *full;
+    __device__ __forceinline__ const int32_t *frame(const SplitWarp &, int x) const { return fin + (f0 + x) * sin; }
+    // the first of `total` child frames of `stride` ints, or null
+    __device__ __forceinline__ int32_t *take(int total, int stride) {
+        unsigned long long to = 0;
+        if ((threadIdx.x & 31) == 0) to = atomicAdd(lvl_ctr, (unsigned long long)total);
+        to = __shfl_sync(FULL, to, 0);
+        if ((long long)(to + total) > cap_frames) {
+            if ((threadIdx.x & 31) == 0) *(volatile long long *)full = 1;
+            return nullptr;
+        }
+        return fout + (long long)to * stride;
+    }
+};
+
 // Tests the n <= 32 waiting candidates from `at` on against their frames' constraints and rule 1,
-// counts and hashes the accepted ones (hs: of frame `lane`), and appends their child frames at
-// offsets reserved on the level's child counter `lvl_ctr`.  A reservation that ends past
-// `cap_frames` raises `full` and writes nothing (the level is then abandoned, see k_split_once).
-template <bool DIR>
-__device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t *fin, long long f0, int depth,
-                                             int32_t *fout, long long cap_frames, unsigned long long *lvl_ctr,
-                                             long long *full, SplitWarp &W, int at, int n, unsigned long long &hs) {
+// counts and hashes the accepted ones (hs: of frame `lane`), and appends their child frames where
+// `out` says.
+template <bool DIR, class O>
+__device__ __forceinline__ void split_accept(const JobDesc *jobs, int depth, O &out, SplitWarp &W, int at, int n,
+                                             unsigned long long &hs) {
     const int lane = threadIdx.x & 31;
-    const int sin = FRAME_HDR + depth, sout = sin + 1;
+    const int sout = FRAME_HDR + depth + 1;
     bool ok = lane < n;
     const int L = W.ql[at + (ok ? lane : 0)], c = W.qc[at + (ok ? lane : 0)];
     const JobDesc &J = jobs[W.job[L]];
     const PosInfo *P = J.pos + depth;
-    const int *Mg = fin + (f0 + L) * sin + FRAME_HDR;
+    const int *Mg = out.frame(W, L) + FRAME_HDR;
     const int nq = ok ? W.nq[L] : 0;
     const int mq = (int)__reduce_max_sync(FULL, (unsigned)nq);
     if (mq > 0) {
@@ -1838,7 +1881,7 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t 
                 const JobDesc &Jx = jobs[W.job[Lx]];
                 if (q < W.nq[Lx] &&
                     !con_holds<DIR>(JobRef{&Jx}, load_pos(Jx.pos + depth), q + (q >= W.skip[Lx] ? 1 : 0), W.li[Lx],
-                                    W.qc[at + x], fin + (f0 + Lx) * sin + FRAME_HDR))
+                                    W.qc[at + x], out.frame(W, Lx) + FRAME_HDR))
                     bad |= 1u << x;
             }
             bad = __reduce_or_sync(FULL, bad);
@@ -1851,7 +1894,7 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t 
     const bool leaf = depth + 1 == J.k;
     for (unsigned m = __ballot_sync(FULL, ok && leaf); m;) {   // matches, one frame's at a time
         const int L0 = __shfl_sync(FULL, L, __ffs(m) - 1);
-        const int32_t *M0 = fin + (f0 + L0) * sin + FRAME_HDR;
+        const int32_t *M0 = out.frame(W, L0) + FRAME_HDR;
         const PosInfo *P0 = jobs[W.job[L0]].pos;
         unsigned long long psum = 0;
         for (int t = lane; t < depth; t += 32) psum += gterm(P0[t].pv, M0[t]);
@@ -1877,16 +1920,11 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t 
     }
     const int total = __shfl_sync(FULL, incl, 31);
     if (total == 0) return;
-    unsigned long long to = 0;
-    if (lane == 0) to = atomicAdd(lvl_ctr, (unsigned long long)total);
-    to = __shfl_sync(FULL, to, 0);
-    if ((long long)(to + total) > cap_frames) {
-        if (lane == 0) *(volatile long long *)full = 1;
-        return;
-    }
+    int32_t *const to = out.take(total, sout);
+    if (to == nullptr) return;
     const bool coop = depth >= SPLIT_COOP_DEPTH;
     for (int q = 0; q < r; ++q) {
-        int32_t *dst = fout + (long long)(to + incl - r + q) * sout;
+        int32_t *dst = to + (long long)(incl - r + q) * sout;
         split_child_header(dst, J, W.job[L], depth + 1, r, q);
         for (int t = 0; t < depth && !coop; ++t) dst[FRAME_HDR + t] = Mg[t];
         dst[FRAME_HDR + depth] = c;
@@ -1895,8 +1933,8 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t 
         for (unsigned m = __ballot_sync(FULL, r > 0); m; m &= m - 1) {
             const int x = __ffs(m) - 1;
             const int rx = __shfl_sync(FULL, r, x), Lx = __shfl_sync(FULL, L, x);
-            const int32_t *from = fin + (f0 + Lx) * sin + FRAME_HDR;
-            int32_t *dst = fout + ((long long)to + __shfl_sync(FULL, incl, x) - rx) * sout + FRAME_HDR;
+            const int32_t *from = out.frame(W, Lx) + FRAME_HDR;
+            int32_t *dst = to + (long long)(__shfl_sync(FULL, incl, x) - rx) * sout + FRAME_HDR;
             for (int t = lane; t < depth; t += 32) {
                 const int y = from[t];
                 for (int q = 0; q < rx; ++q) dst[(long long)q * sout + t] = y;
@@ -1904,13 +1942,10 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, const int32_t 
         }
 }
 
-// Frames [f0, f0 + nf) of a split level (nf <= 32), by one warp.  Returns the longest list.
-template <bool DIR>
-__device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *fin, long long f0, int nf, int depth,
-                                           int32_t *fout, long long cap_frames, unsigned long long *lvl_ctr,
-                                           long long *full, SplitWarp &W) {
+// Expands the nf <= 32 frames of `out`, all at `depth`, by one warp.  Returns the longest list.
+template <bool DIR, class O>
+__device__ __forceinline__ int split_batch(const JobDesc *jobs, int nf, int depth, O &out, SplitWarp &W) {
     const int lane = threadIdx.x & 31;
-    const int sin = FRAME_HDR + depth;
     // the frames' lists: few frames share the warp's lanes out among them
     int G = 32;
     while (G > 1 && 32 / G < nf) G >>= 1;
@@ -1919,7 +1954,7 @@ __device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *f
     {
         const int sub = lane & (G - 1), x = lane / G;
         const bool have = x < nf;
-        const int32_t *fr = fin + (f0 + (have ? x : 0)) * sin;
+        const int32_t *fr = out.frame(W, have ? x : 0);
         const int jx = fr[0];
         const JobDesc &J = jobs[jx];
         const JobRef v{&J};
@@ -2005,7 +2040,7 @@ __device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *f
                 const int skip = W.skip[x], first = W.next[x] - (W.next[x] > skip ? 1 : 0), i = e - W.rbeg[x];
                 const int y = i == 0 ? first : i == first ? 0 : i;
                 const uint64_t *row = con_row<DIR>(JobRef{&J}, load_pos(J.pos + depth), y + (y >= skip ? 1 : 0),
-                                                   fin + (f0 + x) * sin + FRAME_HDR);
+                                                   out.frame(W, x) + FRAME_HDR);
                 W.row[e] = row;
                 if (row == nullptr) W.nq[x] = (unsigned char)bx;
             }
@@ -2103,11 +2138,11 @@ __device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *f
         __syncwarp();
         while (n >= 32) {   // full warps of them, from the end
             n -= 32;
-            split_accept<DIR>(jobs, fin, f0, depth, fout, cap_frames, lvl_ctr, full, W, n, 32, hs);
+            split_accept<DIR>(jobs, depth, out, W, n, 32, hs);
             __syncwarp();
         }
     }
-    if (n > 0) split_accept<DIR>(jobs, fin, f0, depth, fout, cap_frames, lvl_ctr, full, W, 0, n, hs);
+    if (n > 0) split_accept<DIR>(jobs, depth, out, W, 0, n, hs);
     __syncwarp();
     // counters: segmented sums over runs of consecutive lanes with the same job, one atomic per run
     const bool leaf = j >= 0 && depth + 1 == jobs[j].k;
@@ -2140,6 +2175,224 @@ __device__ __forceinline__ int split_batch(const JobDesc *jobs, const int32_t *f
     return warp_max(len);
 }
 
+// ------------------------------------------- the split without barriers
+//
+// Once the levels are narrow and no longer grow, a level lasts as long as its slowest frame and
+// a barrier, however little there is to do (60-126 levels of 12-45 us on deep patterns).  The
+// rest of the split then runs asynchronously: a warp expands a batch of frames of one depth,
+// keeps up to 32 children as its next batch, and pushes the others -- all but one while other
+// warps wait for work -- to a queue whose tickets are drawn in order, one frame to a ticket.
+// Children are written to a bump-allocated arena (the frontier buffer the levels no longer need), a
+// chunk per warp at a time, and handed on only at the end of the batch.  A batch whose
+// children no longer fit is abandoned like a level: its frames are counted and become counted
+// ranges (or, on the last position, empty ones), every warp stops, and what was not expanded is
+// listed for the search kernel.  Waits are bounded by the barrier's guard and end when no frame is
+// pending or the stop flag is up.  Bound by the dependent loads of one batch (header, tables,
+// runs, ids, constraint rows: 5-10 us).  It starts below one frame per resident warp: 160 network
+// queries 5.7 -> 4.1 ms a call, 64 with domains 5.3 -> 4.7, 96 served 4.1 -> 3.0, 10 deep patterns
+// 2.0 -> 1.8, 200,000 molecule pairs 9.75 -> 9.6 (the last position taken here too: 24 directed
+// patterns 1.9 -> 1.5 ms).
+// Arena ints a warp takes at once: a share of the arena, within these limits.
+constexpr int ASYNC_CHUNK_MIN = 256, ASYNC_CHUNK_MAX = 8192;
+constexpr int ASYNC_SEGS = 8;       // pieces of the arena one batch's children may lie in
+constexpr unsigned long long ASYNC_OFFSET = (1ull << 40) - 1;
+
+struct AsyncOut {
+    const SplitCtl &S;
+    int32_t *arena;
+    long long chunk;                 // ints taken at once
+    long long pos, end;              // the warp's chunk: free ints [pos, end)
+    int nseg;                        // the batch's children: pieces of the arena ...
+    bool full;                       // ... or no room for them
+    long long *seg;                  // [ASYNC_SEGS] first int (shared memory)
+    int *segn;                       // [ASYNC_SEGS] frames
+    __device__ __forceinline__ const int32_t *frame(const SplitWarp &W, int x) const { return W.fr[x]; }
+    __device__ __forceinline__ int32_t *take(int total, int stride) {
+        const int lane = threadIdx.x & 31;
+        const long long need = (long long)total * stride;
+        if (full) return nullptr;
+        if (pos + need > end) {
+            // (a batch that goes on to take more takes four times as much each time)
+            const long long size = max(need, chunk << (2 * nseg));
+            unsigned long long t = 0;
+            if (lane == 0) t = atomicAdd(S.top, (unsigned long long)size);
+            t = __shfl_sync(FULL, t, 0);
+            if (nseg == ASYNC_SEGS || (long long)t + size > S.cap_ints) {
+                full = true;
+                return nullptr;
+            }
+            pos = (long long)t;
+            end = pos + size;
+            if (lane == 0) {
+                seg[nseg] = pos;
+                segn[nseg] = 0;
+            }
+            ++nseg;
+        } else if (nseg == 0) {
+            if (lane == 0) {
+                seg[0] = pos;
+                segn[0] = 0;
+            }
+            nseg = 1;
+        }
+        if (lane == 0) segn[nseg - 1] += total;
+        int32_t *p = arena + pos;
+        pos += need;
+        return p;
+    }
+};
+
+// Frame of queue ticket t if it is there (tickets below F: the first level's frames); a fence
+// has to follow before the frame is read.
+__device__ __forceinline__ int32_t *async_frame(const SplitCtl &S, int32_t *fin, long long F, int sin, int32_t *arena,
+                                                long long t) {
+    if (t < F) return fin + t * sin;
+    if (t - F >= S.qcap) return nullptr;
+    const unsigned long long e = load_relaxed(S.qentry + (t - F));
+    return (e >> 40) == S.epoch ? arena + (e & ASYNC_OFFSET) : nullptr;
+}
+
+__device__ __forceinline__ void async_leave(const SplitCtl &S, const int32_t *fr) {
+    S.left[atomicAdd(S.nleft, 1ull)] = fr;
+}
+
+// Frames [0, F) of `fin`, of stride sin (all at one depth), searched to the end or until the arena
+// or the queue is full.
+template <bool DIR>
+__device__ __forceinline__ void split_async(const JobDesc *jobs, const SplitCtl &S, int32_t *fin, int32_t *arena,
+                                            long long F, int sin, SplitWarp &W, long long *seg, int *segn) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long chunk = min((long long)ASYNC_CHUNK_MAX, max((long long)ASYNC_CHUNK_MIN, S.cap_ints / (2 * nw)));
+    AsyncOut out{S, arena, chunk, 0, 0, 0, false, seg, segn};
+    int deepest = sin - FRAME_HDR;   // depth the warp's finished batches reached
+    long long held = 0;   // tickets drawn and not yet served: [held, held + hn)
+    int hn = 0;
+    int nloc = 0, depth = 0;   // the next batch, in W.fr
+    for (;;) {
+        if (nloc == 0) {
+            int got = 0;
+            if (lane == 0) {
+                unsigned backoff = 32;
+                const unsigned long long t0 = globaltimer();
+                for (;;) {
+                    if (load_relaxed(S.stop) != 0) break;
+                    if (hn == 0) {
+                        const long long ready = F + (long long)load_relaxed(S.qtail) - (long long)load_relaxed(S.qhead);
+                        hn = (int)max(1ll, min(32ll, ready / (2 * nw)));
+                        held = (long long)atomicAdd(S.qhead, (unsigned long long)hn);
+                    }
+                    if (async_frame(S, fin, F, sin, arena, held) != nullptr) {
+                        got = 1;
+                        break;
+                    }
+                    if (F + (long long)load_relaxed(reinterpret_cast<unsigned long long *>(S.pend)) == 0) break;
+                    __nanosleep(backoff);
+                    if (backoff < 512) backoff <<= 1;
+                    if (globaltimer() - t0 > BARRIER_GUARD_NS) {
+                        set_status(S.status, -3);
+                        break;
+                    }
+                }
+            }
+            got = __shfl_sync(FULL, got, 0);
+            held = __shfl_sync(FULL, held, 0);
+            hn = __shfl_sync(FULL, hn, 0);
+            if (!got) break;
+            // the tickets' frames that are there, as long as they share a depth
+            int32_t *fr = lane < hn ? async_frame(S, fin, F, sin, arena, held + lane) : nullptr;
+            __threadfence();
+            const int d = fr ? fr[1] & FRAME_DEPTH_MASK : -1;
+            depth = __shfl_sync(FULL, d, 0);
+            nloc = __ffs(~__ballot_sync(FULL, fr != nullptr && d == depth)) - 1;
+            if (nloc < 0) nloc = 32;
+            if (lane < nloc) W.fr[lane] = fr;
+            held += nloc;
+            hn -= nloc;
+            __syncwarp();
+        }
+        const int n = nloc;
+        out.nseg = 0;
+        out.full = false;
+        split_batch<DIR>(jobs, n, depth, out, W);
+        __syncwarp();
+        int nc = 0;
+        for (int q = 0; q < out.nseg; ++q) nc += segn[q];
+        // tickets waiting for frames
+        long long waiting = 0;
+        if (lane == 0 && nc > 1)
+            waiting = (long long)load_relaxed(S.qhead) - (F + (long long)load_relaxed(S.qtail));
+        waiting = __shfl_sync(FULL, waiting, 0);
+        // children to keep as the next batch, and to push
+        int keep = min(nc, 32);
+        if (waiting > 0 && nc > 1) keep = (int)min((long long)keep, max(1ll, nc - waiting));
+        const int push = nc - keep;
+        unsigned long long t = 0;
+        bool fail = out.full;
+        if (!fail && push > 0) {
+            if (lane == 0) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(S.pend), (unsigned long long)push);
+                t = atomicAdd(S.qtail, (unsigned long long)push);
+            }
+            t = __shfl_sync(FULL, t, 0);
+            fail = (long long)t + push > S.qcap;
+        }
+        if (fail) {   // the batch's children are dropped: its frames, counted, go to the search
+            if (lane < n) {
+                int32_t *fr = W.fr[lane];
+                if (depth + 1 == jobs[fr[0]].k) {
+                    fr[2] = fr[3] = 1;
+                } else {
+                    fr[1] |= FRAME_COUNTED;
+                    if (fr[2] < 0) { fr[2] = 0; fr[3] = 0x7fffffff; }
+                }
+                async_leave(S, fr);
+            }
+            nloc = 0;
+            if (lane == 0) atomicExch(S.stop, 1);
+            break;
+        }
+        const int stride = FRAME_HDR + depth + 1;
+        __threadfence();
+        __syncwarp();
+        int32_t *mine = nullptr;
+        for (int i0 = 0; i0 < nc; i0 += 32) {
+            const int i = i0 + lane;
+            if (i < nc) {
+                int q = 0, rest = i;
+                while (rest >= segn[q]) rest -= segn[q++];
+                const long long at = seg[q] + (long long)rest * stride;
+                if (i < keep) mine = arena + at;   // (keep <= 32: one per lane)
+                else store_release(S.qentry + t + (i - keep), S.epoch << 40 | (unsigned long long)at);
+            }
+        }
+        __syncwarp();
+        if (lane < keep) W.fr[lane] = mine;
+        if (lane == 0 && keep != n)
+            atomicAdd(reinterpret_cast<unsigned long long *>(S.pend), (unsigned long long)(long long)(keep - n));
+        __syncwarp();
+        nloc = keep;
+        ++depth;
+        deepest = max(deepest, depth);
+        if (nloc > 0) {   // (one lane's read: the warp leaves as one)
+            const int stop = lane == 0 ? load_relaxed(S.stop) : 0;
+            if (__shfl_sync(FULL, stop, 0) != 0) break;
+        }
+    }
+    if (lane < nloc) async_leave(S, W.fr[lane]);
+    if (lane == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 2), (unsigned long long)deepest);
+    // (either the stop flag is up or no frame is pending: the same for every warp)
+    grid_barrier(S.bar, S.bar + 1, S.status);
+    if (load_relaxed(S.stop) != 0) {   // (no warp-wide operation below)
+        int32_t *fr = lane < hn ? async_frame(S, fin, F, sin, arena, held + lane) : nullptr;
+        if (fr) async_leave(S, fr);
+        const long long h = (long long)load_relaxed(S.qhead);
+        const long long e = F + min((long long)load_relaxed(S.qtail), S.qcap);
+        for (long long x = h + blockIdx.x * (long long)blockDim.x + threadIdx.x; x < e; x += (long long)gridDim.x * blockDim.x)
+            if (int32_t *y = async_frame(S, fin, F, sin, arena, x)) async_leave(S, y);
+    }
+}
+
 // Single-pass split (unsharded runs; the caller's shard counts the levels).
 // Bound by the gathers of the wide levels (id and degree streamed, one bitset word per
 // constraint tested) and, on narrow ones, by the dependent loads of one frame and the barrier.
@@ -2158,6 +2411,8 @@ template <bool DIR>
 __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, long long f0, SplitCtl S) {
     __shared__ SplitWarp Wsh[WARPS_PER_BLOCK];
     const int lane = threadIdx.x & 31;
+    __shared__ long long seg[WARPS_PER_BLOCK][ASYNC_SEGS];
+    __shared__ int segn[WARPS_PER_BLOCK][ASYNC_SEGS];
     SplitWarp &W = Wsh[threadIdx.x >> 5];
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2165,16 +2420,20 @@ __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, lo
     long long F = f0;
     int cur = 0, level = 0;
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 6), ~globaltimer());
+    long long before = 0;   // the last level's frames
+    bool narrow = false;
     for (; level < S.max_levels; ++level) {
-        if (F == 0 || F >= S.target) break;
+        narrow = F > 0 && F < S.narrow && F <= before;
+        if (F == 0 || F >= S.target || narrow) break;
+        before = F;
         int32_t *fin = cur ? S.buf1 : S.buf0;
         int32_t *fout = cur ? S.buf0 : S.buf1;
         const int sin = FRAME_HDR + level, sout = FRAME_HDR + level + 1;
         const long long lo = F * w / nw, hi = F * (w + 1) / nw;
         int longest = 0;
-        for (long long f = lo; f < hi; f += 32)
-            longest = max(longest, split_batch<DIR>(jobs, fin, f, (int)min(32ll, hi - f), level, fout,
-                                                    S.cap_ints / sout, lvl_ctr + level, S.result + 5, W));
+        LevelOut out{fin, lo, sin, fout, S.cap_ints / sout, lvl_ctr + level, S.result + 5};
+        for (; out.f0 < hi; out.f0 += 32)
+            longest = max(longest, split_batch<DIR>(jobs, (int)min(32ll, hi - out.f0), level, out, W));
         if (S.trace && lane == 0 && longest > 0)
             atomicMax(reinterpret_cast<unsigned long long *>(S.trace + KMAX + level), (unsigned long long)longest);
         grid_barrier(S.bar, S.bar + 1, S.status);
@@ -2196,10 +2455,13 @@ __global__ void __launch_bounds__(BLOCK, 4) k_split_once(const JobDesc *jobs, lo
         F = (long long)*(volatile unsigned long long *)(lvl_ctr + level);
         cur ^= 1;
     }
+    if (narrow)
+        split_async<DIR>(jobs, S, cur ? S.buf1 : S.buf0, cur ? S.buf0 : S.buf1, F, FRAME_HDR + level, W,
+                         seg[threadIdx.x >> 5], segn[threadIdx.x >> 5]);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        S.result[0] = F;
+        S.result[0] = narrow ? -1 : F;   // (-1: the frames are those listed in `left`, *nleft of them)
         S.result[1] = cur;
-        S.result[2] = level;
+        if (!narrow) S.result[2] = level;
     }
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 7), globaltimer());
 }
@@ -2309,9 +2571,10 @@ __device__ long long queue_reserve(const SearchCtl &C) {
     return -1;
 }
 
-// Consumer holding ticket t: is its frame published?
+// Consumer holding ticket t: is its frame published?  (An unordered poll: an acquire at every look
+// of every idle warp drops its SM's L1 under the busy ones; acquire_frame fences before it reads.)
 __device__ __forceinline__ bool queue_ready(const SearchCtl &C, unsigned long long t) {
-    return load_acquire(C.pseq + t % (unsigned long long)C.pcap) == t + 1;
+    return load_relaxed(C.pseq + t % (unsigned long long)C.pcap) == t + 1;
 }
 
 // Consumer holding ticket t wants to leave: true if it left (no frame will
@@ -2363,6 +2626,69 @@ __device__ bool push_frame(const SearchCtl &C, int j, int depth, int beg, int en
     }
     __syncwarp();
     return true;
+}
+
+// Warp-collective: push one frame [j, depth, -1, -1, M[0..depth-2], c] for every lane in `mask`
+// (c: the lane's last image), all tickets drawn with one fetch-and-add and every lane working on
+// its own cell.  Some cells may not take a frame (a consumer that left, a cell still in its previous
+// lap): the frames go out lowest lane first, and the lanes whose frame was taken, the lowest ones of
+// `mask`, are returned (a checkpoint writes what is left of a chunk as one range from its lowest
+// pending survivor on).
+__device__ unsigned push_children(const SearchCtl &C, int j, int depth, const int *M, unsigned mask, int c) {
+    const int lane = threadIdx.x & 31;
+    const int n = __popc(mask);
+    const unsigned long long cap = (unsigned long long)C.pcap;
+    unsigned long long t = 0;
+    if (lane == 0) {
+        atomicAdd(C.outstanding, n);
+        t = atomicAdd(C.ptail, (unsigned long long)n);
+    }
+    t = __shfl_sync(FULL, t, 0) + __popc(mask & ((1u << lane) - 1u));
+    bool got = false;
+    if ((mask >> lane) & 1u) {
+        unsigned long long *seq = C.pseq + t % cap;
+        for (long long spin = 0;; ++spin) {
+            const unsigned long long sv = load_acquire(seq);
+            if (sv == t) {
+                if (atomicCAS(seq, t, t | CELL_LOCK) == t) {
+                    got = true;
+                    break;
+                }
+                continue;                                   // consumer t left meanwhile: look again
+            }
+            if ((sv & ~CELL_LOCK) > t) break;               // consumer t left
+            if (spin > RESERVE_SPIN_LIMIT) {                // the cell's previous lap never ended
+                set_status(C.status, -3);
+                break;
+            }
+            __nanosleep(128);
+        }
+    }
+    const unsigned locked = __ballot_sync(FULL, got);
+    int32_t *cell = C.pool + (size_t)(t % cap) * POOL_STRIDE;
+    // the r-th locked cell takes the r-th lane's frame
+    const int from = got ? (int)__fns(mask, 0, __popc(locked & ((1u << lane) - 1u)) + 1) : lane;
+    c = __shfl_sync(FULL, c, from);
+    if (got) {
+        cell[0] = j; cell[1] = depth; cell[2] = -1; cell[3] = -1;
+        cell[FRAME_HDR + depth - 1] = c;
+    }
+    const unsigned sent = __reduce_or_sync(FULL, got ? 1u << from : 0u);
+    for (unsigned m = locked; m; m &= m - 1) {
+        int32_t *to = C.pool + (size_t)(__shfl_sync(FULL, t, __ffs(m) - 1) % cap) * POOL_STRIDE + FRAME_HDR;
+        for (int i = lane; i < depth - 1; i += 32) to[i] = M[i];
+    }
+    __syncwarp();
+    if (got) {
+        __threadfence();
+        store_release(C.pseq + (t % cap), t + 1);   // publish (clears the lock)
+    }
+    if (lane == 0) {
+        if (n > __popc(sent)) atomicSub(C.outstanding, n - __popc(sent));
+        if (sent) atomicAdd(C.donations, (unsigned long long)__popc(sent));
+    }
+    __syncwarp();
+    return sent;
 }
 
 struct Frame {
@@ -2471,7 +2797,7 @@ __device__ bool acquire_frame(const SearchCtl &C, int *M, Frame &fr, unsigned lo
                 if (ticket >= 0 && !queue_leave(C, (unsigned long long)ticket, true)) { kind = 2; idx = ticket; }
                 else kind = 0;
             } else {
-                if (ticket < 0 && load_acquire(C.fnext) < (unsigned long long)C.nfront) {
+                if (ticket < 0 && load_relaxed(C.fnext) < (unsigned long long)C.nfront) {
                     const unsigned long long f = atomicAdd(C.fnext, 1ull);
                     if ((long long)f < C.nfront) { kind = 1; idx = (long long)f; }
                 }
@@ -2515,7 +2841,7 @@ __device__ bool acquire_frame(const SearchCtl &C, int *M, Frame &fr, unsigned lo
     const int32_t *src;
     if (kind == 1) {
         const long long g = idx * (long long)C.shard_count + C.shard_index;
-        src = C.front + g * C.fstride;
+        src = C.front_ptr ? C.front_ptr[g] : C.front + g * C.fstride;
     } else {
         if (lane == 0) __threadfence();
         __syncwarp();
@@ -2571,7 +2897,7 @@ __device__ __forceinline__ bool donation_claim(const SearchCtl &C) {
     int ok = 0;
     if ((threadIdx.x & 31) == 0 && C.donate) {
         // consumer tickets not yet matched by a producer = idle warps waiting for a frame
-        const long long waiting = (long long)(load_acquire(C.phead) - load_acquire(C.ptail));
+        const long long waiting = (long long)(load_relaxed(C.phead) - load_relaxed(C.ptail));
         if (waiting > 0 && atomicAdd(C.promised, 1) < waiting) ok = 1;
         else if (waiting > 0) atomicSub(C.promised, 1);
     }
@@ -2590,15 +2916,9 @@ __device__ __forceinline__ void donation_done(const SearchCtl &C) {
 // when mu_i is unparented), scanned 32 at a time, one candidate per lane; each
 // lane makes its candidate's local tests, the constraints are tested spread over
 // the warp (cand_chunk), and a ballot compacts the chunk's survivors.  Per warp,
-// shared memory holds M, the level records and a compact copy of the job's
-// position table; the job's pointers stay in registers.
+// shared memory holds M and the level records; the job's pointers stay in registers.
 
 __host__ __device__ __forceinline__ size_t round16(size_t x) { return (x + 15) & ~(size_t)15; }
-
-struct PosC {                // hot fields of one position
-    int16_t pv, par, bb, bc;
-    int32_t lab, odeg, ideg, pel, flags;
-};
 
 // What a level's candidates are entries of.
 enum : int16_t { LIST_VERTICES = 0, LIST_DOMAIN, LIST_ROW, LIST_IN_ROW, LIST_RUN, LIST_IN_RUN };
@@ -2614,7 +2934,7 @@ struct LvCsr {
 };
 
 __host__ __device__ __forceinline__ size_t csr_smem_per_warp(int kmax) {
-    return round16((size_t)kmax * sizeof(LvCsr) + ((size_t)kmax + 32) * sizeof(int) + (size_t)kmax * sizeof(PosC));
+    return round16((size_t)kmax * sizeof(LvCsr) + ((size_t)kmax + 32) * sizeof(int));
 }
 
 // A job's pointers in registers, read like JobRef.
@@ -2646,10 +2966,6 @@ struct CsrJob {
     __device__ __forceinline__ int dw() const { return dw_; }
     __device__ __forceinline__ int flags() const { return flags_; }
 };
-
-__device__ __forceinline__ PosV csr_pos(const PosC &q) {
-    return PosV{q.pv, q.par, q.lab, q.odeg, q.ideg, q.pel, q.bb, q.bc, q.flags};
-}
 
 // A level's list as cand_chunk reads it.
 template <bool DIR>
@@ -2685,7 +3001,6 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
     LvCsr *lv = reinterpret_cast<LvCsr *>(base);
     int *M = reinterpret_cast<int *>(lv + kmax);
     int *Cs = M + kmax;
-    PosC *tab = reinterpret_cast<PosC *>(Cs + 32);
 
     const unsigned long long deadline = C.deadline_ns ? globaltimer() + C.deadline_ns : 0ull;
     Frame fr;
@@ -2705,14 +3020,6 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
             B.ulist_ = J.ulist; B.vld_ = J.t.vld; B.filt_ = J.filt; B.adj_ = J.t.adj; B.back_ = J.back; B.pos = J.pos;
             B.hub_slot_ = J.t.hub_slot; B.hub_bits_ = J.t.hub_bits; B.runs_ = J.t.runs; B.plidx_ = J.plidx;
             B.n_ = J.t.n; B.dw_ = J.t.dw; B.k = J.k; B.flags_ = J.flags;
-            for (int t = lane; t < B.k; t += 32) {
-                const PosInfo P = J.pos[t];
-                PosC q;
-                q.pv = (int16_t)P.pv; q.par = (int16_t)P.par; q.bb = (int16_t)P.bbeg; q.bc = (int16_t)P.bcnt;
-                q.lab = P.lab; q.odeg = P.odeg; q.ideg = P.ideg; q.pel = P.pel; q.flags = P.flags;
-                tab[t] = q;
-            }
-            __syncwarp();
         }
         const int k = B.k, d0 = fr.depth;
         // a counted frame re-tests its range at level d0 without counting it again
@@ -2721,11 +3028,36 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
         // since the last fold (every 64 iterations): an iteration adds at most 32 nodes and a
         // candidate list below 2^24 states (longer lists go straight to the 64-bit total)
         unsigned st32 = 0, nd32 = 0, mt32 = 0;
+        const bool eager = C.donate_iters == 1;   // look for idle warps on every second iteration
         bool counts0 = true;   // the frame counted its first node's states
-        // set up level `l` (positions 0..l-1 assigned) and count the node's states: a range
-        // frame counts them if it starts the node, a counted frame not at all
+        // scan the next 32 candidates [cur, ..) of level `l`'s list
+        auto scan = [&](int l, const PosV &p, const Cand &S, int cur, int end) {
+            int c;
+            unsigned bal = cand_chunk<DIR>(B, p, B.pos + l, S, cur, end, M, Cs, c);
+            if (l != quiet) nd32 += __popc(bal);
+            if (l == k - 1) {
+                mt32 += __popc(bal);
+                if (bal) {
+                    // hash prefix sum_{t < l} g(mu_t, M_t), only when this chunk has matches
+                    unsigned long long ps = 0;
+                    for (int t = lane; t < l; t += 32) ps += gterm(__ldg(&B.pos[t].pv), M[t]);
+                    ps = warp_sum(ps);
+                    if ((bal >> lane) & 1u) {
+                        hs += fmix64(ps + gterm(p.pv, c));
+                        if (J.mbuf) emit_match(J, M, l, c);
+                    }
+                }
+                bal = 0;
+            }
+            __syncwarp();
+            if (lane == 0) { lv[l].cur = min(cur + 32, end); lv[l].mask = bal; lv[l].cbase = cur; }
+            __syncwarp();
+        };
+        // set up level `l` (positions 0..l-1 assigned), count the node's states -- a range
+        // frame counts them if it starts the node, a counted frame not at all -- and, below the
+        // frame's first node, scan its first candidates while the list is at hand
         auto setup = [&](int l, int beg, int endv, bool in_run) {
-            const PosV p = csr_pos(tab[l]);
+            const PosV p = load_pos(B.pos + l);
             const Cand S = pick_warp<DIR>(B, p, B.pos + l, M);
             int cur, end;
             const bool counts = list_range<DIR>(B, p, S, M, beg, endv, in_run, cur, end);
@@ -2746,6 +3078,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                 if (S.raw < (1 << 24)) st32 += (unsigned)S.raw;
                 else st += (unsigned long long)S.raw;
             }
+            if (l > d0 && cur < end) scan(l, p, S, cur, end);
         };
         // candidate of entry e of level l's list
         auto entry = [&](const LvCsr &L, int e) {
@@ -2771,49 +3104,51 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                     st = 0;
                 }
                 if (must_stop(C, J, st, deadline, last_check, last_cancel)) { stopped = true; break; }
-                if ((iter - last_don_iter >= (unsigned)C.donate_iters || last_check - last_don_ns >= C.donate_ns) &&
-                    donation_claim(C)) {
-                    // donate the shallowest unexplored work: half of an unscanned
-                    // range, else up to `gran` pending survivors as new search nodes
-                    last_don_iter = iter;
-                    last_don_ns = last_check;
-                    for (int l = d0; l <= lvl && l + 1 + DONATE_MIN_LEVELS <= k; ++l) {
-                        LvCsr &L = lv[l];
-                        int rem = L.end - L.cur;
-                        if (rem >= 64 && L.kind >= LIST_RUN) {   // past the entries no part may start in
-                            const PosV p = csr_pos(tab[l]);
-                            const int drop = run_drop<DIR>(B, p, csr_list<DIR>(B, p, L, M), M);
-                            __syncwarp();
-                            if (lane == 0 && L.cur < drop) L.cur = min(drop, L.end);
-                            __syncwarp();
-                            rem = L.end - L.cur;
-                        }
-                        if (rem >= 64) {
-                            const int mid = L.cur + ((rem / 2 + 31) & ~31);
-                            const int run = L.kind >= LIST_RUN ? FRAME_RUN : 0;
-                            if (push_frame(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0) | run, mid, L.end, M, l,
-                                           -1)) {
-                                __syncwarp();
-                                if (lane == 0) L.end = mid;
-                                __syncwarp();
-                            }
-                            break;
-                        }
-                        if (L.mask != 0) {
-                            int given = 0;
-                            while (L.mask != 0 && given < C.gran) {
-                                const unsigned m = L.mask;
-                                const int c = entry(L, L.cbase + __ffs(m) - 1);
-                                if (!push_frame(C, fr.job, l + 1, -1, -1, M, l, c)) break;
-                                __syncwarp();
-                                if (lane == 0) L.mask = m & (m - 1);
-                                __syncwarp();
-                                ++given;
-                            }
-                            break;
-                        }
+            }
+            if (C.donate && ((eager && (iter & 1) == 0) || iter - last_don_iter >= (unsigned)C.donate_iters ||
+                             ((iter & 7) == 0 && last_check - last_don_ns >= C.donate_ns))) {
+                // idle warps waiting for a frame (their tickets run ahead of the producers')?
+                last_don_iter = iter;
+                last_don_ns = last_check;
+                int want = 0;
+                if (lane == 0)
+                    want = (int)max(-1ll, min(32ll, (long long)(load_relaxed(C.phead) - load_relaxed(C.ptail))));
+                want = __shfl_sync(FULL, want, 0);
+                // donate the shallowest unexplored work: half of an unscanned range, else up to
+                // `gran` pending survivors as new search nodes
+                for (int l = d0; want > 0 && l <= lvl && l + 1 + DONATE_MIN_LEVELS <= k; ++l) {
+                    LvCsr &L = lv[l];
+                    int rem = L.end - L.cur;
+                    if (rem >= 64 && L.kind >= LIST_RUN) {   // past the entries no part may start in
+                        const PosV p = load_pos(B.pos + l);
+                        const int drop = run_drop<DIR>(B, p, csr_list<DIR>(B, p, L, M), M);
+                        __syncwarp();
+                        if (lane == 0 && L.cur < drop) L.cur = min(drop, L.end);
+                        __syncwarp();
+                        rem = L.end - L.cur;
                     }
-                    donation_done(C);
+                    if (rem >= 64) {
+                        const int mid = L.cur + ((rem / 2 + 31) & ~31);
+                        const int run = L.kind >= LIST_RUN ? FRAME_RUN : 0;
+                        if (push_frame(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0) | run, mid, L.end, M, l, -1)) {
+                            __syncwarp();
+                            if (lane == 0) L.end = mid;
+                            __syncwarp();
+                        }
+                        break;
+                    }
+                    unsigned m = L.mask;
+                    // (the current level keeps one for this warp, which would else be out of work)
+                    const int most = min(min(want, C.gran), __popc(m) - (l == lvl ? 1 : 0));
+                    if (most > 0) {
+                        // the lowest ones, one per lane
+                        while (__popc(m) > most) m &= ~(0x80000000u >> __clz(m));
+                        const int c = (m >> lane) & 1u ? entry(L, L.cbase + lane) : 0;
+                        const unsigned sent = push_children(C, fr.job, l + 1, M, m, c);
+                        if (lane == 0) L.mask &= ~sent;
+                        __syncwarp();
+                        break;
+                    }
                 }
             }
             LvCsr &L = lv[lvl];
@@ -2825,28 +3160,8 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                     --lvl;
                     continue;
                 }
-                const PosV p = csr_pos(tab[lvl]);
-                const Cand S = csr_list<DIR>(B, p, L, M);
-                int c;
-                unsigned bal = cand_chunk<DIR>(B, p, B.pos + lvl, S, cur, end, M, Cs, c);
-                if (lvl != quiet) nd32 += __popc(bal);
-                if (lvl == k - 1) {
-                    mt32 += __popc(bal);
-                    if (bal) {
-                        // hash prefix sum_{t < lvl} g(mu_t, M_t), only when this chunk has matches
-                        unsigned long long ps = 0;
-                        for (int t = lane; t < lvl; t += 32) ps += gterm(tab[t].pv, M[t]);
-                        ps = warp_sum(ps);
-                        if ((bal >> lane) & 1u) {
-                            hs += fmix64(ps + gterm(p.pv, c));
-                            if (J.mbuf) emit_match(J, M, lvl, c);
-                        }
-                    }
-                    bal = 0;
-                }
-                __syncwarp();
-                if (lane == 0) { L.cur = min(cur + 32, end); L.mask = bal; L.cbase = cur; }
-                __syncwarp();
+                const PosV p = load_pos(B.pos + lvl);
+                scan(lvl, p, csr_list<DIR>(B, p, L, M), cur, end);
                 continue;
             }
             // descend into the lowest pending survivor
@@ -2868,7 +3183,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
             // when it is resumed: they are taken back here.
             for (int l = d0; l <= lvl; ++l) {
                 const LvCsr L = lv[l];
-                const PosV p = csr_pos(tab[l]);
+                const PosV p = load_pos(B.pos + l);
                 const Cand S = csr_list<DIR>(B, p, L, M);
                 const int cb = L.mask ? L.cbase + __ffs(L.mask) - 1 : L.cur;
                 int beg, end;
@@ -3614,8 +3929,14 @@ cudaError_t launch_split_coop(const JobDesc *jobs, long long f0, int32_t *buf0, 
                               long long target, int max_levels, long long *wtot, long long wtot_cap,
                               unsigned *bar, long long *result, int *status, int count_ctr, int directed,
                               int blocks_per_sm, uint32_t *masks, long long mask_total, int ordered,
-                              long long *trace, cudaStream_t st) {
+                              const SplitAsync &async, long long *trace, cudaStream_t st) {
     SplitCtl S;
+    S.narrow = ordered ? 0 : async.narrow;
+    unsigned long long *aw = static_cast<unsigned long long *>(async.ctl);   // one line each, zeroed
+    S.qhead = aw; S.qtail = aw + 16; S.pend = reinterpret_cast<long long *>(aw + 32); S.top = aw + 48;
+    S.nleft = aw + 64; S.stop = reinterpret_cast<int *>(aw + 80);
+    S.qentry = async.entries; S.qcap = async.qcap; S.epoch = async.epoch;
+    S.left = async.left;
     S.trace = ordered ? nullptr : trace;
     S.buf0 = buf0; S.buf1 = buf1; S.cap_ints = cap_ints; S.target = target; S.max_levels = max_levels;
     S.wtot = wtot; S.bar = bar; S.result = result; S.status = status; S.count_ctr = count_ctr;
