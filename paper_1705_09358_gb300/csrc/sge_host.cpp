@@ -43,6 +43,7 @@ constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device 
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
 constexpr int POOL_CELLS = 1 << 15;
 constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
+constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
 constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
 constexpr int BLOCK_FIXPOINT_MAX_N = 16384;      // auto domain mode: in-block fixpoint for targets up to this
@@ -293,6 +294,13 @@ struct TargetRec {
     DevBuf ldm;            // small undirected targets: label-degree masks
     DevBuf runs;           // label-grouped rows: a LabelRuns record, then its arrays
     int maxrun = 0;        // longest label run
+    std::vector<int32_t> labcnt_h;   // host copy of the vertices per distinct label, beside labs_h
+    // most vertices a domain of this label can hold
+    long long label_count(int32_t lab) const {
+        if (labcnt_h.empty()) return n;
+        const auto it = std::lower_bound(labs_h.begin(), labs_h.end(), lab);
+        return it != labs_h.end() && *it == lab ? labcnt_h[(size_t)(it - labs_h.begin())] : 0;
+    }
     TargetView view() const {
         TargetView v;
         v.n = n;
@@ -992,6 +1000,10 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         // below, whose sweeps spread one job's candidates over the whole device
         // (on small targets the blocks scan domains word by word; large targets' domains are
         // mostly empty words, so there the blocks walk candidate lists, built first, below)
+        // (SGE_DOMAIN_WORDS=1 forces the word sweeps, which otherwise serve only lists beyond CAND_MAX)
+        static const bool force_words = std::getenv("SGE_DOMAIN_WORDS") != nullptr &&
+                                        std::getenv("SGE_DOMAIN_WORDS")[0] == '1';
+        int coop_status = 0;
         int nrids = 0;
         bool small_targets = true;
         for (int q : fjobs) {
@@ -1001,7 +1013,39 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         const bool block_fixpoint = any_rids && small_targets &&
                                     (o.domain_fixpoint == SGE_DOMAIN_BLOCKS ||
                                      (o.domain_fixpoint == SGE_DOMAIN_AUTO && nrids >= ctx->sms / 2));
-        if (block_fixpoint) {
+        // few pairs: the whole device sweeps them in one cooperative launch, if the slots that its
+        // candidates can need (a domain holds vertices of one label) fit
+        bool coop = any_rids && !block_fixpoint && o.domain_fixpoint == SGE_DOMAIN_AUTO && nrids == nf &&
+                    !force_words && nverts <= DOMAIN_COOP_VERTS;
+        long long slots = 0, arcs = 0;
+        std::vector<int> edge_off;
+        int longest = 0;
+        for (int x = 0; x < nf && coop; ++x) {
+            const Job &J = jobs[fjobs[x]];
+            edge_off.push_back((int)arcs);
+            longest = std::max(longest, J.t->cached.runs ? J.t->maxrun : J.t->maxdeg);
+            for (int v = 0; v < J.p->k; ++v) {
+                slots += J.t->label_count(J.p->lab[(size_t)v]);
+                arcs += J.p->odeg[(size_t)v] + (directed ? J.p->ideg[(size_t)v] : 0);
+            }
+            coop = slots <= COOP_CANDIDATES;
+        }
+        if (coop) {
+            CK(W.vchg.ensure(domain_coop_bytes(nverts, arcs)), "alloc domain flags");
+            CK(W.cand.ensure((size_t)std::max(slots, 1ll) * 3 * 4), "alloc candidate lists");
+            CK(upload(W.deoff, edge_off, st), "upload edge offsets");
+            coop = launch_domain_coop(W.fjobs.as<JobDesc>(), W.vert_off.as<long long>(), W.deoff.as<int>(), nf, nverts,
+                                      arcs, any_fc ? 1 : 0, longest, W.vchg.p, W.cand.as<int>(), slots, st) == cudaSuccess;
+            if (coop) ++launches;
+            else (void)cudaGetLastError();   // refused: the paths below
+        }
+        if (coop) {
+            CK(cudaMemcpyAsync(&coop_status, W.vchg.p, sizeof(int), cudaMemcpyDeviceToHost, st), "read domain status");
+            if (trace_on()) {
+                CK(cudaStreamSynchronize(st), "fixpoint sync");
+                std::fprintf(stderr, "[sge] domain fixpoint by the whole device: %d jobs at %.3f ms\n", nf, now_ms() - t_start);
+            }
+        } else if (block_fixpoint) {
             CK(launch_domain_fixpoint(W.fjobs.as<JobDesc>(), nf, nullptr, nullptr, nullptr, nullptr,
                                       W.flag.as<int>() + 8, st),
                "domain fixpoint");
@@ -1045,9 +1089,6 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                     ncand += csize[(size_t)g];
                 }
             }
-            // SGE_DOMAIN_WORDS=1 forces the word sweeps (they otherwise serve only lists beyond CAND_MAX)
-            static const bool force_words = std::getenv("SGE_DOMAIN_WORDS") != nullptr &&
-                                            std::getenv("SGE_DOMAIN_WORDS")[0] == '1';
             const bool cand_mode = !force_words && ncand > 0 && ncand <= CAND_MAX;
             if (cand_mode) {
                 std::vector<int> tj, tv, to;
@@ -1180,6 +1221,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         if (sizes.size() < (size_t)nverts) sizes.resize((size_t)nverts);
         CK(cudaMemcpyAsync(sizes.data(), W.sizes.p, (size_t)nverts * 8, cudaMemcpyDeviceToHost, st), "read sizes");
         CK(cudaStreamSynchronize(st), "sizes sync");
+        if (coop_status != 0) return fail(ctx, SGE_ERR_CUDA, "device domain fixpoint failed");
         parallel_for(nf, [&](int x0, int x1) {
             for (int x = x0; x < x1; ++x) {
                 Job &J = jobs[fjobs[x]];
@@ -2309,6 +2351,8 @@ sge_status sge_load_target(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *sr
         if ((long long)n * L <= LABEL_TABLE_MAX) {
             T->nlab = (int)L;
             T->labs_h = labs;
+            T->labcnt_h.assign(labs.size(), 0);
+            for (int v = 0; v < n; ++v) ++T->labcnt_h[(size_t)lidx[(size_t)v]];
             T->ltab_off = (int)((L + 3) & ~3LL);
             CK(T->ltab.ensure(((size_t)T->ltab_off + (size_t)n * L) * 4), "alloc label table");
             CK(cudaMemcpyAsync(T->ltab.p, labs.data(), (size_t)L * 4, cudaMemcpyHostToDevice, st), "upload labels");

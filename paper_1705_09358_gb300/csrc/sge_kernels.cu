@@ -596,6 +596,9 @@ __global__ void __launch_bounds__(KMAX) k_label_index(const JobDesc *jobs) {
 // Initial domain of pattern vertex v on a target with label buckets: the prefix of
 // lab(v)'s bucket with degree at least v's (descending order), then, for RI-DS, the
 // label-degree support test of k_domain_init; bits set with atomicOr into the zeroed filter.
+// BUCKET_PARTS warps share a prefix (a frequent label's holds a quarter of the target, and one
+// warp walking it through the dependent table look-ups set the launch's length).
+constexpr int BUCKET_PARTS = 16;
 __global__ void __launch_bounds__(BLOCK) k_domain_init_buckets(const JobDesc *jobs, const long long *vert_off,
                                                                int njobs, long long nverts) {
     const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(BLOCK) k_domain_init_buckets(const JobDesc *jo
     }
     const bool nbcheck = (J.flags & JOB_RIDS) && !(J.flags & JOB_ELAB) && J.t.nbmax != nullptr && J.plidx != nullptr;
     uint64_t *Fv = J.filt + (size_t)v * J.t.dw;
-    for (int x = b0 + lane; x < e; x += 32) {
+    for (int x = b0 + blockIdx.y * 32 + lane; x < e; x += 32 * BUCKET_PARTS) {
         const int t = __ldg(J.t.lbuck + x);
         bool ok = true;
         if (nbcheck) {
@@ -769,39 +772,87 @@ __global__ void __launch_bounds__(BLOCK) k_domain_init(const JobDesc *jobs, cons
     }
 }
 
-// Arc consistency of one candidate (Section 4): does target vertex t keep,
-// for every pattern edge at v, a compatible target edge into the other
-// endpoint's domain?
+// Where a target vertex t may find support for a pattern edge into vertex u: its row (out- or
+// in-), or, on a target with label runs, the run of u's label in it.
+struct AcList {
+    const int32_t *ids;   // entry f is ids[f << shift]
+    const int32_t *lab;   // edge labels, one per entry
+    int len, shift;
+};
+
+__device__ __forceinline__ AcList ac_list(const JobDesc &J, int u, int t, bool in) {
+    AcList A;
+    const LabelRuns *R = J.t.runs;
+    if (R != nullptr && J.plidx != nullptr) {
+        const int li = J.plidx[u];
+        A.ids = nullptr; A.lab = nullptr; A.len = 0; A.shift = 1;
+        if (li < 0) return A;   // no vertex carries u's label
+        const int32_t *r = (in ? R->irun : R->run) + (size_t)t * R->stride + li;
+        const int b = __ldg(r);
+        A.len = __ldg(r + 1) - b;
+        A.ids = reinterpret_cast<const int32_t *>((in ? R->icol : R->col) + b);
+        A.lab = (in ? R->ielab : R->elab) + b;
+    } else {
+        const int32_t *rp = (in ? J.t.irowptr : J.t.rowptr) + t;
+        const int b = __ldg(rp);
+        A.len = __ldg(rp + 1) - b;
+        A.ids = (in ? J.t.icol : J.t.col) + b;
+        A.lab = (in ? J.t.ielab : J.t.elab) + b;
+        A.shift = 0;
+    }
+    return A;
+}
+
+// Is one of the first n entries of A (with edge label bl when `chk`) in the domain Du?  Four entries'
+// ids, then their domain words, are in flight together: the scan is a chain of such pairs of loads.
+__device__ __forceinline__ bool ac_scan(const AcList &A, int n, const uint64_t *Du, bool chk, int bl) {
+    for (int f0 = 0; f0 < n; f0 += 4) {
+        int y[4];
+        uint64_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[i] = f0 + i < n ? __ldg(A.ids + ((size_t)(f0 + i) << A.shift)) : -1;
+        if (chk) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (y[i] >= 0 && __ldg(A.lab + f0 + i) != bl) y[i] = -1;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = y[i] >= 0 ? Du[y[i] >> 6] : 0ull;
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) any = any || ((w[i] >> (y[i] & 63)) & 1ull);
+        if (any) return true;
+    }
+    return false;
+}
+
+// Arc consistency of one candidate (Section 4): does target vertex t keep, for every pattern
+// edge at v, a compatible target edge into the other endpoint's domain?
 __device__ __forceinline__ bool ac_supported(const JobDesc &J, int v, int t, bool DIR, bool chk) {
     const int dw = J.t.dw;
-    for (int e = J.p.rowptr[v]; e < J.p.rowptr[v + 1]; ++e) {
-        const int uu = J.p.col[e], bl = chk ? J.p.elab[e] : 0;
-        const uint64_t *Du = J.filt + (size_t)uu * dw;
-        bool found = false;
-        for (int f = __ldg(J.t.rowptr + t), fe = __ldg(J.t.rowptr + t + 1); f < fe; ++f) {
-            const int y = __ldg(J.t.col + f);
-            if ((!chk || __ldg(J.t.elab + f) == bl) && ((Du[y >> 6] >> (y & 63)) & 1ull)) { found = true; break; }
-        }
-        if (!found) return false;
-    }
-    if (DIR) {
-        for (int e = J.p.irowptr[v]; e < J.p.irowptr[v + 1]; ++e) {
-            const int uu = J.p.icol[e], bl = chk ? J.p.ielab[e] : 0;
-            const uint64_t *Du = J.filt + (size_t)uu * dw;
-            bool found = false;
-            for (int f = __ldg(J.t.irowptr + t), fe = __ldg(J.t.irowptr + t + 1); f < fe; ++f) {
-                const int y = __ldg(J.t.icol + f);
-                if ((!chk || __ldg(J.t.ielab + f) == bl) && ((Du[y >> 6] >> (y & 63)) & 1ull)) { found = true; break; }
-            }
-            if (!found) return false;
+    for (int pass = 0; pass < (DIR ? 2 : 1); ++pass) {
+        const int32_t *prow = pass ? J.p.irowptr : J.p.rowptr;
+        const int32_t *pcol = pass ? J.p.icol : J.p.col;
+        const int32_t *pel = pass ? J.p.ielab : J.p.elab;
+        for (int e = prow[v], ee = prow[v + 1]; e < ee; ++e) {
+            const int u = pcol[e];
+            const AcList A = ac_list(J, u, t, pass != 0);
+            if (!ac_scan(A, A.len, J.filt + (size_t)u * dw, chk, chk ? pel[e] : 0)) return false;
         }
     }
     return true;
 }
 
-// Warp-collective form of ac_supported for a candidate with a long row: for each
-// pattern edge the 32 lanes stride t's row and a ballot says whether any of them
-// found a compatible neighbour in the other endpoint's domain.
+// A list longer than AC_WARP_LIST is searched by the whole warp (ac_supported_warp) -- unless the
+// domains at the other ends of v's pattern edges are dense (each at least 1/AC_DENSE of the
+// target), where a scan finds support within a few entries: then the candidate's own lane scans
+// AC_LANE_SCAN entries first.  Lists longer than AC_WARP_DIRECT always go to the warp.
+constexpr int AC_WARP_LIST = 48;
+constexpr int AC_LANE_SCAN = 32;
+constexpr int AC_WARP_DIRECT = 512;
+
+// Warp-collective: are the pattern edges at v with long lists supported at t?  For each the 32
+// lanes stride the list and a ballot says whether any of them found support.
 __device__ __forceinline__ bool ac_supported_warp(const JobDesc &J, int v, int t, bool DIR, bool chk) {
     const int lane = threadIdx.x & 31;
     const int dw = J.t.dw;
@@ -809,20 +860,21 @@ __device__ __forceinline__ bool ac_supported_warp(const JobDesc &J, int v, int t
         const int32_t *prow = pass ? J.p.irowptr : J.p.rowptr;
         const int32_t *pcol = pass ? J.p.icol : J.p.col;
         const int32_t *pel = pass ? J.p.ielab : J.p.elab;
-        const int32_t *trow = pass ? J.t.irowptr : J.t.rowptr;
-        const int32_t *tcol = pass ? J.t.icol : J.t.col;
-        const int32_t *tel = pass ? J.t.ielab : J.t.elab;
-        const int fb = __ldg(trow + t), fe = __ldg(trow + t + 1);
-        for (int e = prow[v]; e < prow[v + 1]; ++e) {
-            const int uu = pcol[e], bl = chk ? pel[e] : 0;
-            const uint64_t *Du = J.filt + (size_t)uu * dw;
+        for (int e = prow[v], ee = prow[v + 1]; e < ee; ++e) {
+            const int u = pcol[e], bl = chk ? pel[e] : 0;
+            const AcList A = ac_list(J, u, t, pass != 0);
+            if (A.len <= AC_WARP_LIST) continue;   // (the candidate's lane has found its support)
+            const uint64_t *Du = J.filt + (size_t)u * dw;
             bool found = false;
-            for (int f0 = fb; f0 < fe && !found; f0 += 32) {
-                const int f = f0 + lane;
+            for (int f0 = 0; f0 < A.len && !found; f0 += 64) {
                 bool ok = false;
-                if (f < fe) {
-                    const int y = __ldg(tcol + f);
-                    ok = (!chk || __ldg(tel + f) == bl) && ((Du[y >> 6] >> (y & 63)) & 1ull);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int f = f0 + 32 * i + lane;
+                    if (f < A.len) {
+                        const int y = __ldg(A.ids + ((size_t)f << A.shift));
+                        ok = ok || ((!chk || __ldg(A.lab + f) == bl) && ((Du[y >> 6] >> (y & 63)) & 1ull));
+                    }
                 }
                 found = __any_sync(FULL, ok);
             }
@@ -832,63 +884,30 @@ __device__ __forceinline__ bool ac_supported_warp(const JobDesc &J, int v, int t
     return true;
 }
 
-// A candidate whose row (out- plus in-row) is longer than AC_WARP_ROW is searched
-// by the whole warp (ac_supported_warp) -- unless the domains at the other ends of
-// its pattern edges are dense (each at least 1/AC_DENSE of the target), where a
-// row scan finds support within a few entries: then its own lane scans at most
-// AC_LANE_SCAN entries per pattern edge first, and only an edge left open sends
-// it to the warp.  Rows longer than AC_WARP_ROW_DIRECT always go to the warp.
-constexpr int AC_WARP_ROW = 48;
-constexpr int AC_LANE_SCAN = 32;
-constexpr int AC_WARP_ROW_DIRECT = 512;
-
-// ac_supported with each row scan cut after `bound` entries: returns false if
-// some pattern edge has no support (its whole row scanned), true if every edge
-// found one, and sets `open` (result then true) when no edge failed but some
-// scan stopped at the bound.
-__device__ __forceinline__ bool ac_supported_bounded(const JobDesc &J, int v, int t, bool DIR, bool chk, int bound, bool &open) {
+// Lane-local part of the arc-consistency test of candidate t of D(v): whether to drop it, or
+// (`heavy`) to have the warp look at its long lists.
+__device__ __forceinline__ bool ac_lane_check(const JobDesc &J, int v, int t, bool DIR, bool chk, bool dense,
+                                              bool &heavy) {
     const int dw = J.t.dw;
-    open = false;
+    heavy = false;
     for (int pass = 0; pass < (DIR ? 2 : 1); ++pass) {
         const int32_t *prow = pass ? J.p.irowptr : J.p.rowptr;
         const int32_t *pcol = pass ? J.p.icol : J.p.col;
         const int32_t *pel = pass ? J.p.ielab : J.p.elab;
-        const int32_t *trow = pass ? J.t.irowptr : J.t.rowptr;
-        const int32_t *tcol = pass ? J.t.icol : J.t.col;
-        const int32_t *tel = pass ? J.t.ielab : J.t.elab;
-        const int f0 = __ldg(trow + t), fe = __ldg(trow + t + 1);
-        const int fb = min(fe, f0 + bound);
-        for (int e = prow[v]; e < prow[v + 1]; ++e) {
-            const int uu = pcol[e], bl = chk ? pel[e] : 0;
-            const uint64_t *Du = J.filt + (size_t)uu * dw;
-            bool found = false;
-            for (int f = f0; f < fb; ++f) {
-                const int y = __ldg(tcol + f);
-                if ((!chk || __ldg(tel + f) == bl) && ((Du[y >> 6] >> (y & 63)) & 1ull)) { found = true; break; }
+        for (int e = prow[v], ee = prow[v + 1]; e < ee; ++e) {
+            const int u = pcol[e];
+            const AcList A = ac_list(J, u, t, pass != 0);
+            const bool all = A.len <= AC_WARP_LIST;
+            const int n = all ? A.len : dense && A.len <= AC_WARP_DIRECT ? AC_LANE_SCAN : 0;
+            if (ac_scan(A, n, J.filt + (size_t)u * dw, chk, chk ? pel[e] : 0)) continue;
+            if (all) {
+                heavy = false;
+                return true;
             }
-            if (!found) {
-                if (fb == fe) return false;
-                open = true;
-            }
+            heavy = true;
         }
     }
-    return true;
-}
-
-// Lane-local part of the arc-consistency test of candidate t of D(v) with a row of
-// `len` entries: whether to drop it, or (`heavy`) to leave it to the warp.
-__device__ __forceinline__ bool ac_lane_check(const JobDesc &J, int v, int t, bool DIR, bool chk, int len,
-                                              bool dense, bool &heavy) {
-    heavy = false;
-    if (len <= AC_WARP_ROW) return !ac_supported(J, v, t, DIR, chk);
-    if (!dense || len > AC_WARP_ROW_DIRECT) {
-        heavy = true;
-        return false;
-    }
-    bool open = false;
-    const bool sup = ac_supported_bounded(J, v, t, DIR, chk, AC_LANE_SCAN, open);
-    heavy = open;
-    return !sup;
+    return false;
 }
 
 // The same sweep over explicit candidate lists: one lane per listed candidate of
@@ -920,10 +939,7 @@ __global__ void __launch_bounds__(BLOCK, 1) k_domain_ac_cand(const JobDesc *jobs
         if (!(*wp & (1ull << (t & 63)))) {
             *slot = -1;                                  // removed by forward checking
         } else {
-            const bool DIR = (J.flags & JOB_DIRECTED) != 0;
-            const int len = __ldg(J.t.rowptr + t + 1) - __ldg(J.t.rowptr + t) +
-                            (DIR ? __ldg(J.t.irowptr + t + 1) - __ldg(J.t.irowptr + t) : 0);
-            drop = ac_lane_check(J, v, t, DIR, (J.flags & JOB_ELAB) != 0, len, dense_v, heavy);
+            drop = ac_lane_check(J, v, t, (J.flags & JOB_DIRECTED) != 0, (J.flags & JOB_ELAB) != 0, dense_v, heavy);
         }
     }
     unsigned hv = __ballot_sync(FULL, heavy);
@@ -1286,9 +1302,7 @@ __global__ void __launch_bounds__(FIXPOINT_BIG_BLOCK, 1) k_domain_fixpoint(const
                             if (!((J.filt[(size_t)v * dw + (t >> 6)] >> (t & 63)) & 1ull)) {
                                 *slot = -1;                      // removed by forward checking
                             } else {
-                                const int len = __ldg(J.t.rowptr + t + 1) - __ldg(J.t.rowptr + t) +
-                                                (DIR ? __ldg(J.t.irowptr + t + 1) - __ldg(J.t.irowptr + t) : 0);
-                                drop = ac_lane_check(J, v, t, DIR, chk, len, dns[v] != 0, heavy);
+                                drop = ac_lane_check(J, v, t, DIR, chk, dns[v] != 0, heavy);
                             }
                         }
                         unsigned hv = __ballot_sync(FULL, heavy);
@@ -1372,6 +1386,359 @@ __global__ void __launch_bounds__(FIXPOINT_BIG_BLOCK, 1) k_domain_fixpoint(const
             __syncthreads();
         }
         __syncthreads();   // the shared arrays are reused by the next job
+    }
+}
+
+__device__ __forceinline__ void grid_barrier(unsigned *count, unsigned *gen, int *status);
+
+// The same joint fixpoint for a few pairs, by the whole device in one cooperative launch: a sweep
+// (or forward-checking round) ends at a grid barrier instead of the host reading back which domains
+// shrank and launching the next.  Every candidate has a slot, found once at the start; a sweep goes
+// over all slots and tests, for each, the pattern edges whose other endpoint shrank in the last one;
+// lists too long for a lane are gathered and searched by a warp each.  When a
+// sweep removes nothing, one block per pair runs a forward-checking round; when that removes
+// nothing either, both fixpoints hold.  Flags rotate over three generations (read, being set,
+// being cleared), so a sweep costs one barrier.  Bound by the barrier (3 us) and the dependent loads of one candidate's
+// test: all domain work of 10 deep patterns (9 sweeps, 2 rounds) 0.86 ms under the host loop ->
+// 0.40 here, of 24 directed ones (11 sweeps) 0.65 -> 0.25; of 64 network queries, a block per pair
+// there, 2.4 -> 1.4 ms.  It takes calls that the block-per-pair form is not meant for (few pairs),
+// and on large targets all of up to DOMAIN_COOP_VERTS pattern vertices.
+// What a sweep reads of a pattern vertex and of its edges, gathered once: a candidate's test is then
+// slot, these, list bounds, ids, domain words -- six dependent loads where the job and
+// pattern records took twice that for every edge.
+struct __align__(16) CoopEdge {
+    const uint64_t *Du;      // the other endpoint's domain
+    int li, bl;              // its label index (plain rows: 0; absent label: -1), the edge's label
+    int in, u;               // out- or in-rows; the other endpoint (global vertex)
+    int pad[2];
+};
+struct __align__(16) CoopVert {
+    const int32_t *at[2];    // list bounds at at[in][t * stride + li], .. + 1: run tables or row offsets
+    const int32_t *ids[2];   // list entries, every (1 << shift)-th word
+    const int32_t *lab[2];
+    uint64_t *Dv;
+    int e0, e1;              // its edges
+    int job, stride;
+    short shift, chk, dense, pad;
+};
+
+struct DomainCoop {
+    const JobDesc *jobs;
+    const long long *vert_off;
+    int njobs, nverts;
+    const int *edge_off;    // [njobs] first edge of a job
+    CoopVert *vert;         // [nverts]
+    CoopEdge *edge;
+    int *size;              // [nverts] as found at the start
+    unsigned char *chg;     // [3][nverts] domains that shrank; zeroed
+    unsigned char *done;    // [nverts] forward checking: singleton propagated; zeroed
+    int *any;               // [3] something was removed; zeroed
+    int *nheavy;            // [3] candidates whose long lists are still to be searched; zeroed
+    int *heavy;             // [cap] their slots
+    int2 *slot;             // [cap] candidate (-1: removed) and its global vertex
+    long long cap;
+    unsigned *bar;          // [2], zeroed
+    int *status;            // zeroed; -2: more candidates than `cap`
+    int any_fc, any_long;   // some pair checks forward; some list may be longer than AC_WARP_LIST
+};
+
+constexpr int DOMAIN_COOP_BLOCKS = 4;     // most blocks per SM of that launch
+
+__device__ __forceinline__ AcList coop_list(const CoopVert &V, const CoopEdge &E, int t) {
+    AcList A;
+    A.shift = V.shift;
+    A.len = 0;
+    A.ids = A.lab = nullptr;
+    if (E.li < 0) return A;
+    const int32_t *r = V.at[E.in] + (size_t)t * V.stride + E.li;
+    const int b = __ldg(r);
+    A.len = __ldg(r + 1) - b;
+    A.ids = V.ids[E.in] + ((size_t)b << A.shift);
+    A.lab = V.lab[E.in] + b;
+    return A;
+}
+
+// The edges e0 + sub, e0 + sub + G, .. of V whose other endpoint shrank (a bit of `chg`; all in the first
+// sweep): is candidate t without support for one of them, or (`heavy`) has one too long a list for a lane?
+__device__ __forceinline__ bool coop_lane_check(const DomainCoop &D, const CoopVert &V, int t, int sub, int G,
+                                                const unsigned *chg, bool &heavy) {
+    heavy = false;
+    for (int e = V.e0 + sub; e < V.e1; e += G) {
+        const CoopEdge &E = D.edge[e];
+        if (!((chg[E.u >> 5] >> (E.u & 31)) & 1u)) continue;
+        const AcList A = coop_list(V, E, t);
+        const bool all = A.len <= AC_WARP_LIST;
+        const int n = all ? A.len : V.dense && A.len <= AC_WARP_DIRECT ? AC_LANE_SCAN : 0;
+        if (ac_scan(A, n, E.Du, V.chk != 0, E.bl)) continue;
+        if (all) return true;
+        heavy = true;
+    }
+    return false;
+}
+
+// Warp-collective: its long lists.
+__device__ __forceinline__ bool coop_supported_warp(const DomainCoop &D, const CoopVert &V, int t, const unsigned *chg) {
+    const int lane = threadIdx.x & 31;
+    for (int e = V.e0; e < V.e1; ++e) {
+        const CoopEdge &E = D.edge[e];
+        if (!((chg[E.u >> 5] >> (E.u & 31)) & 1u)) continue;
+        const AcList A = coop_list(V, E, t);
+        if (A.len <= AC_WARP_LIST) continue;   // (the candidate's lane has found its support)
+        bool found = false;
+        for (int f0 = 0; f0 < A.len && !found; f0 += 64) {
+            bool ok = false;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int f = f0 + 32 * i + lane;
+                if (f < A.len) {
+                    const int y = __ldg(A.ids + ((size_t)f << A.shift));
+                    ok = ok || ((!V.chk || __ldg(A.lab + f) == E.bl) && ((E.Du[y >> 6] >> (y & 63)) & 1ull));
+                }
+            }
+            found = __any_sync(FULL, ok);
+        }
+        if (!found) return false;
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(BLOCK, 4) k_domain_coop(DomainCoop D) {
+    extern __shared__ int start[];   // [nverts + 1] first slot of each global vertex
+    __shared__ int wsum[32];
+    __shared__ int newu[KMAX], elem[KMAX], nnew;
+    __shared__ unsigned was[DOMAIN_COOP_VERTS / 32], is[DOMAIN_COOP_VERTS / 32];   // shrank: last step, now (this block)
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int words = (D.nverts + 31) / 32;
+    // sizes and records
+    for (long long g = w; g < D.nverts; g += nw) {
+        const int j = find_job(D.vert_off, D.njobs, g);
+        const JobDesc &J = D.jobs[j];
+        const int v = (int)(g - D.vert_off[j]);
+        const bool DIR = (J.flags & JOB_DIRECTED) != 0, chk = (J.flags & JOB_ELAB) != 0;
+        const LabelRuns *R = J.t.runs != nullptr && J.plidx != nullptr ? J.t.runs : nullptr;
+        uint64_t *row = J.filt + (size_t)v * J.t.dw;
+        unsigned long long c = 0;
+        for (int q = lane; q < J.t.dw; q += 32) c += __popcll(row[q]);
+        c = warp_sum(c);
+        const int no = J.p.rowptr[v + 1] - J.p.rowptr[v], ni = DIR ? J.p.irowptr[v + 1] - J.p.irowptr[v] : 0;
+        const int e0 = D.edge_off[j] + J.p.rowptr[v] + (DIR ? J.p.irowptr[v] : 0);
+        if (lane == 0) {
+            D.size[g] = (int)c;
+            CoopVert V;
+            V.at[0] = R ? R->run : J.t.rowptr;
+            V.at[1] = R ? R->irun : J.t.irowptr;
+            V.ids[0] = R ? reinterpret_cast<const int32_t *>(R->col) : J.t.col;
+            V.ids[1] = R ? reinterpret_cast<const int32_t *>(R->icol) : J.t.icol;
+            V.lab[0] = R ? R->elab : J.t.elab;
+            V.lab[1] = R ? R->ielab : J.t.ielab;
+            V.Dv = row;
+            V.e0 = e0;
+            V.e1 = e0 + no + ni;
+            V.job = j;
+            V.stride = R ? R->stride : 1;
+            V.shift = R ? 1 : 0;
+            V.chk = chk;
+            V.dense = 0;
+            V.pad = 0;
+            D.vert[g] = V;
+        }
+        for (int i = lane; i < no + ni; i += 32) {
+            const bool in = i >= no;
+            const int e = in ? J.p.irowptr[v] + i - no : J.p.rowptr[v] + i;
+            const int u = in ? J.p.icol[e] : J.p.col[e];
+            CoopEdge E;
+            E.Du = J.filt + (size_t)u * J.t.dw;
+            E.li = R ? J.plidx[u] : 0;
+            E.bl = chk ? (in ? J.p.ielab[e] : J.p.elab[e]) : 0;
+            E.in = in;
+            E.u = (int)(g - v) + u;
+            E.pad[0] = E.pad[1] = 0;
+            D.edge[e0 + i] = E;
+        }
+    }
+    grid_barrier(D.bar, D.bar + 1, D.status);
+    // slot offsets, by every block for itself
+    int total = 0;
+    bool over = false;
+    for (int g0 = 0; g0 < D.nverts; g0 += BLOCK) {
+        const int g = g0 + threadIdx.x;
+        const int c = g < D.nverts ? __ldcg(D.size + g) : 0;
+        int sum;
+        const int ex = block_scan_int(c, wsum, sum);
+        if (g < D.nverts) start[g] = total + ex;
+        over = over || (long long)total + sum > D.cap;
+        total += over ? 0 : sum;
+    }
+    if (threadIdx.x == 0) start[D.nverts] = total;
+    __syncthreads();
+    if (over) {   // (the same for every block; the caller's bound rules it out)
+        if (blockIdx.x == 0 && threadIdx.x == 0) set_status(D.status, -2);
+        return;
+    }
+    // slots, and which vertices' neighbours are dense
+    for (long long g = w; g < D.nverts; g += nw) {
+        const CoopVert &V = D.vert[g];
+        const TargetView &T = D.jobs[V.job].t;
+        int at = start[g];
+        for (int q0 = 0; q0 < T.dw; q0 += 32) {
+            const int q = q0 + lane;
+            uint64_t x = q < T.dw ? V.Dv[q] : 0;
+            const int c = __popcll(x);
+            if (__reduce_or_sync(FULL, (unsigned)c) == 0) continue;
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            int o = at + incl - c;
+            for (; x; x &= x - 1, ++o) D.slot[o] = make_int2(q * 64 + __ffsll((long long)x) - 1, (int)g);
+            at += __shfl_sync(FULL, incl, 31);
+        }
+        bool d = true;
+        for (int e = V.e0 + lane; e < V.e1; e += 32) d = d && (long long)__ldcg(D.size + D.edge[e].u) * AC_DENSE >= T.n;
+        d = __all_sync(FULL, d);
+        if (lane == 0) D.vert[g].dense = d;
+    }
+    grid_barrier(D.bar, D.bar + 1, D.status);
+    // few candidates: several lanes each, sharing its vertex's edges
+    int G = 1;
+    while (G < 32 && total <= nw * (32 / (2 * G))) G *= 2;
+    const int per = 32 / G, sub = lane & (G - 1);
+    bool fc = false, first = true;   // this step is a forward-checking round; ... the first sweep
+    for (int s = 0;; s = s == 2 ? 0 : s + 1) {
+        const int s1 = s == 2 ? 0 : s + 1, s2 = s1 == 2 ? 0 : s1 + 1;
+        const unsigned char *cur = D.chg + (size_t)s * D.nverts;
+        unsigned char *next = D.chg + (size_t)s1 * D.nverts;
+        // which domains shrank in the last step, as bits
+        __syncthreads();
+        for (int q = wid; q < words; q += WARPS_PER_BLOCK) {
+            const int g = 32 * q + lane;
+            const unsigned bits = __ballot_sync(FULL, g < D.nverts && (first || __ldcg(cur + g)));
+            if (lane == 0) {
+                was[q] = bits;
+                is[q] = 0;
+            }
+        }
+        for (long long g = blockIdx.x * (long long)BLOCK + threadIdx.x; g < D.nverts; g += (long long)gridDim.x * BLOCK)
+            D.chg[(size_t)s2 * D.nverts + g] = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) D.any[s2] = D.nheavy[s2] = 0;
+        __syncthreads();
+        if (!fc) {
+            for (long long x0 = w * per; x0 < total; x0 += nw * per) {
+                const long long x = x0 + lane / G;
+                int2 c = make_int2(-1, 0);
+                if (x < total) c = __ldcg(D.slot + x);
+                bool drop = false, heavy = false;
+                const CoopVert &V = D.vert[c.y];
+                if (c.x >= 0) {
+                    if ((__ldcg(V.Dv + (c.x >> 6)) >> (c.x & 63)) & 1ull) drop = coop_lane_check(D, V, c.x, sub, G, was, heavy);
+                    else if (sub == 0) D.slot[x].x = -1;   // (removed by forward checking)
+                }
+                // the group's verdict, at its first lane
+                const unsigned mine = (G == 32 ? FULL : ((1u << G) - 1u)) << (lane & ~(G - 1));
+                const unsigned drops = __ballot_sync(FULL, drop), heavies = __ballot_sync(FULL, heavy);
+                drop = (drops & mine) != 0;
+                heavy = !drop && (heavies & mine) != 0;
+                if (drop && sub == 0) {
+                    atomicAnd((unsigned long long *)(V.Dv + (c.x >> 6)), ~(1ull << (c.x & 63)));
+                    D.slot[x].x = -1;
+                    atomicOr(&is[c.y >> 5], 1u << (c.y & 31));
+                }
+                // long lists are left for the whole device: hubs come in runs of slots, and one
+                // warp searching all of a run's lists set the sweep's length
+                const unsigned hv = __ballot_sync(FULL, heavy && sub == 0);
+                if (hv) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(D.nheavy + s1, __popc(hv));
+                    at = __shfl_sync(FULL, at, 0);
+                    if (heavy && sub == 0) D.heavy[at + __popc(hv & ((1u << lane) - 1u))] = (int)x;
+                }
+            }
+            if (D.any_long) {
+                grid_barrier(D.bar, D.bar + 1, D.status);
+                const int nh = __ldcg(D.nheavy + s1);
+                for (long long i = w; i < nh; i += nw) {
+                    const int x = __ldcg(D.heavy + i);
+                    const int2 c = __ldcg(D.slot + x);
+                    const CoopVert &V = D.vert[c.y];
+                    if (!coop_supported_warp(D, V, c.x, was) && lane == 0) {
+                        atomicAnd((unsigned long long *)(V.Dv + (c.x >> 6)), ~(1ull << (c.x & 63)));
+                        D.slot[x].x = -1;
+                        atomicOr(&is[c.y >> 5], 1u << (c.y & 31));
+                    }
+                    __syncwarp();
+                }
+            }
+        } else {
+            for (int j = blockIdx.x; j < D.njobs; j += gridDim.x) {
+                const JobDesc &J = D.jobs[j];
+                if (!(J.flags & JOB_FC)) continue;
+                const int k = J.k, dw = J.t.dw;
+                const long long g0 = D.vert_off[j];
+                __syncthreads();
+                if (threadIdx.x == 0) nnew = 0;
+                __syncthreads();
+                // new singletons: a vertex's words until a second element shows
+                for (int v = wid; v < k; v += WARPS_PER_BLOCK) {
+                    if (__ldcg(D.done + g0 + v)) continue;
+                    int n = 0, at = -1;
+                    for (int q0 = 0; q0 < dw && n <= 1; q0 += 64) {
+                        uint64_t x[2];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const int q = q0 + 32 * i + lane;
+                            x[i] = q < dw ? __ldcg(J.filt + (size_t)v * dw + q) : 0ull;
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const unsigned bal = __ballot_sync(FULL, x[i] != 0);
+                            if (bal == 0) continue;
+                            const int L = __ffs(bal) - 1;
+                            const uint64_t xl = __shfl_sync(FULL, x[i], L);
+                            n += __popc(bal) > 1 ? 2 : min(2, __popcll(xl));
+                            at = (q0 + 32 * i + L) * 64 + __ffsll((long long)xl) - 1;
+                        }
+                    }
+                    if (lane == 0 && n == 1) {
+                        D.done[g0 + v] = 1;
+                        const int y = atomicAdd(&nnew, 1);
+                        newu[y] = v;
+                        elem[y] = at;
+                    }
+                }
+                __syncthreads();
+                const int nn = nnew;
+                for (int x = threadIdx.x; x < nn * k; x += BLOCK) {
+                    const int u = newu[x / k], v = x % k, t = elem[x / k], g = (int)g0 + v;
+                    if (v == u) continue;
+                    const unsigned long long bit = 1ull << (t & 63);
+                    if (atomicAnd((unsigned long long *)(J.filt + (size_t)v * dw + (t >> 6)), ~bit) & bit)
+                        atomicOr(&is[g >> 5], 1u << (g & 31));
+                }
+            }
+        }
+        // this block's shrunk domains, told once each (every removal telling on its own queued
+        // thousands of updates on the same lines: 55 us of a 62 us sweep)
+        __syncthreads();
+        for (int q = threadIdx.x; q < words; q += BLOCK)
+            for (unsigned m = is[q]; m; m &= m - 1) {
+                next[32 * q + __ffs(m) - 1] = 1;
+                if (__ldcg(D.any + s1) == 0) D.any[s1] = 1;
+            }
+        grid_barrier(D.bar, D.bar + 1, D.status);
+        first = false;
+        const bool any = __ldcg(D.any + s1) != 0;
+        if (__ldcg(D.status) != 0) break;
+        if (!any) {
+            // nothing left to sweep: a forward-checking round, or, after one, the end
+            if (fc || !D.any_fc) break;
+            fc = true;
+        } else {
+            fc = false;
+        }
     }
 }
 
@@ -3827,7 +4194,7 @@ unsigned grid_for(long long warps) {
 cudaError_t launch_domain_init_buckets(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
                                        cudaStream_t st) {
     if (nverts <= 0) return cudaSuccess;
-    k_domain_init_buckets<<<grid_for(nverts), BLOCK, 0, st>>>(jobs, vert_off, njobs, nverts);
+    k_domain_init_buckets<<<dim3(grid_for(nverts), BUCKET_PARTS), BLOCK, 0, st>>>(jobs, vert_off, njobs, nverts);
     return cudaGetLastError();
 }
 
@@ -3896,6 +4263,49 @@ cudaError_t launch_domain_fixpoint(const JobDesc *jobs, int njobs, const long lo
     if (e != cudaSuccess) return e;
     k_domain_fixpoint<<<grid, threads, 0, st>>>(jobs, njobs, vert_off, cstart, csize, cand, next_job);
     return cudaGetLastError();
+}
+
+size_t domain_coop_bytes(long long nverts, long long nedges) {
+    return 128 + (size_t)nverts * (sizeof(CoopVert) + 4 + 3 + 1) + (size_t)nedges * sizeof(CoopEdge) + 64;
+}
+
+cudaError_t launch_domain_coop(const JobDesc *jobs, const long long *vert_off, const int *edge_off, int njobs,
+                               long long nverts, long long nedges, int any_fc, int longest_list, void *scratch,
+                               int *slots, long long cap, cudaStream_t st) {
+    if (nverts <= 0) return cudaSuccess;
+    if (nverts > DOMAIN_COOP_VERTS) return cudaErrorInvalidValue;
+    DomainCoop D;
+    D.jobs = jobs; D.vert_off = vert_off; D.edge_off = edge_off; D.njobs = njobs; D.nverts = (int)nverts;
+    D.any_fc = any_fc;
+    D.any_long = longest_list > AC_WARP_LIST;
+    char *b = static_cast<char *>(scratch);
+    D.status = reinterpret_cast<int *>(b);
+    D.bar = reinterpret_cast<unsigned *>(b) + 1;
+    D.any = reinterpret_cast<int *>(b) + 4;
+    D.nheavy = reinterpret_cast<int *>(b) + 8;
+    b += 128;
+    D.size = reinterpret_cast<int *>(b); b += 4 * nverts;
+    D.chg = reinterpret_cast<unsigned char *>(b); b += 3 * nverts;
+    D.done = reinterpret_cast<unsigned char *>(b); b += nverts;
+    const size_t zeroed = (size_t)(b - static_cast<char *>(scratch));
+    b = static_cast<char *>(scratch) + ((zeroed + 15) & ~(size_t)15);
+    D.vert = reinterpret_cast<CoopVert *>(b); b += nverts * sizeof(CoopVert);
+    D.edge = reinterpret_cast<CoopEdge *>(b);
+    D.slot = reinterpret_cast<int2 *>(slots);
+    D.heavy = slots + 2 * cap;
+    D.cap = cap;
+    cudaError_t e = cudaMemsetAsync(scratch, 0, zeroed, st);
+    if (e != cudaSuccess) return e;
+    const size_t smem = ((size_t)nverts + 1) * sizeof(int);
+    int dev = 0, sms = 0, occ = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_domain_coop, BLOCK, smem);
+    if (e != cudaSuccess) return e;
+    if (occ < 1) return cudaErrorInvalidConfiguration;
+    void *args[] = {(void *)&D};
+    return cudaLaunchCooperativeKernel((void *)k_domain_coop, dim3(sms * std::min(occ, DOMAIN_COOP_BLOCKS)), dim3(BLOCK),
+                                       args, smem, st);
 }
 
 cudaError_t launch_domain_sizes(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
