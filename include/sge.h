@@ -143,7 +143,8 @@ typedef struct {
  * images of pattern vertices 0..k-1.  The buffer is valid only during the
  * call; calls come from the thread that called sge_enumerate.  Return
  * nonzero to stop the enumeration (sge_enumerate then returns
- * SGE_ERR_STOPPED).  Call order is unspecified. */
+ * SGE_ERR_STOPPED).  Matches come in ascending order of the images of pattern
+ * vertices 0, 1, ... */
 typedef int (*sge_match_sink)(void *user, const int32_t *matches, int64_t count, int32_t k);
 
 /* Create a context on CUDA device `device`.  `cuda_stream` is a cudaStream_t

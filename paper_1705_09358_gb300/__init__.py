@@ -463,10 +463,9 @@ class Context:
 
     def enumerate(self, tid, pid, check=True, **opts):
         d, chunks = sge_enumerate(self.h, tid, pid, make_opts(**opts), check=check)
-        rows = np.concatenate(chunks) if chunks else np.zeros((0, 0), np.int32)
-        if rows.shape[0]:
-            rows = rows[np.lexsort(rows.T[::-1])]
-        d["match_list"] = rows
+        # (the library hands them over sorted by the images of pattern vertices 0, 1, ...)
+        d["match_list"] = (chunks[0] if len(chunks) == 1 else np.concatenate(chunks) if chunks
+                           else np.zeros((0, 0), np.int32))
         return d
 
     def serve_submit(self, tid, pid, **opts) -> int:

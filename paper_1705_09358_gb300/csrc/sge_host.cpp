@@ -41,6 +41,7 @@ constexpr int BITSET_MAX_N = 16384;              // adjacency bitset kept for n 
 constexpr int HUB_MIN_DEGREE = 24;               // larger targets: bitset rows for vertices of this degree+
 constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device memory
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
+constexpr long long LIST_FIRST_ROWS = 1 << 16;   // matches a listing call has room for at first
 constexpr int POOL_CELLS = 1 << 15;
 constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
 constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
@@ -411,7 +412,7 @@ struct Workspace {
         ctask;
     DevBuf front[2], counts, offs, scan_tmp, total, splitctl;
     DevBuf pool, pseq, ctl, slab;
-    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft;
+    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft, msort, mout;
     unsigned long long aepoch = 0;   // last launch's mark in aentry (0: the entries are to be cleared)
     std::vector<Job> hjobs;       // the call's pairs, reused (their vectors keep their capacity)
     std::vector<JobDesc> hdesc;   // host job records, reused
@@ -429,7 +430,7 @@ struct Workspace {
 #define SGE_WS_BUFFERS                                                                                             \
     &jobs, &fjobs, &ctr, &filt, &pos, &back, &ulist, &unit_off, &vert_off, &sizes, &task, &flag, &dent, &deoff, &vchg, \
         &cand, &ctask, &front[0], &front[1], &counts, &offs, &scan_tmp, &total, &splitctl, &pool, &pseq, &ctl, &slab, \
-        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart, &aentry, &aleft
+        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart, &aentry, &aleft, &msort, &mout
     // Every buffer of this workspace is used on `st` only: allocate them stream-ordered there.
     void bind(cudaStream_t st) {
         if (bound == st && st != nullptr) return;
@@ -1807,13 +1808,22 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             r.kernel = kernel;
         }
     });
-    if (enumerate && match_rows && nj == 1) {
-        const long long produced = (long long)ctr[4 * (size_t)nj + 0];
-        const long long rows = std::min(produced, match_cap);
-        match_rows->resize((size_t)rows * jobs[0].p->k);
-        if (rows > 0)
-            CK(cudaMemcpy(match_rows->data(), W.mbuf.p, (size_t)rows * jobs[0].p->k * 4, cudaMemcpyDeviceToHost),
+    if (enumerate && match_rows && nj == 1 && status == 0) {
+        const long long rows = (long long)ctr[4 * (size_t)nj + 0];
+        const int k = jobs[0].p->k;
+        match_rows->clear();
+        if (rows > match_cap) return SGE_OK;   // (the caller comes again with room for them)
+        match_rows->resize((size_t)rows * k);
+        if (rows > 0) {
+            int sorting = 0;
+            CK(W.msort.ensure(match_sort_bytes(rows)), "alloc match order");
+            CK(W.mout.ensure((size_t)rows * k * 4), "alloc sorted matches");
+            CK(launch_match_sort(W.mbuf.as<int32_t>(), rows, k, W.msort.p, W.mout.as<int32_t>(), &sorting, st), "sort matches");
+            out[jobs[0].pair].launches += sorting;
+            CK(cudaMemcpyAsync(match_rows->data(), W.mout.p, (size_t)rows * k * 4, cudaMemcpyDeviceToHost, st),
                "read matches");
+            CK(cudaStreamSynchronize(st), "read matches");
+        }
     }
     if (status != 0) {
         const char *why = status == SGE_ERR_BUDGET ? "state budget reached"
@@ -2648,20 +2658,24 @@ sge_status sge_enumerate(sge_ctx *ctx, int32_t target_id, int32_t pattern_id, co
     cudaSetDevice(ctx->device);
     *ctx->cancel_host = 0;
     std::vector<PairReq> reqs{{target_id, pattern_id}};
-    // count first to size the match buffer exactly, then enumerate
-    sge_result first;
-    sge_status rc = run_pairs(ctx, ctx->ws, ctx->stream, reqs, opts, &first, false, nullptr, 0);
-    if (rc != SGE_OK) { *out = first; return rc; }
+    // list into a buffer of a usual size; when there are more matches (the run has counted them
+    // all the same) again into one that holds them
+    std::vector<int32_t> rows;
+    long long cap = LIST_FIRST_ROWS;
+    sge_status rc = run_pairs(ctx, ctx->ws, ctx->stream, reqs, opts, out, true, &rows, cap);
+    if (rc != SGE_OK) return rc;
     int k = 0;
     {
         std::lock_guard<std::mutex> g(ctx->mu);
         k = ctx->patterns.at(pattern_id)->k;
     }
-    if ((long long)first.matches * std::max(k, 1) * 4 > (1ll << 32))
-        return fail(ctx, SGE_ERR_OOM, "match list larger than 4 GiB; use sge_count");
-    std::vector<int32_t> rows;
-    rc = run_pairs(ctx, ctx->ws, ctx->stream, reqs, opts, out, true, &rows, (long long)first.matches);
-    if (rc != SGE_OK) return rc;
+    if ((long long)out->matches > cap) {
+        if ((long long)out->matches * std::max(k, 1) * 4 > (1ll << 32))
+            return fail(ctx, SGE_ERR_OOM, "match list larger than 4 GiB; use sge_count");
+        cap = (long long)out->matches;
+        rc = run_pairs(ctx, ctx->ws, ctx->stream, reqs, opts, out, true, &rows, cap);
+        if (rc != SGE_OK) return rc;
+    }
     const long long n = k > 0 ? (long long)rows.size() / k : 0;
     const long long chunk = 1 << 16;
     for (long long i = 0; i < n; i += chunk) {

@@ -315,6 +315,12 @@ cudaError_t launch_frames_to_rows(const JobDesc *jobs, int32_t *frames, long lon
 cudaError_t launch_build_hubs(const int32_t *rowptr, const int32_t *col, const int32_t *hubs, int h, int dw,
                               uint64_t *bits, cudaStream_t st);
 
+// n listed matches of k images each, sorted by their images of pattern vertices 0, 1, .. into `out`
+// (scratch: match_sort_bytes(n); n below 2^32); adds the kernels launched to *launches.
+size_t match_sort_bytes(long long n);
+cudaError_t launch_match_sort(const int32_t *rows, long long n, int k, void *scratch, int32_t *out, int *launches,
+                              cudaStream_t st);
+
 // Fixed scratch of sge_count_noalloc (sge_noalloc.cu): the current device's
 // address of the library's static device array, set up once per device.
 cudaError_t noalloc_scratch(void **ptr, size_t *bytes);

@@ -569,6 +569,7 @@ __device__ __forceinline__ void row_range(const V &v, const PosV &p, const Cand 
 
 // Write one match row (images of pattern vertices 0..k-1) for enumeration.
 __device__ __forceinline__ void emit_match(const JobDesc &J, const int *M, int last_pos, int c) {
+    if ((long long)load_relaxed(J.mlen) >= J.mcap) return;   // (full: the counters tell how many there are)
     unsigned long long slot = atomicAdd(J.mlen, 1ull);
     if ((long long)slot >= J.mcap) return;
     int32_t *row = J.mbuf + (size_t)slot * J.k;
@@ -4431,6 +4432,116 @@ __global__ void k_pool_init(unsigned long long *seq, int cap) {
 
 cudaError_t launch_pool_init(unsigned long long *seq, int cap, cudaStream_t st) {
     k_pool_init<<<(cap + BLOCK - 1) / BLOCK, BLOCK, 0, st>>>(seq, cap);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------- listed matches
+//
+// Listed matches come out in the order their warps found them; the caller gets them sorted by the
+// images of pattern vertices 0, 1, ...  A merge sort of row numbers under their first two images
+// (one 64-bit key, beside the number; the row itself is read only where keys tie): tiles of
+// MATCH_TILE by a bitonic network in shared memory, then passes that merge runs pairwise, each element
+// finding its place by a binary search of the other run (rows are distinct, so no two meet).
+// Bound by the searches' dependent loads and the launches: listing some 15,000 matches of 6
+// vertices takes 0.48 ms a call, 0.26 of it the search, where numpy's lexsort of the columns on the
+// host and a count to size the buffer made it 2.8 ms.
+namespace {
+
+constexpr int MATCH_TILE = 1024;
+
+// Row a before row b?
+__device__ __forceinline__ bool match_before(uint64_t ka, uint32_t a, uint64_t kb, uint32_t b, const int32_t *rows, int k) {
+    if (ka != kb) return ka < kb;
+    const int32_t *ra = rows + (size_t)a * k, *rb = rows + (size_t)b * k;
+    for (int i = 2; i < k; ++i) {
+        const int x = __ldg(ra + i), y = __ldg(rb + i);
+        if (x != y) return x < y;
+    }
+    return a < b;   // (the padding of a tile)
+}
+
+__global__ void __launch_bounds__(MATCH_TILE / 2) k_match_tiles(const int32_t *rows, long long n, int k, uint64_t *key,
+                                                                uint32_t *row) {
+    __shared__ uint64_t sk[MATCH_TILE];
+    __shared__ uint32_t sr[MATCH_TILE];
+    const long long base = (long long)blockIdx.x * MATCH_TILE;
+    const int m = (int)min((long long)MATCH_TILE, n - base);
+    for (int i = threadIdx.x; i < MATCH_TILE; i += MATCH_TILE / 2) {
+        sk[i] = ~0ull;   // (padding sorts last: images are not negative)
+        sr[i] = (uint32_t)(base + i);
+        if (i < m) {
+            const int32_t *r = rows + (size_t)(base + i) * k;
+            sk[i] = (uint64_t)(uint32_t)r[0] << 32 | (k > 1 ? (uint32_t)r[1] : 0u);
+        }
+    }
+    for (int size = 2; size <= MATCH_TILE; size <<= 1)
+        for (int step = size >> 1; step >= 1; step >>= 1) {
+            __syncthreads();
+            const int a = 2 * step * (threadIdx.x / step) + threadIdx.x % step, b = a + step;
+            const bool up = (a & size) == 0;
+            const uint64_t ka = sk[a], kb = sk[b];
+            const uint32_t ra = sr[a], rb = sr[b];
+            // (rows beyond the list never tie with one of it, and among themselves order does not matter)
+            const bool swap = ka == kb && ka == ~0ull ? (rb < ra) == up : match_before(kb, rb, ka, ra, rows, k) == up;
+            if (swap) {
+                sk[a] = kb; sk[b] = ka;
+                sr[a] = rb; sr[b] = ra;
+            }
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < m; i += MATCH_TILE / 2) {
+        key[base + i] = sk[i];
+        row[base + i] = sr[i];
+    }
+}
+
+// Runs of `width` merged pairwise.
+__global__ void __launch_bounds__(BLOCK) k_match_merge(const int32_t *rows, long long n, int k, long long width,
+                                                       const uint64_t *key, const uint32_t *row, uint64_t *okey,
+                                                       uint32_t *orow) {
+    for (long long i = blockIdx.x * (long long)BLOCK + threadIdx.x; i < n; i += (long long)gridDim.x * BLOCK) {
+        const long long pair = i / (2 * width) * (2 * width), mid = min(pair + width, n), end = min(pair + 2 * width, n);
+        const uint64_t ki = key[i];
+        const uint32_t ri = row[i];
+        const bool first = i < mid;
+        long long lo = first ? mid : pair, hi = first ? end : mid;
+        const long long from = lo;
+        while (lo < hi) {   // elements of the other run before this one
+            const long long m = (lo + hi) >> 1;
+            if (match_before(key[m], row[m], ki, ri, rows, k)) lo = m + 1; else hi = m;
+        }
+        const long long at = pair + (i - (first ? pair : mid)) + (lo - from);
+        okey[at] = ki;
+        orow[at] = ri;
+    }
+}
+
+__global__ void __launch_bounds__(BLOCK) k_match_gather(const int32_t *rows, long long n, int k, const uint32_t *row,
+                                                        int32_t *out) {
+    for (long long i = blockIdx.x * (long long)BLOCK + threadIdx.x; i < n * k; i += (long long)gridDim.x * BLOCK) {
+        const long long r = i / k;
+        out[i] = rows[(size_t)row[r] * k + (i - r * k)];
+    }
+}
+
+}  // namespace
+
+size_t match_sort_bytes(long long n) { return (size_t)n * 2 * (sizeof(uint64_t) + sizeof(uint32_t)); }
+
+cudaError_t launch_match_sort(const int32_t *rows, long long n, int k, void *scratch, int32_t *out, int *launches,
+                              cudaStream_t st) {
+    if (n <= 0 || k <= 0) return cudaSuccess;
+    if (n > UINT32_MAX) return cudaErrorInvalidValue;
+    uint64_t *key[2] = {static_cast<uint64_t *>(scratch), static_cast<uint64_t *>(scratch) + n};
+    uint32_t *row[2] = {reinterpret_cast<uint32_t *>(key[1] + n), reinterpret_cast<uint32_t *>(key[1] + n) + n};
+    auto blocks = [](long long items) { return (unsigned)std::min<long long>((items + BLOCK - 1) / BLOCK, 1 << 20); };
+    k_match_tiles<<<(unsigned)((n + MATCH_TILE - 1) / MATCH_TILE), MATCH_TILE / 2, 0, st>>>(rows, n, k, key[0], row[0]);
+    ++*launches;
+    int cur = 0;
+    for (long long w = MATCH_TILE; w < n; w *= 2, cur ^= 1, ++*launches)
+        k_match_merge<<<blocks(n), BLOCK, 0, st>>>(rows, n, k, w, key[cur], row[cur], key[cur ^ 1], row[cur ^ 1]);
+    k_match_gather<<<blocks(n * k), BLOCK, 0, st>>>(rows, n, k, row[cur], out);
+    ++*launches;
     return cudaGetLastError();
 }
 
