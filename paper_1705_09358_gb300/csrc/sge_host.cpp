@@ -42,6 +42,7 @@ constexpr int HUB_MIN_DEGREE = 24;               // larger targets: bitset rows 
 constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device memory
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
 constexpr long long LIST_FIRST_ROWS = 1 << 16;   // matches a listing call has room for at first
+constexpr int LEAN_MIN_PAIRS = 4096;             // plain RI batches from this many pairs: records built on the device
 constexpr int POOL_CELLS = 1 << 15;
 constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
 constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
@@ -412,7 +413,7 @@ struct Workspace {
         ctask;
     DevBuf front[2], counts, offs, scan_tmp, total, splitctl;
     DevBuf pool, pseq, ctl, slab;
-    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft, msort, mout;
+    DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft, msort, mout, btarget, bpattern, bpair;
     unsigned long long aepoch = 0;   // last launch's mark in aentry (0: the entries are to be cleared)
     std::vector<Job> hjobs;       // the call's pairs, reused (their vectors keep their capacity)
     std::vector<JobDesc> hdesc;   // host job records, reused
@@ -425,12 +426,15 @@ struct Workspace {
     std::vector<std::vector<BackEdge>> hjback;
     std::vector<long long> hri_off;        // per pattern id: offsets of its RI tables in this call
     std::vector<int> hri_rep;              // per pattern id: a job of that pattern in this call (-1 after)
+    std::vector<int> htgt_rep;             // per target id: likewise, for the device-built records
+    std::vector<int2> hpair;               // device-built records: the pairs' table rows, and their first root frames
+    std::vector<int32_t> hroot;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, ev3 = nullptr;   // search kernel, split kernel
     cudaStream_t bound = nullptr;
 #define SGE_WS_BUFFERS                                                                                             \
     &jobs, &fjobs, &ctr, &filt, &pos, &back, &ulist, &unit_off, &vert_off, &sizes, &task, &flag, &dent, &deoff, &vchg, \
         &cand, &ctask, &front[0], &front[1], &counts, &offs, &scan_tmp, &total, &splitctl, &pool, &pseq, &ctl, &slab, \
-        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart, &aentry, &aleft, &msort, &mout
+        &mbuf, &ckpt, &wtrace, &smask, &plidx, &cstart, &aentry, &aleft, &msort, &mout, &btarget, &bpattern, &bpair
     // Every buffer of this workspace is used on `st` only: allocate them stream-ordered there.
     void bind(cudaStream_t st) {
         if (bound == st && st != nullptr) return;
@@ -816,12 +820,85 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     long long launches = 0;   // kernels launched by this call
     const int algo = o.algo;
     const int nj = (int)idx.size();
-    std::vector<Job> &jobs = W.hjobs;   // kept across calls (no fresh pages)
-    if (jobs.size() < (size_t)nj) jobs.resize((size_t)nj);
     bool directed = false, any_elab = false, any_runs = false;
     int kmax = 1, nmax = 1, max_pid = 0;
     std::mutex red;   // merges the threads' partial maxima
-    parallel_for(nj, [&](int q0, int q1) {
+    // a huge plain RI batch on the CSR kernel: no host record per pair, the device builds them from
+    // per-graph tables (lean); what the general path would take stays there
+    bool lean = algo == SGE_RI && nj >= LEAN_MIN_PAIRS && resume == nullptr && ckpt_frames == nullptr && !enumerate;
+    long long lean_roots = 0;   // root candidates of the searched pairs
+    std::vector<const TargetRec *> lean_targets;    // the call's distinct graphs, in id order
+    std::vector<const PatternRec *> lean_patterns;
+    std::vector<size_t> lean_at;                    // per distinct pattern: its tables' offsets (pos, back)
+    std::vector<int> &trep = W.htgt_rep, &prep = W.hri_rep;   // [id]: a pair of that graph, then its row; -1 after
+    if (lean) {
+        {
+            std::lock_guard<std::mutex> g(ctx->mu);
+            if (trep.size() < (size_t)ctx->next_target) trep.resize((size_t)ctx->next_target, -1);
+            if (prep.size() < (size_t)ctx->next_pattern) prep.resize((size_t)ctx->next_pattern, -1);
+        }
+        bool all_adj = true;
+        int max_tid = 0;
+        parallel_for(nj, [&](int q0, int q1) {
+            bool el = false, rn = false, adj = true;
+            int km = 1, nm = 1, mt = 0, mp = 0;
+            long long nr = 0;
+            for (int q = q0; q < q1; ++q) {
+                const PairReq &r = reqs[(size_t)idx[q]];
+                mt = std::max(mt, r.tid);
+                mp = std::max(mp, r.pid);
+                __atomic_store_n(&trep[(size_t)r.tid], q, __ATOMIC_RELAXED);
+                __atomic_store_n(&prep[(size_t)r.pid], q, __ATOMIC_RELAXED);
+                if (r.p->k == 0 || r.p->k > r.t->n) continue;
+                km = std::max(km, r.p->k);
+                nm = std::max(nm, r.t->n);
+                nr += r.t->n;
+                el = el || r.t->any_elab || r.p->any_elab;
+                rn = rn || r.t->cached.runs != nullptr;
+                adj = adj && r.t->cached.adj != nullptr;
+            }
+            std::lock_guard<std::mutex> g(red);
+            kmax = std::max(kmax, km);
+            nmax = std::max(nmax, nm);
+            max_tid = std::max(max_tid, mt);
+            max_pid = std::max(max_pid, mp);
+            any_elab = any_elab || el;
+            any_runs = any_runs || rn;
+            all_adj = all_adj && adj;
+            lean_roots += nr;
+        });
+        directed = reqs[(size_t)idx[0]].t->directed;
+        const bool csr = o.kernel == SGE_KERNEL_CSR ||
+                         (o.kernel == SGE_KERNEL_AUTO && (directed || any_elab || !all_adj));
+        lean = csr && !any_runs;
+        for (int id = 0; id <= max_tid; ++id)
+            if (int &x = trep[(size_t)id]; x >= 0) {
+                if (lean) lean_targets.push_back(reqs[(size_t)idx[x]].t);
+                x = lean ? (int)lean_targets.size() - 1 : -1;
+            }
+        for (int id = 0; id <= max_pid; ++id)
+            if (int &x = prep[(size_t)id]; x >= 0) {
+                if (lean) lean_patterns.push_back(reqs[(size_t)idx[x]].p);
+                x = lean ? (int)lean_patterns.size() - 1 : -1;
+            }
+        if (lean) {   // the pairs as rows of the tables, and the ids' marks taken back
+            W.hpair.resize((size_t)nj);
+            parallel_for(nj, [&](int q0, int q1) {
+                for (int q = q0; q < q1; ++q) {
+                    const PairReq &r = reqs[(size_t)idx[q]];
+                    W.hpair[(size_t)q] = make_int2(trep[(size_t)r.tid], prep[(size_t)r.pid]);
+                }
+            });
+            std::fill(trep.begin(), trep.begin() + max_tid + 1, -1);
+            std::fill(prep.begin(), prep.begin() + max_pid + 1, -1);
+        } else {
+            directed = any_elab = any_runs = false;
+            kmax = nmax = 1;
+        }
+    }
+    std::vector<Job> &jobs = W.hjobs;   // kept across calls (no fresh pages)
+    if (!lean && jobs.size() < (size_t)nj) jobs.resize((size_t)nj);
+    if (!lean) parallel_for(nj, [&](int q0, int q1) {
         bool el = false, rn = false;
         int km = 1, nm = 1, mp = 0;
         for (int q = q0; q < q1; ++q) {
@@ -854,13 +931,13 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         any_elab = any_elab || el;
         any_runs = any_runs || rn;
     });
-    if (nj > 0) directed = jobs[0].t->directed;   // (a group holds pairs of one directedness)
+    if (nj > 0 && !lean) directed = jobs[0].t->directed;   // (a group holds pairs of one directedness)
     // kernel family: the bitset kernel needs undirected, unlabelled edges, an
     // adjacency bitset and at most 4 words per lane with the level stack in
     // shared memory
-    bool bits_ok = !directed && !any_elab;
+    bool bits_ok = !directed && !any_elab && !lean;
     int nwl = 1;
-    for (int q = 0; q < nj; ++q)   // (the workspace's job vector may be longer than this call)
+    for (int q = 0; q < nj && !lean; ++q)   // (the workspace's job vector may be longer than this call)
         if (const Job &J = jobs[q]; J.active) {
             if (!J.t->adj.p) bits_ok = false;
             nwl = std::max(nwl, (J.t->dw + 31) / 32);
@@ -879,7 +956,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     // ---------------------------------------------------------- job tables
     long long filt_words = 0, nverts = 0, nunits = 0;
     std::vector<long long> unit_off, vert_off;
-    for (int q = 0; q < nj; ++q) {
+    for (int q = 0; q < nj && !lean; ++q) {
         Job &J = jobs[q];
         if (!J.active) continue;
         if (J.algo != SGE_RI || need_filt_all) {
@@ -888,12 +965,12 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         }
     }
     std::vector<JobDesc> &desc = W.hdesc;   // host copy kept across calls (no fresh pages)
-    desc.resize((size_t)nj);
+    if (!lean) desc.resize((size_t)nj);
     CK(W.filt.ensure(std::max<long long>(filt_words, 1) * 8), "alloc filter");
     // per job: 4 counters, then nj match-row counts, then nj byte counters
     CK(W.ctr.ensure((size_t)nj * 6 * sizeof(unsigned long long)), "alloc counters");
     CK(cudaMemsetAsync(W.ctr.p, 0, (size_t)nj * 6 * sizeof(unsigned long long), st), "clear counters");
-    parallel_for(nj, [&](int q0, int q1) {
+    if (!lean) parallel_for(nj, [&](int q0, int q1) {
         for (int q = q0; q < q1; ++q) {
             const Job &J = jobs[q];
             JobDesc &D = desc[q];
@@ -917,14 +994,14 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     const double t_desc = now_ms();
     // units of the domain kernels: (job, pattern vertex, 64-target word)
     std::vector<int> fjobs;  // jobs with a filter block, in order
-    for (int q = 0; q < nj; ++q)
+    for (int q = 0; q < nj && !lean; ++q)
         if (jobs[q].active && jobs[q].filt_off >= 0) fjobs.push_back(q);
     // jobs on targets with label runs, and RI-DS jobs on targets with a label-degree table
     // (undirected, no edge labels in the batch): their pattern vertices' label indices among
     // the target's labels, written on the device below
     bool any_plidx = false;
     const bool table = algo != SGE_RI && !any_elab && !directed;
-    if (any_runs || table) {
+    if ((any_runs || table) && !lean) {
         auto wants = [&](const Job &J) {
             return J.active && (J.t->cached.runs != nullptr || (table && !J.t->labs_h.empty()));
         };
@@ -1235,9 +1312,9 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     std::vector<BackEdge> &back = W.hback;
     pos.clear();
     back.clear();
-    std::vector<long long> pos_off(nj, 0), back_off(nj, 0);
+    std::vector<long long> pos_off(lean ? 0 : nj, 0), back_off(lean ? 0 : nj, 0);
     std::vector<int> task_job, task_vert, task_out;
-    std::vector<int> fidx(nj, -1);
+    std::vector<int> fidx(lean ? 0 : nj, -1);
     for (int x = 0; x < nf; ++x) fidx[fjobs[x]] = x;
     // an RI pattern's tables are appended once per call: their offsets, by pattern id
     std::vector<long long> &ri_off = W.hri_off;   // [pid]: pos offset, back offset (-1: not yet)
@@ -1253,7 +1330,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         jpos.resize((size_t)nj);
         jback.resize((size_t)nj);
     }
-    parallel_for(nj, [&](int q0, int q1) {
+    if (!lean) parallel_for(nj, [&](int q0, int q1) {
         for (int q = q0; q < q1; ++q) {
             Job &J = jobs[q];
             if (!J.active || J.algo == SGE_RI) continue;
@@ -1263,10 +1340,25 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     }, 64);
     if (trace_on()) {
         int act = 0;
-        for (int q = 0; q < nj; ++q) act += jobs[q].active && jobs[q].algo != SGE_RI;
+        for (int q = 0; q < nj && !lean; ++q) act += jobs[q].active && jobs[q].algo != SGE_RI;
         std::fprintf(stderr, "[sge] RI-DS orderings of %d live pairs built at %.3f ms\n", act, now_ms() - t_start);
     }
-    if (algo == SGE_RI) {
+    if (lean) {
+        // the distinct patterns' tables, in the order of the records' pattern rows
+        long long np = 0, nb = 0;
+        for (const PatternRec *P : lean_patterns) {
+            np += (long long)P->ri_pos.size();
+            nb += (long long)P->ri_back.size();
+        }
+        pos.reserve((size_t)np);
+        back.reserve((size_t)nb);
+        for (const PatternRec *P : lean_patterns) {
+            lean_at.push_back(pos.size());
+            lean_at.push_back(back.size());
+            pos.insert(pos.end(), P->ri_pos.begin(), P->ri_pos.end());
+            back.insert(back.end(), P->ri_back.begin(), P->ri_back.end());
+        }
+    } else if (algo == SGE_RI) {
         // the distinct patterns' tables: a job of each pattern is noted on several threads
         // (any job will do), the tables appended by pattern id, then every job's offsets set
         std::vector<int> &rep = W.hri_rep;   // [pid]: a job of that pattern, or -1
@@ -1356,7 +1448,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         const long long rows = std::max<long long>(match_cap, 1);
         CK(W.mbuf.ensure((size_t)rows * kmax * 4), "alloc match buffer");
     }
-    parallel_for(nj, [&](int q0, int q1) {
+    if (!lean) parallel_for(nj, [&](int q0, int q1) {
         for (int q = q0; q < q1; ++q) {
             JobDesc &D = desc[q];
             D.pos = W.pos.as<PosInfo>() + pos_off[q];
@@ -1379,7 +1471,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         }
     });
     const double t_up = now_ms();
-    CK(upload(W.jobs, desc, st), "upload jobs");
+    if (!lean) CK(upload(W.jobs, desc, st), "upload jobs");
     if (any_plidx && nf == 0) {   // (with domains they are there already)
         CK(launch_label_index(W.jobs.as<JobDesc>(), nj, st), "label indices");
         ++launches;
@@ -1402,12 +1494,12 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     // few as spread the call's root candidates over the resident warps, 32 to ROOT_CHUNK (a
     // single 1,000-vertex root scanned by one warp took 40 us, the first level's whole time)
     std::vector<std::array<int32_t, 4>> roots;
-    roots.reserve((size_t)nj);
-    long long nroot = 0;
-    for (int q = 0; q < nj; ++q)
+    if (!lean) roots.reserve((size_t)nj);
+    long long nroot = lean_roots;
+    for (int q = 0; q < nj && !lean; ++q)
         if (const Job &J = jobs[q]; J.active) nroot += J.algo == SGE_RI ? J.t->n : pos[pos_off[q]].ucnt;
     const long long chunk = std::min<long long>(ROOT_CHUNK, std::max<long long>(32, (nroot / resident_warps + 31) & ~31ll));
-    for (int q = 0; q < nj; ++q) {
+    for (int q = 0; q < nj && !lean; ++q) {
         const Job &J = jobs[q];
         if (!J.active) continue;
         const long long len = J.algo == SGE_RI ? J.t->n : pos[pos_off[q]].ucnt;
@@ -1419,6 +1511,77 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         }
     }
     long long F0 = (long long)roots.size();
+    JobTables tables;
+    std::memset(&tables, 0, sizeof(tables));
+    if (lean) {
+        std::vector<TargetView> trow;
+        std::vector<PatternRow> prow(lean_patterns.size());
+        for (const TargetRec *T : lean_targets) trow.push_back(T->cached);
+        for (size_t x = 0; x < prow.size(); ++x) {
+            const PatternRec &P = *lean_patterns[x];
+            PatternRow &r = prow[x];
+            std::memset(&r, 0, sizeof(r));
+            r.view = P.cached;
+            r.pos = W.pos.as<PosInfo>() + lean_at[2 * x];
+            r.back = W.back.as<BackEdge>() + lean_at[2 * x + 1];
+            for (size_t i = 1; i < P.ri_pos.size(); ++i) r.unparented |= P.ri_pos[i].par < 0;
+        }
+        // the pairs' first root frames (counted, then placed, in slices)
+        constexpr int SLICE = 8192;
+        const int slices = (nj + SLICE - 1) / SLICE;
+        std::vector<long long> first((size_t)slices + 1, 0);
+        const std::vector<int2> &pair = W.hpair;
+        std::vector<int32_t> &off = W.hroot;
+        off.resize((size_t)nj + 1);
+        auto frames_of = [&](const PairReq &r) -> long long {
+            if (r.p->k == 0 || r.p->k > r.t->n) return 0;
+            return r.t->n <= chunk ? 1 : (r.t->n + chunk - 1) / chunk;
+        };
+        parallel_for(slices, [&](int s0, int s1) {
+            for (int x = s0; x < s1; ++x) {
+                long long f = 0;
+                for (int q = x * SLICE; q < std::min(nj, (x + 1) * SLICE); ++q) f += frames_of(reqs[(size_t)idx[q]]);
+                first[(size_t)x + 1] = f;
+            }
+        }, 1);
+        for (int x = 0; x < slices; ++x) first[(size_t)x + 1] += first[(size_t)x];
+        F0 = first[(size_t)slices];
+        if (F0 > INT32_MAX) return fail(ctx, SGE_ERR_OOM, "too many root ranges");
+        parallel_for(slices, [&](int s0, int s1) {
+            for (int x = s0; x < s1; ++x) {
+                long long f = first[(size_t)x];
+                for (int q = x * SLICE; q < std::min(nj, (x + 1) * SLICE); ++q) {
+                    const PairReq &r = reqs[(size_t)idx[q]];
+                    off[(size_t)q] = (int32_t)f;
+                    f += frames_of(r);
+                }
+            }
+        }, 1);
+        off[(size_t)nj] = (int32_t)F0;
+        const size_t pair_bytes = ((size_t)nj * 8 + 15) & ~(size_t)15;
+        CK(W.bpair.ensure(pair_bytes + ((size_t)nj + 1) * 4), "alloc pairs");
+        CK(upload(W.btarget, trow, st), "upload target table");
+        CK(upload(W.bpattern, prow, st), "upload pattern table");
+        CK(cudaMemcpyAsync(W.bpair.p, pair.data(), (size_t)nj * 8, cudaMemcpyHostToDevice, st), "upload pairs");
+        CK(cudaMemcpyAsync(W.bpair.as<char>() + pair_bytes, off.data(), ((size_t)nj + 1) * 4, cudaMemcpyHostToDevice, st),
+           "upload root offsets");
+        CK(W.jobs.ensure((size_t)nj * sizeof(JobDesc)), "alloc jobs");
+        tables.target = W.btarget.as<TargetView>();
+        tables.pattern = W.bpattern.as<PatternRow>();
+        tables.pair = W.bpair.as<int2>();
+        tables.root_off = reinterpret_cast<const int32_t *>(W.bpair.as<char>() + pair_bytes);
+        tables.ctr = W.ctr.as<unsigned long long>();
+        tables.out = W.jobs.as<JobDesc>();
+        tables.nj = nj;
+        tables.flags = (any_elab ? JOB_ELAB : 0) | (directed ? JOB_DIRECTED : 0);
+        tables.chunk = (int32_t)chunk;
+        CK(W.front[0].ensure((size_t)std::max<long long>(F0 * FRAME_HDR, o.frontier_kib > 0 ? 256ll * o.frontier_kib
+                                                                                       : FRONTIER_MAX_INTS) * 4),
+           "alloc frontier");
+        tables.roots = W.front[0].as<int32_t>();
+        CK(launch_build_jobs(tables, st), "job records");
+        ++launches;
+    }
     long long F = 0;
     float split_ms = 0.f;   // device time of the cooperative split (CUDA events)
     float split_exec_ms = 0.f, search_exec_ms = 0.f;   // the kernels' own spans (device clock)
@@ -1459,8 +1622,9 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         const bool ordered = shard_count > 1 || !count_ctr;
         CK(W.front[0].ensure((size_t)cap_ints * 4), "alloc frontier");
         CK(W.front[1].ensure((size_t)cap_ints * 4), "alloc frontier");
-        CK(cudaMemcpyAsync(W.front[0].p, roots.data(), (size_t)F0 * sizeof(roots[0]), cudaMemcpyHostToDevice, st),
-           "upload roots");
+        if (!lean)
+            CK(cudaMemcpyAsync(W.front[0].p, roots.data(), (size_t)F0 * sizeof(roots[0]), cudaMemcpyHostToDevice, st),
+               "upload roots");
         const long long wcap = (long long)ctx->sms * 32 * search_warps_per_block();
         // (+ the level trace, + the asynchronous end's control lines)
         const size_t async_at = ((size_t)wcap + 16 + 2 * KMAX + 15) & ~(size_t)15;
@@ -1551,10 +1715,12 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     }
     if (!split_done && resume == nullptr) {
         fstride = FRAME_HDR;
-        std::vector<int32_t> f0;
-        for (const auto &r : roots) f0.insert(f0.end(), r.begin(), r.end());
         F = F0;
-        CK(upload(W.front[0], f0, st), "upload roots");
+        if (!lean) {
+            std::vector<int32_t> f0;
+            for (const auto &r : roots) f0.insert(f0.end(), r.begin(), r.end());
+            CK(upload(W.front[0], f0, st), "upload roots");
+        }
         while (F > 0 && depth < max_levels) {
             if (o.split_depth <= 0 && F >= target_frames) break;
             CK(W.counts.ensure((size_t)F * 4), "alloc counts");
@@ -1782,12 +1948,14 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
     }
     std::vector<unsigned long long> &ctr = W.hctr;   // kept across calls (no fresh pages)
     if (ctr.size() < (size_t)nj * 6) ctr.resize((size_t)nj * 6);
-    CK(cudaMemcpyAsync(ctr.data(), W.ctr.p, (size_t)nj * 6 * 8, cudaMemcpyDeviceToHost, st), "read counters");
+    // (the row counts and byte counters only where something wrote them)
+    const int nctr = kernel == SGE_KERNEL_BITSET || enumerate ? 6 : 4;
+    CK(cudaMemcpyAsync(ctr.data(), W.ctr.p, (size_t)nj * nctr * 8, cudaMemcpyDeviceToHost, st), "read counters");
     CK(cudaStreamSynchronize(st), "counter sync");
     const double t_end = now_ms();
     parallel_for(nj, [&](int q0, int q1) {
         for (int q = q0; q < q1; ++q) {
-            sge_result &r = out[jobs[q].pair];
+            sge_result &r = out[idx[q]];
             std::memset(&r, 0, sizeof(r));
             r.matches = ctr[4 * (size_t)q + 0];
             r.states = ctr[4 * (size_t)q + 1];

@@ -315,6 +315,27 @@ cudaError_t launch_frames_to_rows(const JobDesc *jobs, int32_t *frames, long lon
 cudaError_t launch_build_hubs(const int32_t *rowptr, const int32_t *col, const int32_t *hubs, int h, int dw,
                               uint64_t *bits, cudaStream_t st);
 
+// The records and root frames of a plain RI batch, built on the device (see k_build_jobs).
+struct PatternRow {
+    PatternView view;
+    const PosInfo *pos;
+    const BackEdge *back;
+    int32_t unparented;   // some position after the first has no parent
+    int32_t pad;
+};
+struct JobTables {
+    const TargetView *target;     // the call's distinct targets
+    const PatternRow *pattern;    // and patterns
+    const int2 *pair;             // a pair's rows in the two tables
+    const int32_t *root_off;      // [nj + 1] first root frame of a job (none: no search)
+    unsigned long long *ctr;      // 4 counters a job, then nj row counts, then nj byte counters
+    JobDesc *out;
+    int32_t *roots;               // frames of 4 ints
+    long long nj;
+    int32_t flags, chunk;         // JOB_ELAB, JOB_DIRECTED; candidates per root range
+};
+cudaError_t launch_build_jobs(const JobTables &T, cudaStream_t st);
+
 // n listed matches of k images each, sorted by their images of pattern vertices 0, 1, .. into `out`
 // (scratch: match_sort_bytes(n); n below 2^32); adds the kernels launched to *launches.
 size_t match_sort_bytes(long long n);

@@ -4435,6 +4435,65 @@ cudaError_t launch_pool_init(unsigned long long *seq, int cap, cudaStream_t st) 
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------- records of a huge batch
+//
+// A plain RI batch of many pairs repeats few targets and patterns, so its job records (368 bytes
+// each) and root frames are put together here from per-graph tables and 12 bytes per pair: one warp
+// writes one record, its words spread over the lanes.  Bound by the record writes (200,000
+// pairs: 74 MB; written by 16 host threads, uploaded, and given their roots by one, they took
+// 4.5 ms of a 9.7 ms call).
+namespace {
+__global__ void __launch_bounds__(BLOCK) k_build_jobs(JobTables T) {
+    __shared__ JobDesc rec[WARPS_PER_BLOCK];
+    const int lane = threadIdx.x & 31;
+    JobDesc &D = rec[threadIdx.x >> 5];
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < T.nj; q += nw) {
+        const int2 pair = T.pair[q];
+        const TargetView *t = T.target + pair.x;
+        const PatternRow *p = T.pattern + pair.y;
+        static_assert(sizeof(TargetView) % 4 == 0 && sizeof(PatternView) % 4 == 0 && sizeof(JobDesc) % 4 == 0, "copied as words");
+        for (int i = lane; i < (int)(sizeof(TargetView) / 4); i += 32)
+            reinterpret_cast<int *>(&D.t)[i] = reinterpret_cast<const int *>(t)[i];
+        for (int i = lane; i < (int)(sizeof(PatternView) / 4); i += 32)
+            reinterpret_cast<int *>(&D.p)[i] = reinterpret_cast<const int *>(&p->view)[i];
+        __syncwarp();
+        const int n = D.t.n, k = D.p.k;
+        if (lane == 0) {
+            const bool longl = D.t.maxdeg == 0 || D.t.maxdeg > SPLIT_RANGE || (p->unparented && n > SPLIT_RANGE);
+            D.pos = p->pos;
+            D.back = p->back;
+            D.filt = nullptr;
+            D.ulist = nullptr;
+            D.plidx = nullptr;
+            D.k = k;
+            D.flags = T.flags | (longl ? JOB_LONG_LISTS : 0);
+            D.ctr = T.ctr + 4 * q;
+            D.mbuf = nullptr;
+            D.mcap = 0;
+            D.mlen = T.ctr + 4 * T.nj + q;
+            D.abytes = T.ctr + 5 * T.nj + q;
+        }
+        __syncwarp();
+        for (int i = lane; i < (int)(sizeof(JobDesc) / 4); i += 32)
+            reinterpret_cast<int *>(T.out + q)[i] = reinterpret_cast<const int *>(&D)[i];
+        // its root frames: the whole list, or ranges of `chunk` candidates
+        const int r0 = T.root_off[q], r1 = T.root_off[q + 1];
+        for (int r = r0 + lane; r < r1; r += 32) {
+            const int b = r1 - r0 == 1 ? -1 : (r - r0) * T.chunk;
+            reinterpret_cast<int4 *>(T.roots)[r] = make_int4((int)q, 0, b, b < 0 ? -1 : min(b + T.chunk, n));
+        }
+        __syncwarp();
+    }
+}
+}  // namespace
+
+cudaError_t launch_build_jobs(const JobTables &T, cudaStream_t st) {
+    if (T.nj <= 0) return cudaSuccess;
+    k_build_jobs<<<(unsigned)std::min<long long>((T.nj + WARPS_PER_BLOCK - 1) / WARPS_PER_BLOCK, 1 << 16), BLOCK, 0, st>>>(T);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------- listed matches
 //
 // Listed matches come out in the order their warps found them; the caller gets them sorted by the
