@@ -50,6 +50,7 @@ constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per
 constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
 constexpr int BLOCK_FIXPOINT_MAX_N = 16384;      // auto domain mode: in-block fixpoint for targets up to this
 constexpr long long LABEL_TABLE_MAX = 1ll << 26; // most (vertex, label) entries of a target's degree table
+constexpr int WARP_FIXPOINT_MIN_JOBS = 8;        // auto domain mode: a warp per pair from this many pairs per SM
 constexpr int LIST_FIXPOINT_MIN_JOBS = 32;      // auto domain mode, small targets: in-block fixpoint over lists from
                                                  // this many pairs (large targets: always; on the 100k-vertex target it
                                                  // beat the sweeps from 1 to 32 pairs)
@@ -358,6 +359,7 @@ struct PatternRec {
     PatternView cached{};   // view(), taken once the record is complete
     int k = 0;
     bool directed = false, any_elab = false;
+    int edge_classes = 1;                  // distinct labels among its out-edges, plus those among its in-edges
     std::vector<int32_t> lab, odeg, ideg;
     std::vector<int> amat;                 // k x k arc labels, NO_ARC if absent
     std::vector<uint64_t> nb;              // undirected neighbourhood bitsets (2 words per vertex)
@@ -426,6 +428,8 @@ struct Workspace {
     std::vector<std::vector<BackEdge>> hjback;
     std::vector<long long> hri_off;        // per pattern id: offsets of its RI tables in this call
     std::vector<int> hri_rep;              // per pattern id: a job of that pattern in this call (-1 after)
+    std::vector<int2> hlive;               // pairs left by the fixpoint of a huge batch {pair, first size}, reused
+    std::vector<int32_t> hlive_size;
     std::vector<int> htgt_rep;             // per target id: likewise, for the device-built records
     std::vector<int2> hpair;               // device-built records: the pairs' table rows, and their first root frames
     std::vector<int32_t> hroot;
@@ -1050,7 +1054,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             CK(launch_label_index(W.fjobs.as<JobDesc>(), nf, st), "label indices");
             ++launches;
         }
-        CK(W.sizes.ensure((size_t)nverts * 8), "alloc sizes");
+        CK(W.sizes.ensure((size_t)nverts * 8 + (size_t)nf * 8), "alloc sizes");
         CK(W.flag.ensure(64), "alloc flag");
         trace_phase(st, "domain uploads", t_start);
         if (any_buckets) CK(cudaMemsetAsync(W.filt.p, 0, (size_t)filt_words * 8, st), "clear domains");
@@ -1078,13 +1082,20 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         int coop_status = 0;
         int nrids = 0;
         bool small_targets = true;
+        int classes_max = 1;   // edge classes (direction and label) of a pattern
         for (int q : fjobs) {
+            classes_max = std::max(classes_max, any_elab ? jobs[q].p->edge_classes : directed ? 2 : 1);
             nrids += jobs[q].algo != SGE_RI ? 1 : 0;
             small_targets = small_targets && jobs[q].t->n <= BLOCK_FIXPOINT_MAX_N;
         }
         const bool block_fixpoint = any_rids && small_targets &&
                                     (o.domain_fixpoint == SGE_DOMAIN_BLOCKS ||
                                      (o.domain_fixpoint == SGE_DOMAIN_AUTO && nrids >= ctx->sms / 2));
+        // very many of them, of small graphs: one warp a pair (below eight to an SM the SM's 32
+        // warps would not all have one, and a block's four warps end a pair sooner)
+        const bool warp_fixpoint = block_fixpoint && o.domain_fixpoint == SGE_DOMAIN_AUTO && nrids == nf &&
+                                   domain_fixpoint_warp_fits(kmax, nmax, classes_max) && nf <= 1 << 23 &&
+                                   nf >= ctx->sms * WARP_FIXPOINT_MIN_JOBS;
         // few pairs: the whole device sweeps them in one cooperative launch, if the slots that its
         // candidates can need (a domain holds vertices of one label) fit
         bool coop = any_rids && !block_fixpoint && o.domain_fixpoint == SGE_DOMAIN_AUTO && nrids == nf &&
@@ -1116,6 +1127,33 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             if (trace_on()) {
                 CK(cudaStreamSynchronize(st), "fixpoint sync");
                 std::fprintf(stderr, "[sge] domain fixpoint by the whole device: %d jobs at %.3f ms\n", nf, now_ms() - t_start);
+            }
+        } else if (warp_fixpoint) {
+            WarpFixpoint X;
+            X.nmax = (nmax + 31) & ~31;
+            X.classes = classes_max;
+            X.next = W.flag.as<unsigned long long>() + 4;
+            X.alive = X.next + 1;
+            X.list = W.sizes.as<int2>();
+            X.sizes = reinterpret_cast<int32_t *>(X.list + nf);
+            CK(launch_domain_fixpoint_warp(W.fjobs.as<JobDesc>(), nf, X, st), "domain fixpoint");
+            ++launches;
+            unsigned long long listed = 0;
+            CK(cudaMemcpyAsync(&listed, X.alive, 8, cudaMemcpyDeviceToHost, st), "read live pairs");
+            CK(cudaStreamSynchronize(st), "fixpoint sync");
+            const int live = (int)(listed >> 40);
+            const long long nsize = (long long)(listed & ((1ull << 40) - 1));
+            W.hlive.resize((size_t)live);
+            W.hlive_size.resize((size_t)nsize);
+            if (live > 0) {
+                CK(cudaMemcpyAsync(W.hlive.data(), X.list, (size_t)live * 8, cudaMemcpyDeviceToHost, st), "read live pairs");
+                CK(cudaMemcpyAsync(W.hlive_size.data(), X.sizes, (size_t)nsize * 4, cudaMemcpyDeviceToHost, st), "read sizes");
+                CK(cudaStreamSynchronize(st), "sizes sync");
+            }
+            if (trace_on()) {
+                CK(cudaStreamSynchronize(st), "fixpoint sync");
+                std::fprintf(stderr, "[sge] domain fixpoint in warps: %d of %d pairs live at %.3f ms\n", live, nf,
+                             now_ms() - t_start);
             }
         } else if (block_fixpoint) {
             CK(launch_domain_fixpoint(W.fjobs.as<JobDesc>(), nf, nullptr, nullptr, nullptr, nullptr,
@@ -1286,15 +1324,30 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                 mark_neighbours();   // only neighbours of domains that forward checking shrank
             }
         }
-        CK(launch_domain_sizes(W.fjobs.as<JobDesc>(), W.vert_off.as<long long>(), nf, nverts,
-                               W.sizes.as<long long>(), st), "domain sizes");
-        ++launches;
         std::vector<long long> &sizes = W.hsizes;   // kept across calls (no fresh pages)
         if (sizes.size() < (size_t)nverts) sizes.resize((size_t)nverts);
-        CK(cudaMemcpyAsync(sizes.data(), W.sizes.p, (size_t)nverts * 8, cudaMemcpyDeviceToHost, st), "read sizes");
-        CK(cudaStreamSynchronize(st), "sizes sync");
+        if (warp_fixpoint) {
+            parallel_for(nf, [&](int x0, int x1) {
+                for (int x = x0; x < x1; ++x) jobs[fjobs[x]].active = false;
+            });
+            parallel_for((int)W.hlive.size(), [&](int x0, int x1) {
+                for (int x = x0; x < x1; ++x) {
+                    Job &J = jobs[fjobs[W.hlive[(size_t)x].x]];
+                    J.active = true;
+                    J.dsize = sizes.data() + J.vert_off;
+                    const int32_t *from = W.hlive_size.data() + W.hlive[(size_t)x].y;
+                    std::copy(from, from + J.p->k, sizes.data() + J.vert_off);
+                }
+            });
+        } else {
+            CK(launch_domain_sizes(W.fjobs.as<JobDesc>(), W.vert_off.as<long long>(), nf, nverts,
+                                   W.sizes.as<long long>(), st), "domain sizes");
+            ++launches;
+            CK(cudaMemcpyAsync(sizes.data(), W.sizes.p, (size_t)nverts * 8, cudaMemcpyDeviceToHost, st), "read sizes");
+            CK(cudaStreamSynchronize(st), "sizes sync");
+        }
         if (coop_status != 0) return fail(ctx, SGE_ERR_CUDA, "device domain fixpoint failed");
-        parallel_for(nf, [&](int x0, int x1) {
+        if (!warp_fixpoint) parallel_for(nf, [&](int x0, int x1) {
             for (int x = x0; x < x1; ++x) {
                 Job &J = jobs[fjobs[x]];
                 J.dsize = sizes.data() + J.vert_off;
@@ -2650,6 +2703,9 @@ sge_status sge_load_pattern(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *s
             P->nb[2 * v + (w >> 6)] |= 1ull << (w & 63);
             P->nb[2 * w + (v >> 6)] |= 1ull << (v & 63);
         }
+    std::vector<int32_t> el(g.out.lab);
+    std::sort(el.begin(), el.end());
+    P->edge_classes = std::max(1, (int)(std::unique(el.begin(), el.end()) - el.begin()) * (g.directed ? 2 : 1));
     gcf_order(*P, SGE_RI, nullptr, P->ri_mu, P->ri_par);
     build_positions(*P, P->ri_mu, P->ri_par, SGE_RI, nullptr, 0, P->ri_pos, P->ri_back);
     std::vector<int32_t> img;   // the host image of P->dall

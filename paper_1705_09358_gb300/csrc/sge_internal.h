@@ -247,6 +247,16 @@ cudaError_t launch_domain_fc(const JobDesc *jobs, const long long *vert_off, con
 // sweeps scan domain words; else they walk each vertex's candidate list
 // (slots [cstart[g], cstart[g] + csize[g]), g = vert_off[job] + v).  Blocks
 // take jobs from the counter `next_job` (one int of device scratch, zeroed here).
+// The fixpoint with a warp per pair (sizes within domain_fixpoint_warp_fits, all RI-DS): the pairs left with candidates everywhere are listed, with their domain sizes.
+struct WarpFixpoint {
+    int nmax, classes;           // largest target (rounded up to 32), most edge classes of a pattern
+    unsigned long long *next;    // next pair
+    unsigned long long *alive;   // (next + 1) listed pairs << 40 | sizes written
+    int2 *list;                  // {pair, first size}
+    int32_t *sizes;              // |D(v)| of the listed pairs, v = 0, 1, ..
+};
+cudaError_t launch_domain_fixpoint_warp(const JobDesc *jobs, int njobs, const WarpFixpoint &W, cudaStream_t st);
+bool domain_fixpoint_warp_fits(int k, int n, int classes);   // of the largest pattern, target, class count
 cudaError_t launch_domain_fixpoint(const JobDesc *jobs, int njobs, const long long *vert_off, const long long *cstart,
                                    const long long *csize, int32_t *cand, int *next_job, cudaStream_t st);
 // The same for a few jobs by the whole device, one cooperative launch (see k_domain_coop): at most
