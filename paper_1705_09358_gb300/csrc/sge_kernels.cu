@@ -4491,7 +4491,9 @@ cudaError_t launch_domain_fixpoint_warp(const JobDesc *jobs, int njobs, const Wa
     if (W.nmax > WARP_FP_N || W.classes > WARP_FP_CLASSES || (W.nmax & 31)) return cudaErrorInvalidValue;
     const int smem = WARPS_PER_BLOCK * warp_fixpoint_smem(W.nmax, W.classes);
     int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = cudaFuncSetAttribute(k_domain_fixpoint_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (the attribute is the function's, for every thread of the process: always the largest launch's)
+    cudaError_t e = cudaFuncSetAttribute(k_domain_fixpoint_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         WARPS_PER_BLOCK * warp_fixpoint_smem(WARP_FP_N, WARP_FP_CLASSES));
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_domain_fixpoint_warp, BLOCK, smem);
