@@ -344,6 +344,22 @@ struct TargetRec {
     ~TargetRec() { release(); }
 };
 
+// Readies the asynchronous split's queue for one launch: its entries, its list of frames left,
+// and the mark that tells this launch's entries from what the block held before -- `epoch`, below
+// 2^24 and new for every launch.  0 says that the entries may hold anything: it is set before the
+// block is allocated, and a launch gets a mark only once the clearing of the whole block is queued,
+// so a call that fails in between leaves the next one to clear it.
+template <class Buf, class Clear>
+cudaError_t split_queue_ready(Buf &entry, size_t entry_bytes, Buf &left, size_t left_bytes, unsigned long long &epoch,
+                              Clear clear) {
+    if (entry.p == nullptr || entry.cap < entry_bytes || epoch + 1 >= (1ull << 24)) epoch = 0;
+    cudaError_t e = left.ensure(left_bytes);
+    if (e == cudaSuccess) e = entry.ensure(entry_bytes);
+    if (e == cudaSuccess && epoch == 0) e = clear(entry.p, entry.cap);
+    if (e == cudaSuccess) ++epoch;
+    return e;
+}
+
 // The host-side facts about a pattern that the ordering and the position
 // tables read: labels, degrees, the k x k arc-label matrix and undirected
 // neighbourhood bitsets (two words per vertex, k <= 128).
@@ -416,7 +432,7 @@ struct Workspace {
     DevBuf front[2], counts, offs, scan_tmp, total, splitctl;
     DevBuf pool, pseq, ctl, slab;
     DevBuf mbuf, ckpt, wtrace, smask, plidx, cstart, aentry, aleft, msort, mout, btarget, bpattern, bpair;
-    unsigned long long aepoch = 0;   // last launch's mark in aentry (0: the entries are to be cleared)
+    unsigned long long aepoch = 0;   // last launch's mark in aentry (0: see split_queue_ready)
     std::vector<Job> hjobs;       // the call's pairs, reused (their vectors keep their capacity)
     std::vector<JobDesc> hdesc;   // host job records, reused
     std::vector<JobDesc> hfdesc;  // host records of the jobs with a filter block, reused
@@ -1699,14 +1715,11 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             async.narrow = resident_warps;
             async.ctl = wtot + async_at;
             async.qcap = ASYNC_QUEUE;
-            const bool fresh = W.aentry.p == nullptr || W.aepoch + 1 >= (1ull << 24);
-            CK(W.aentry.ensure((size_t)ASYNC_QUEUE * 8), "alloc split queue");
-            CK(W.aleft.ensure((size_t)(ASYNC_QUEUE + 64 * wcap + async.narrow) * 8), "alloc split list");
-            if (fresh) {
-                CK(cudaMemsetAsync(W.aentry.p, 0, (size_t)ASYNC_QUEUE * 8, st), "clear split queue");
-                W.aepoch = 0;
-            }
-            async.epoch = ++W.aepoch;
+            CK(split_queue_ready(W.aentry, (size_t)ASYNC_QUEUE * 8, W.aleft,
+                                 (size_t)(ASYNC_QUEUE + 64 * wcap + async.narrow) * 8, W.aepoch,
+                                 [&](void *p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st); }),
+               "split queue");
+            async.epoch = W.aepoch;
             async.entries = W.aentry.as<unsigned long long>();
             async.left = W.aleft.as<const int32_t *>();
         }
