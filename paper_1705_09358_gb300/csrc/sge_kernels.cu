@@ -42,6 +42,7 @@ constexpr int DONATE_MIN_LEVELS = 2;     // a donated node keeps at least this m
 constexpr unsigned long long IDLE_GUARD_NS = 60ull * 1000000000ull;   // 60 s idle: internal error
 constexpr long long RESERVE_SPIN_LIMIT = 1 << 20;   // bounded wait for a queue cell's previous lap
 constexpr int RESERVE_TICKETS = 64;                  // producer tickets tried before keeping the work
+constexpr int DRAW_TRIES = 4;                        // attempts at waiting tickets before looking again later
 // Idle back-off caps (ns): one warp per block polls for work at short
 // intervals, the others at longer ones.  A waiting consumer polls only its own
 // queue cell, so short intervals cost little and hand donated work over fast
@@ -3134,27 +3135,54 @@ __global__ void __launch_bounds__(BLOCK) k_scan_add(long long *out, long long n,
 // and every frame reaches exactly one consumer.  Lane 0 only.
 constexpr unsigned long long CELL_LOCK = 1ull << 63;
 
+// Producer holding ticket t: locks its cell for writing.  False if consumer t left, or if the
+// launch is stopping (the caller keeps its work).  The cell's previous lap ends by itself: its
+// frame is being written or goes to a consumer that waits for it.
+__device__ bool cell_lock(const SearchCtl &C, unsigned long long t) {
+    unsigned long long *seq = C.pseq + t % (unsigned long long)C.pcap;
+    for (long long spin = 0;; ++spin) {
+        const unsigned long long sv = load_acquire(seq);
+        if (sv == t) {
+            if (atomicCAS(seq, t, t | CELL_LOCK) == t) return true;
+            continue;                                   // consumer t left meanwhile: look again
+        }
+        if ((sv & ~CELL_LOCK) > t) return false;        // consumer t left
+        if ((spin & 63) == 63 && load_relaxed(C.status) != 0) return false;
+        if (spin > RESERVE_SPIN_LIMIT) {                // the cell's previous lap never ended
+            set_status(C.status, -3);
+            return false;
+        }
+        __nanosleep(128);
+    }
+}
+
 // Producer: a ticket whose cell is locked for writing, or -1 (the caller keeps its work).
 __device__ long long queue_reserve(const SearchCtl &C) {
-    const unsigned long long cap = (unsigned long long)C.pcap;
-    for (int a = 0; a < RESERVE_TICKETS; ++a) {
+    for (int a = 0; a < RESERVE_TICKETS && load_relaxed(C.status) == 0; ++a) {
         const unsigned long long t = atomicAdd(C.ptail, 1ull);
-        unsigned long long *seq = C.pseq + t % cap;
-        for (long long spin = 0;; ++spin) {
-            const unsigned long long sv = load_acquire(seq);
-            if (sv == t) {
-                if (atomicCAS(seq, t, t | CELL_LOCK) == t) return (long long)t;
-                continue;                                   // consumer t left meanwhile: look again
-            }
-            if ((sv & ~CELL_LOCK) > t) break;               // consumer t left: draw another ticket
-            if (spin > RESERVE_SPIN_LIMIT) {                // the cell's previous lap never ended
-                set_status(C.status, -3);
-                return -1;
-            }
-            __nanosleep(128);
-        }
+        if (cell_lock(C, t)) return (long long)t;
     }
     return -1;
+}
+
+// Producer: draws up to `most` consecutive tickets, but only ones that consumers hold already, and
+// returns how many (the first one in t).  Consumer tickets only grow in number, so ptail never
+// passes phead: however many donors see the same idle warps, together they hand out no more frames
+// than there are warps waiting, and no frame lies in a cell that nobody comes for.
+__device__ int queue_draw(const SearchCtl &C, int most, unsigned long long &t) {
+    unsigned long long tail = load_relaxed(C.ptail);
+    for (int a = 0; a < DRAW_TRIES; ++a) {
+        const long long waiting = (long long)(load_relaxed(C.phead) - tail);
+        if (waiting <= 0) return 0;
+        const int n = (int)min((long long)most, waiting);
+        const unsigned long long seen = atomicCAS(C.ptail, tail, tail + (unsigned long long)n);
+        if (seen == tail) {
+            t = tail;
+            return n;
+        }
+        tail = seen;   // another donor was first
+    }
+    return 0;
 }
 
 // Consumer holding ticket t: is its frame published?  (An unordered poll: an acquire at every look
@@ -3179,7 +3207,8 @@ __device__ bool queue_leave(const SearchCtl &C, unsigned long long t, bool stopp
             continue;
         }
         if (!(sv & CELL_LOCK) && sv < t) return stopping;   // previous lap still in use
-        // locked by producer t, which publishes within a few instructions: wait
+        // locked by a producer, which publishes once its warp has the other cells of its donation
+        // (each of them waits for a consumer that is there): wait
         if (spin > RESERVE_SPIN_LIMIT) {
             set_status(C.status, -3);
             return true;
@@ -3188,18 +3217,11 @@ __device__ bool queue_leave(const SearchCtl &C, unsigned long long t, bool stopp
     }
 }
 
-// Warp-collective: push frame [j, depth, beg, end, M[0..mlen-1] (+ last)]
-// (`last` >= 0 appends one more image).  Returns false if the queue is full.
-__device__ bool push_frame(const SearchCtl &C, int j, int depth, int beg, int end, const int *M, int mlen, int last) {
+// Warp-collective: writes frame [j, depth, beg, end, M[0..mlen-1] (+ last)] to the locked cell
+// of ticket t and publishes it (`last` >= 0 appends one more image).
+__device__ __forceinline__ void publish_frame(const SearchCtl &C, long long t, int j, int depth, int beg, int end,
+                                              const int *M, int mlen, int last) {
     const int lane = threadIdx.x & 31;
-    long long t = -1;
-    if (lane == 0) {
-        atomicAdd(C.outstanding, 1);
-        t = queue_reserve(C);
-        if (t < 0) atomicSub(C.outstanding, 1);
-    }
-    t = __shfl_sync(FULL, t, 0);
-    if (t < 0) return false;
     int32_t *cell = C.pool + (size_t)(t % C.pcap) * POOL_STRIDE;
     if (lane == 0) { cell[0] = j; cell[1] = depth; cell[2] = beg; cell[3] = end; }
     for (int i = lane; i < mlen; i += 32) cell[FRAME_HDR + i] = M[i];
@@ -3211,45 +3233,59 @@ __device__ bool push_frame(const SearchCtl &C, int j, int depth, int beg, int en
         atomicAdd(C.donations, 1ull);
     }
     __syncwarp();
+}
+
+// Warp-collective: push one frame.  Returns false if no cell would take it.
+__device__ bool push_frame(const SearchCtl &C, int j, int depth, int beg, int end, const int *M, int mlen, int last) {
+    long long t = -1;
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(C.outstanding, 1);
+        t = queue_reserve(C);
+        if (t < 0) atomicSub(C.outstanding, 1);
+    }
+    t = __shfl_sync(FULL, t, 0);
+    if (t < 0) return false;
+    publish_frame(C, t, j, depth, beg, end, M, mlen, last);
     return true;
 }
 
-// Warp-collective: push one frame [j, depth, -1, -1, M[0..depth-2], c] for every lane in `mask`
-// (c: the lane's last image), all tickets drawn with one fetch-and-add and every lane working on
-// its own cell.  Some cells may not take a frame (a consumer that left, a cell still in its previous
-// lap): the frames go out lowest lane first, and the lanes whose frame was taken, the lowest ones of
-// `mask`, are returned (a checkpoint writes what is left of a chunk as one range from its lowest
-// pending survivor on).
-__device__ unsigned push_children(const SearchCtl &C, int j, int depth, const int *M, unsigned mask, int c) {
-    const int lane = threadIdx.x & 31;
-    const int n = __popc(mask);
-    const unsigned long long cap = (unsigned long long)C.pcap;
-    unsigned long long t = 0;
-    if (lane == 0) {
-        atomicAdd(C.outstanding, n);
-        t = atomicAdd(C.ptail, (unsigned long long)n);
-    }
-    t = __shfl_sync(FULL, t, 0) + __popc(mask & ((1u << lane) - 1u));
-    bool got = false;
-    if ((mask >> lane) & 1u) {
-        unsigned long long *seq = C.pseq + t % cap;
-        for (long long spin = 0;; ++spin) {
-            const unsigned long long sv = load_acquire(seq);
-            if (sv == t) {
-                if (atomicCAS(seq, t, t | CELL_LOCK) == t) {
-                    got = true;
-                    break;
-                }
-                continue;                                   // consumer t left meanwhile: look again
-            }
-            if ((sv & ~CELL_LOCK) > t) break;               // consumer t left
-            if (spin > RESERVE_SPIN_LIMIT) {                // the cell's previous lap never ended
-                set_status(C.status, -3);
-                break;
-            }
-            __nanosleep(128);
+// Warp-collective: the same for a warp that is already waiting; false if none is.
+__device__ bool push_to_waiting(const SearchCtl &C, int j, int depth, int beg, int end, const int *M, int mlen) {
+    long long t = -1;
+    if ((threadIdx.x & 31) == 0) {
+        unsigned long long at = 0;
+        if (queue_draw(C, 1, at) == 1) {
+            atomicAdd(C.outstanding, 1);
+            if (cell_lock(C, at)) t = (long long)at;
+            else atomicSub(C.outstanding, 1);
         }
     }
+    t = __shfl_sync(FULL, t, 0);
+    if (t < 0) return false;
+    publish_frame(C, t, j, depth, beg, end, M, mlen, -1);
+    return true;
+}
+
+// Warp-collective: push a frame [j, depth, -1, -1, M[0..depth-2], c] for up to `most` lanes of
+// `mask` (c: the lane's last image), as many as warps wait, every lane working on its own cell.
+// Some cells may not take a frame (a consumer that left): the frames go out lowest lane first, and
+// the lanes whose frame was taken, the lowest ones of `mask`, are returned (a checkpoint writes
+// what is left of a chunk as one range from its lowest pending survivor on).
+__device__ unsigned push_children(const SearchCtl &C, int j, int depth, const int *M, unsigned mask, int most, int c) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long cap = (unsigned long long)C.pcap;
+    unsigned long long t = 0;
+    int n = 0;
+    if (lane == 0) {
+        n = queue_draw(C, most, t);
+        if (n > 0) atomicAdd(C.outstanding, n);   // (this warp's own frame keeps the count above 0)
+    }
+    n = __shfl_sync(FULL, n, 0);
+    if (n == 0) return 0;
+    while (__popc(mask) > n) mask &= ~(0x80000000u >> __clz(mask));
+    t = __shfl_sync(FULL, t, 0) + __popc(mask & ((1u << lane) - 1u));
+    const bool got = ((mask >> lane) & 1u) && cell_lock(C, t);
+    __syncwarp();
     const unsigned locked = __ballot_sync(FULL, got);
     int32_t *cell = C.pool + (size_t)(t % cap) * POOL_STRIDE;
     // the r-th locked cell takes the r-th lane's frame
@@ -3716,21 +3752,20 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                     if (rem >= 64) {
                         const int mid = L.cur + ((rem / 2 + 31) & ~31);
                         const int run = L.kind >= LIST_RUN ? FRAME_RUN : 0;
-                        if (push_frame(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0) | run, mid, L.end, M, l, -1)) {
+                        if (push_to_waiting(C, fr.job, l | (l == quiet ? FRAME_COUNTED : 0) | run, mid, L.end, M, l)) {
                             __syncwarp();
                             if (lane == 0) L.end = mid;
                             __syncwarp();
                         }
                         break;
                     }
-                    unsigned m = L.mask;
+                    const unsigned m = L.mask;
                     // (the current level keeps one for this warp, which would else be out of work)
                     const int most = min(min(want, C.gran), __popc(m) - (l == lvl ? 1 : 0));
                     if (most > 0) {
                         // the lowest ones, one per lane
-                        while (__popc(m) > most) m &= ~(0x80000000u >> __clz(m));
                         const int c = (m >> lane) & 1u ? entry(L, L.cbase + lane) : 0;
-                        const unsigned sent = push_children(C, fr.job, l + 1, M, m, c);
+                        const unsigned sent = push_children(C, fr.job, l + 1, M, m, most, c);
                         if (lane == 0) L.mask &= ~sent;
                         __syncwarp();
                         break;

@@ -1,0 +1,64 @@
+"""Donation in the CSR search when many warps start at once and most find nothing: a thousand heavy
+frames for a device with several thousand warps, donors that look on every iteration and hand out
+from one to 32 frames, undirected and directed, on targets with and without label runs, stopped and
+resumed, and in the entry point whose queue has fewer cells than the device has warps."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from gen.graphs import Graph
+from gpu_common import counters, engine
+
+pytestmark = pytest.mark.gpu
+
+
+def _target(seed, n, degree, directed):
+    r = np.random.default_rng(seed)
+    m = n * degree // (1 if directed else 2)
+    a, b = r.integers(0, n, 2 * m), r.integers(0, n, 2 * m)
+    lo, hi = (a, b) if directed else (np.minimum(a, b), np.maximum(a, b))
+    key = np.unique((lo.astype(np.int64) * n + hi)[lo != hi])
+    key = r.permutation(key)[:m]
+    return Graph(n, (key // n).astype(np.int32), (key % n).astype(np.int32), np.zeros(n, np.int32), None, directed)
+
+
+def _path(k, directed):
+    i = np.arange(k - 1, dtype=np.int32)
+    return Graph(k, i, i + 1, np.zeros(k, np.int32), None, directed)
+
+
+@pytest.mark.parametrize("n,degree,k,directed", [(1201, 11, 5, False), (1201, 3, 10, False), (800, 12, 5, True)])
+def test_heavy_frames_for_few_of_many_warps(n, degree, k, directed):
+    from paper_1705_09358_gb300 import sge_count_noalloc, sge_unload_pattern, sge_unload_target
+    g, p = _target(n + k, n, degree, directed), _path(k, directed)
+    want = tuple(oracle.run(g, p, 0)[key] for key in ("matches", "states", "nodes", "hash"))
+    assert want[1] > 5_000_000
+    E = engine()
+    tid, pid = E.load_target(g), E.load_pattern(p)
+    try:
+        for depth in (1, 2):
+            for opts in ({}, {"steal_granularity": 1}, {"steal_granularity": 32, "donate_every_iters": 1},
+                         {"donate_every_iters": 1, "blocks_per_sm": 1}, {"donate_every_us": 1}):
+                res = E.count(tid, pid, kernel=1, split_depth=depth, **opts)
+                assert counters(res) == want, (depth, opts)
+                assert res["donations"] > 0
+        # stopped before the end, then resumed with the frames that are left: all start at once
+        rc, rows, blob = E.count_batch_ckpt([tid], [pid], kernel=1, split_depth=1, state_budget=want[1] // 4)
+        assert rc == -4 and blob is not None
+        for _ in range(200):
+            rc, rows, blob = E.resume(blob, kernel=1, donate_every_iters=1, state_budget=want[1] // 3)
+            if blob is None:
+                break
+        assert rc == 0 and counters(rows[0]) == want
+        if not directed:
+            import torch
+            from test_zz_no_alloc import _device_csr
+            d = _device_csr(g)
+            rc, got = sge_count_noalloc(g.n, d["rowptr"].data_ptr(), d["col"].data_ptr(), d["vlabel"].data_ptr(), 0, p,
+                                        stream=torch.cuda.current_stream())
+            assert rc == 0 and counters(got) == want
+    finally:
+        sge_unload_pattern(E.h, pid)
+        sge_unload_target(E.h, tid)
