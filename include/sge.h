@@ -84,7 +84,8 @@ typedef struct {
     int32_t no_donation;       /* 1 = persistent kernel without work donation */
     int32_t donate_every_iters;/* a warp donates at most once per this many search iterations ... */
     int32_t donate_every_us;   /* ... or once per this many microseconds, whichever comes first
-                                  (defaults: CSR kernel 1024 / 500, bitset kernel 2^30 / 50) */
+                                  (defaults: CSR kernel 16 / 500, 1024 iterations with
+                                  donate_every_us given; bitset kernel 2^30 / 50) */
     int32_t domain_fixpoint;   /* RI-DS domains (arc consistency with forward checking, Section 4):
                                   SGE_DOMAIN_SWEEPS = sweeps over the whole device under a host
                                   loop; SGE_DOMAIN_BLOCKS = each pair's whole fixpoint in one block

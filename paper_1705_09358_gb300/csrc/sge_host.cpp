@@ -44,6 +44,14 @@ constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffe
 constexpr long long LIST_FIRST_ROWS = 1 << 16;   // matches a listing call has room for at first
 constexpr int LEAN_MIN_PAIRS = 4096;             // plain RI batches from this many pairs: records built on the device
 constexpr int POOL_CELLS = 1 << 15;
+// Iterations of the CSR search from one look for idle warps to the next.  A look reads two words
+// that every warp shares, an L2 round trip that the next iteration waits for; without it idle
+// warps wait.  Looking after every iteration / 2 / 4 / 16 / 64 / 1024, search kernel in ms: 160
+// queries on a 100,000-vertex network under a state budget 18.7 / 14.1 / 12.8 / 10.0 / 12.6 / 38.6,
+// 24 directed patterns 5.6 / 4.4 / 3.6 / 3.0 / 3.1 / 4.1, a dense 5,003-vertex target on this kernel
+// 59.7 / 38.6 / 25.6 / 18.6 / 17.2 / 18.7, paths of 5 on a sparse one from 20,000 frames
+// 20.6 / 16.1 / 12.5 / 10.9 / 10.8 / 11.7.
+constexpr int CSR_DONATE_ITERS = 16;
 constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
 constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
@@ -1853,14 +1861,12 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         // kernel sends a chunk's survivors together)
         C.gran = o.steal_granularity > 0 ? o.steal_granularity : kernel == SGE_KERNEL_BITSET ? 8 : 32;
         // donation cadence: a busy warp checks whether idle warps wait for work at most once
-        // per this many iterations or this much device time.  Donating costs a few microseconds
-        // (two fetch-and-adds and one cell write), so the bitset kernel checks every 50 us; the
-        // CSR kernel's searches are mostly finished by the breadth-first split and keep 500 us,
-        // except in serving groups: every 20 us there, so that the frames a group's split left
-        // (its deepest, heaviest subtrees) are shared before idle warps leave.
+        // per this many iterations or this much device time.  The bitset kernel's iterations are
+        // short, so it goes by time, 50 us (a donation costs a few microseconds).  The CSR kernel
+        // goes by iterations (CSR_DONATE_ITERS), or by 20 us in serving groups, where idle warps leave soon.
         const bool bits_k = kernel == SGE_KERNEL_BITSET;
         C.donate_iters = o.donate_every_iters > 0 ? o.donate_every_iters
-                         : bits_k ? (1 << 30) : o.donate_every_us > 0 ? 1024 : 1;
+                         : bits_k ? (1 << 30) : o.donate_every_us > 0 ? 1024 : CSR_DONATE_ITERS;
         C.donate_ns = (unsigned long long)(o.donate_every_us > 0 ? o.donate_every_us
                                            : (bits_k ? 50 : (serving ? 20 : 500))) * 1000ull;
         // serving groups: a warp idle for 200 us (ten donation periods without a frame for it)

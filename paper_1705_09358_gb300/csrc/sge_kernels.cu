@@ -3650,7 +3650,6 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
         // since the last fold (every 64 iterations): an iteration adds at most 32 nodes and a
         // candidate list below 2^24 states (longer lists go straight to the 64-bit total)
         unsigned st32 = 0, nd32 = 0, mt32 = 0;
-        const bool eager = C.donate_iters == 1;   // look for idle warps on every second iteration
         bool counts0 = true;   // the frame counted its first node's states
         // scan the next 32 candidates [cur, ..) of level `l`'s list
         auto scan = [&](int l, const PosV &p, const Cand &S, int cur, int end) {
@@ -3727,7 +3726,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                 }
                 if (must_stop(C, J, st, deadline, last_check, last_cancel)) { stopped = true; break; }
             }
-            if (C.donate && ((eager && (iter & 1) == 0) || iter - last_don_iter >= (unsigned)C.donate_iters ||
+            if (C.donate && (iter - last_don_iter >= (unsigned)C.donate_iters ||
                              ((iter & 7) == 0 && last_check - last_don_ns >= C.donate_ns))) {
                 // idle warps waiting for a frame (their tickets run ahead of the producers')?
                 last_don_iter = iter;

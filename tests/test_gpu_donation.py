@@ -62,3 +62,26 @@ def test_heavy_frames_for_few_of_many_warps(n, degree, k, directed):
     finally:
         sge_unload_pattern(E.h, pid)
         sge_unload_target(E.h, tid)
+
+
+def test_default_cadence_costs_no_more_than_a_wide_one():
+    """Looking for idle warps must not be what the search spends its time on: the default against
+    one look in 64 iterations, alternating (on directed patterns from few frames a look at
+    every iteration took 2.2 times as long)."""
+    from time import perf_counter
+    from paper_1705_09358_gb300 import sge_unload_pattern, sge_unload_target
+    g, p = _target(3, 3001, 10, True), _path(5, True)
+    E = engine()
+    tid, pid = E.load_target(g), E.load_pattern(p)
+    try:
+        times = {0: [], 64: []}
+        for _ in range(12):
+            for iters in times:
+                t0 = perf_counter()
+                E.count(tid, pid, kernel=1, split_depth=1, donate_every_iters=iters)
+                times[iters].append(perf_counter() - t0)
+        best = {i: sorted(t)[len(t) // 4] for i, t in times.items()}
+        assert best[0] < 1.5 * best[64], best
+    finally:
+        sge_unload_pattern(E.h, pid)
+        sge_unload_target(E.h, tid)
