@@ -233,6 +233,20 @@ __global__ void __launch_bounds__(IB) k_label_nbmax(const int32_t *rowptr, const
         }
 }
 
+// Each vertex's place among the ascending labels (every label is among them); one thread each.
+__global__ void __launch_bounds__(IB) k_label_places(const int32_t *vlab, int n, const int32_t *labs, int nlab,
+                                                     int32_t *lidx) {
+    const int v = blockIdx.x * IB + threadIdx.x;
+    if (v >= n) return;
+    const int x = vlab[v];
+    int lo = 0, hi = nlab - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(labs + mid) < x) lo = mid + 1; else hi = mid;
+    }
+    lidx[v] = lo;
+}
+
 // Label runs: one warp per vertex regroups its row by the neighbours' label index, ids
 // ascending within a label -- a counting sort whose counters are the vertex's own slots of
 // the run table: count, scan to the runs' ends, then place the row from its last entry
@@ -324,6 +338,13 @@ cudaError_t launch_label_degree_masks(const int2 *vld, int n, const int32_t *lab
     const long long units = (long long)nlab * LDM_DEGREES * dw;
     if (units <= 0) return cudaSuccess;
     k_label_degree_masks<<<blocks_for(units * 32, IB), IB, 0, st>>>(vld, n, labs, units, dw, ldm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_label_places(const int32_t *vlab, int n, const int32_t *labs, int nlab, int32_t *lidx,
+                                cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_label_places<<<(unsigned)((n + (long long)IB - 1) / IB), IB, 0, st>>>(vlab, n, labs, nlab, lidx);
     return cudaGetLastError();
 }
 

@@ -383,6 +383,10 @@ cudaError_t launch_label_degree_masks(const int2 *vld, int n, const int32_t *lab
 cudaError_t launch_label_nbmax(const int32_t *rowptr, const int32_t *col, const int2 *vld, const int32_t *lidx, int n,
                                int nlab, int32_t *nbmax, cudaStream_t st);
 
+// lidx[v]: v's label's place among the ascending labs[0..nlab), which hold them all.
+cudaError_t launch_label_places(const int32_t *vlab, int n, const int32_t *labs, int nlab, int32_t *lidx,
+                                cudaStream_t st);
+
 // Label runs of one direction (see LabelRuns): run[v * (nlab + 1) + l], col, elab and degrees
 // grouped by the label index lidx[] of the neighbour; *maxrun is raised to the longest run.
 cudaError_t launch_label_runs(const int32_t *rowptr, const int32_t *col, const int32_t *elab, const int2 *vld,
