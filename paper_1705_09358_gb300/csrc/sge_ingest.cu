@@ -251,17 +251,53 @@ __global__ void __launch_bounds__(IB) k_label_places(const int32_t *vlab, int n,
 // ascending within a label -- a counting sort whose counters are the vertex's own slots of
 // the run table: count, scan to the runs' ends, then place the row from its last entry
 // back, each slot counting down to its run's start.  Bound by the row's reads and the
-// serial 32-entry steps of the longest row (a 1,256-neighbour hub: 40 steps twice).
+// serial 32-entry steps of the longest row (a 1,256-neighbour hub: 40 steps twice).  A row of at
+// most 32 entries stays in registers: an entry's place is the number of entries before it in label
+// order, and a run starts where a search among the sorted labels says.  Short rows are bound by
+// their 460 instructions and the chain row, neighbour, label (100,000 directed vertices of 16 arcs,
+// 64 labels, one direction: 85 us by the slots, 75 in registers; 300,000 of 8, 200 labels: 278 -> 217).
 __global__ void __launch_bounds__(IB) k_label_runs(const int32_t *rowptr, const int32_t *col, const int32_t *elab,
                                                    const int2 *vld, const int32_t *lidx, int n, int nlab, int32_t *run,
                                                    int2 *rcol, int32_t *relab, int32_t *maxrun) {
     const int lane = threadIdx.x & 31;
     const long long w0 = (blockIdx.x * (long long)IB + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * IB) >> 5;
+    __shared__ int sorted[IB];   // per warp: a short row's label indices in order
+    int *const mine = sorted + (threadIdx.x & ~31);
     int longest = 0;
     for (long long v = w0; v < n; v += nw) {
         volatile int32_t *slot = run + (size_t)v * (nlab + 1);
         const int b = rowptr[v], e = rowptr[v + 1];
+        if (e - b <= 32) {
+            const int len = e - b;
+            const int y = lane < len ? col[b + lane] : -1;
+            const int l = y >= 0 ? lidx[y] : -1;
+            const int deg = y >= 0 ? vld[y].y : 0, el = y >= 0 ? elab[b + lane] : 0;
+            int rank = 0, same = 0;
+#pragma unroll 4
+            for (int i = 0; i < len; ++i) {
+                const int li = __shfl_sync(FULLMASK, l, i);
+                rank += li < l || (li == l && i < lane) ? 1 : 0;
+                same += li == l ? 1 : 0;
+            }
+            if (y >= 0) {
+                longest = max(longest, same);
+                rcol[b + rank] = make_int2(y, deg);
+                relab[b + rank] = el;
+                mine[rank] = l;
+            }
+            __syncwarp();
+            for (int s = lane; s <= nlab; s += 32) {   // the first entry of label index s or above
+                int lo = 0;
+#pragma unroll
+                for (int h = 16; h >= 1; h >>= 1)
+                    if (lo + h <= len && mine[lo + h - 1] < s) lo += h;
+                if (lo < len && mine[lo] < s) ++lo;
+                run[(size_t)v * (nlab + 1) + s] = b + lo;
+            }
+            __syncwarp();
+            continue;
+        }
         for (int l = lane; l <= nlab; l += 32) slot[l] = l == nlab ? e : 0;
         __syncwarp();
         for (int x0 = b; x0 < e; x0 += 32) {
