@@ -359,7 +359,9 @@ __device__ __forceinline__ int run_drop(const V &v, const PosV &p, const Cand &S
 
 // The candidate list of position P of a node with images M[0..], found by a group of G lanes (a
 // power of two; every lane of the warp calls, `sub` its lane within the group): the group's lanes
-// look up the constraints' runs side by side, then agree on the shortest and the next.
+// look up the constraints' runs side by side, then agree on the shortest and the next.  With fewer
+// constraints than lanes the group works as several smaller ones doing the same (most positions
+// have one to three; agreeing among 32 lanes costs five rounds of shuffles, with one constraint none).
 template <bool DIR, class V>
 __device__ __forceinline__ Cand pick_group(const V &v, const PosV &p, const PosInfo *P, const int *M, int G, int sub) {
     Cand S = plain_list<DIR>(v, p, P, M);
@@ -368,11 +370,15 @@ __device__ __forceinline__ Cand pick_group(const V &v, const PosV &p, const PosI
     constexpr unsigned long long NONE = ~0ull;
     unsigned long long k1 = NONE, k2 = NONE;   // (length, constraint) of the shortest and next run
     int b1 = 0;
+    // (the warp's groups shuffle together: as many lanes as the one with most constraints needs)
+    int most = runs ? p.bc : 0;
+    if (G < 32) most = (int)__reduce_max_sync(FULL, (unsigned)most);
+    if (G > 1 && most + 1 < G) G = most == 0 ? 1 : 2 << (31 - __clz(most));
     if (runs) {
         S.li = v.plidx()[p.pv];
         if (S.li >= 0) {
 #pragma unroll 4
-            for (int q = sub; q <= p.bc; q += G) {
+            for (int q = sub & (G - 1); q <= p.bc; q += G) {
                 int len;
                 const int b = run_of<DIR>(v, R, p, q, S.li, M, len);
                 const unsigned long long k = (unsigned long long)len << 32 | (unsigned)q;
