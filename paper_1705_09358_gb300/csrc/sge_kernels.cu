@@ -373,7 +373,19 @@ __device__ __forceinline__ Cand pick_group(const V &v, const PosV &p, const PosI
     // (the warp's groups shuffle together: as many lanes as the one with most constraints needs)
     int most = runs ? p.bc : 0;
     if (G < 32) most = (int)__reduce_max_sync(FULL, (unsigned)most);
-    if (G > 1 && most + 1 < G) G = most == 0 ? 1 : 2 << (31 - __clz(most));
+    if (most == 0) {   // the parent's run, if any
+        if (runs) {
+            S.li = v.plidx()[p.pv];
+            S.len = 0;
+            if (S.li >= 0) {
+                int len;
+                const int b = run_of<DIR>(v, R, p, 0, S.li, M, len);
+                set_run<DIR>(v, R, p, M, 0, b, len, S);
+            }
+        }
+        return S;
+    }
+    if (most + 1 < G) G = 2 << (31 - __clz(most));
     if (runs) {
         S.li = v.plidx()[p.pv];
         if (S.li >= 0) {
@@ -3679,10 +3691,13 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
             __syncwarp();
             if (lane == 0) { lv[l].cur = min(cur + 32, end); lv[l].mask = bal; lv[l].cbase = cur; }
             __syncwarp();
+            return bal != 0 || end - cur > 32;   // something is left on the level
         };
         // set up level `l` (positions 0..l-1 assigned), count the node's states -- a range
         // frame counts them if it starts the node, a counted frame not at all -- and, below the
-        // frame's first node, scan its first candidates while the list is at hand
+        // frame's first node, scan its first candidates while the list is at hand.  Returns
+        // whether anything is left on the level: most nodes at the bottom have one chunk, and a
+        // round of the loop to find them done cost as much as some of them.
         auto setup = [&](int l, int beg, int endv, bool in_run) {
             const PosV p = load_pos(B.pos + l);
             const Cand S = pick_warp<DIR>(B, p, B.pos + l, M);
@@ -3705,7 +3720,8 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                 if (S.raw < (1 << 24)) st32 += (unsigned)S.raw;
                 else st += (unsigned long long)S.raw;
             }
-            if (l > d0 && cur < end) scan(l, p, S, cur, end);
+            if (l > d0 && cur < end) return scan(l, p, S, cur, end);
+            return cur < end;
         };
         // candidate of entry e of level l's list
         auto entry = [&](const LvCsr &L, int e) {
@@ -3798,8 +3814,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                 M[lvl] = c;
             }
             __syncwarp();
-            ++lvl;
-            setup(lvl, -1, 0, false);
+            if (setup(lvl + 1, -1, 0, false)) ++lvl;
         }
         if (stopped && C.ckpt != nullptr) {
             // checkpoint, per level: the part of the current chunk from its lowest pending
