@@ -85,3 +85,34 @@ def test_default_cadence_costs_no_more_than_a_wide_one():
     finally:
         sge_unload_pattern(E.h, pid)
         sge_unload_target(E.h, tid)
+
+
+def test_a_search_from_one_frame_spreads_as_fast_as_a_batched_call():
+    """sge_count_noalloc starts from the root alone: sharing that out must not make it several times
+    as long as the batched call on the same kernel from a split of depth 1 (2.5 times when donors
+    handed out two frames in 1,024 iterations)."""
+    from time import perf_counter
+    import torch
+    from paper_1705_09358_gb300 import sge_count_noalloc, sge_unload_pattern, sge_unload_target
+    from test_zz_no_alloc import _device_csr
+    g, p = _target(5, 2001, 40, False), _path(4, False)
+    E = engine()
+    tid, pid = E.load_target(g), E.load_pattern(p)
+    d = _device_csr(g)
+    try:
+        times = {"batched": [], "noalloc": []}
+        for _ in range(12):
+            t0 = perf_counter()
+            want = E.count(tid, pid, kernel=1, split_depth=1)
+            t1 = perf_counter()
+            rc, got = sge_count_noalloc(g.n, d["rowptr"].data_ptr(), d["col"].data_ptr(), d["vlabel"].data_ptr(), 0, p,
+                                        stream=torch.cuda.current_stream())
+            t2 = perf_counter()
+            assert rc == 0 and counters(got) == counters(want)
+            times["batched"].append(t1 - t0)
+            times["noalloc"].append(t2 - t1)
+        best = {k: sorted(t)[len(t) // 4] for k, t in times.items()}
+        assert best["noalloc"] < 2.5 * best["batched"], best
+    finally:
+        sge_unload_pattern(E.h, pid)
+        sge_unload_target(E.h, tid)
