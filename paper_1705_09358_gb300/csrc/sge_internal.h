@@ -262,12 +262,13 @@ cudaError_t launch_domain_fixpoint(const JobDesc *jobs, int njobs, const long lo
 // The same for a few jobs by the whole device, one cooperative launch (see k_domain_coop): at most
 // DOMAIN_COOP_VERTS pattern vertices.  scratch: domain_coop_bytes(), whose first int receives 0, or -2 when the
 // domains hold more than `cap` candidates (then untouched); slots: 3 * cap ints; longest_list: no row (run) is longer; edge_off: per
-// job the first of its pattern arcs (out, then in) among all jobs', nedges.
+// job the first of its pattern arcs (out, then in) among all jobs', nedges; blocks_per_sm: 0 = as many
+// as are of use (the launch starts only when all its blocks have room at once).
 constexpr int DOMAIN_COOP_VERTS = 8192;   // (slot offsets in shared memory)
 size_t domain_coop_bytes(long long nverts, long long nedges);
 cudaError_t launch_domain_coop(const JobDesc *jobs, const long long *vert_off, const int *edge_off, int njobs,
                                long long nverts, long long nedges, int any_fc, int longest_list, void *scratch,
-                               int *slots, long long cap, cudaStream_t st);
+                               int *slots, long long cap, int blocks_per_sm, cudaStream_t st);
 cudaError_t launch_domain_sizes(const JobDesc *jobs, const long long *vert_off, int njobs,
                                 long long nverts, long long *sizes, cudaStream_t st);
 cudaError_t launch_domain_lists(const JobDesc *jobs, const int *task_job, const int *task_vert,

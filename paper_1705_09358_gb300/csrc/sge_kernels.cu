@@ -4568,7 +4568,7 @@ size_t domain_coop_bytes(long long nverts, long long nedges) {
 
 cudaError_t launch_domain_coop(const JobDesc *jobs, const long long *vert_off, const int *edge_off, int njobs,
                                long long nverts, long long nedges, int any_fc, int longest_list, void *scratch,
-                               int *slots, long long cap, cudaStream_t st) {
+                               int *slots, long long cap, int blocks_per_sm, cudaStream_t st) {
     if (nverts <= 0) return cudaSuccess;
     if (nverts > DOMAIN_COOP_VERTS) return cudaErrorInvalidValue;
     DomainCoop D;
@@ -4601,8 +4601,8 @@ cudaError_t launch_domain_coop(const JobDesc *jobs, const long long *vert_off, c
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     void *args[] = {(void *)&D};
-    return cudaLaunchCooperativeKernel((void *)k_domain_coop, dim3(sms * std::min(occ, DOMAIN_COOP_BLOCKS)), dim3(BLOCK),
-                                       args, smem, st);
+    const int per_sm = std::min(occ, blocks_per_sm > 0 ? blocks_per_sm : DOMAIN_COOP_BLOCKS);
+    return cudaLaunchCooperativeKernel((void *)k_domain_coop, dim3(sms * per_sm), dim3(BLOCK), args, smem, st);
 }
 
 cudaError_t launch_domain_sizes(const JobDesc *jobs, const long long *vert_off, int njobs, long long nverts,
