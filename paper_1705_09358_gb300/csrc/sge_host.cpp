@@ -125,6 +125,13 @@ struct BlockCache {
     }
 };
 
+// Testing aid: with SGE_BLOCK_MAX set, device blocks of more bytes than that count as not to be
+// had, so that what a call does without a block can be checked (read when a block is allocated).
+bool block_refused(size_t bytes) {
+    const char *env = std::getenv("SGE_BLOCK_MAX");
+    return env != nullptr && bytes > (size_t)std::atoll(env);
+}
+
 struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
@@ -142,6 +149,7 @@ struct DevBuf {
         if (async) {
             if (nb < cap + cap / 2) nb = cap + cap / 2;
             release();
+            if (block_refused(bytes)) return cudaErrorMemoryAllocation;
             cudaError_t e = cudaMallocAsync(&p, nb, astream);
             if (e != cudaSuccess) {
                 (void)cudaGetLastError();
@@ -153,6 +161,7 @@ struct DevBuf {
             return cudaSuccess;
         }
         release();
+        if (block_refused(bytes)) return cudaErrorMemoryAllocation;
         if (cache) {
             size_t c = 0;
             if (void *q = cache->take(nb, &c)) {
@@ -2619,6 +2628,10 @@ sge_status sge_load_target(sge_ctx *ctx, int32_t n, int64_t m, const int32_t *sr
             at = part[d][2] + pad(cap[d]);
         }
         cudaError_t e = T->runs.ensure((size_t)at * 4);
+        if (e == cudaErrorMemoryAllocation) {   // no room: every kernel runs on the rows as well
+            (void)cudaGetLastError();
+            return cudaSuccess;
+        }
         if (e != cudaSuccess) return e;
         int32_t *b = T->runs.as<int32_t>();
         LabelRuns R;

@@ -1,0 +1,40 @@
+"""Device blocks that a call can do without: when one is not to be had, the call takes its other
+way and gives the same results.  SGE_BLOCK_MAX makes larger blocks count as not to be had."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from gen.graphs import Graph
+from gpu_common import counters, engine
+from test_gpu_label_runs import _graph, _pattern
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("matches", "states", "nodes", "hash")
+
+
+@pytest.fixture
+def fresh():
+    """A context of its own: no block is there from earlier calls."""
+    import paper_1705_09358_gb300 as sge
+    engine()
+    with sge.Context(0) as E:
+        yield E
+
+
+@pytest.mark.parametrize("directed", [False, True])
+def test_target_without_room_for_label_runs(fresh, monkeypatch, directed):
+    g = _graph(7, 2000, 12000, 150, 1, directed, 2 if directed else 0)
+    pats = [_pattern(s, g, 3 + s % 3) for s in range(6)]
+    table = 2000 * 151 * 4                      # the runs' table alone, per direction
+    monkeypatch.setenv("SGE_BLOCK_MAX", str(table + 20_000))
+    tid = fresh.load_target(g)
+    monkeypatch.delenv("SGE_BLOCK_MAX")
+    pids = [fresh.load_pattern(p) for p in pats]
+    for algo in range(4):
+        want = [tuple(oracle.run(g, p, algo)[k] for k in KEYS) for p in pats]
+        for kernel in (0, 1):
+            rc, rows = fresh.count_batch([tid] * len(pids), pids, algo=algo, kernel=kernel)
+            assert [counters(r) for r in rows] == want, (algo, kernel)
