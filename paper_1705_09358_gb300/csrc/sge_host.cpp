@@ -1202,11 +1202,19 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             }
             coop = slots <= COOP_CANDIDATES;
         }
+        if (coop) {   // (without room for its slots the sweeps below do: they list the real candidates only)
+            cudaError_t e = W.vchg.ensure(domain_coop_bytes(nverts, arcs));
+            if (e == cudaSuccess) e = W.cand.ensure((size_t)std::max(slots, 1ll) * 3 * 4);
+            if (e == cudaErrorMemoryAllocation) {
+                (void)cudaGetLastError();
+                coop = false;
+            } else {
+                CK(e, "alloc domain slots");
+            }
+        }
         if (coop) {
             // (a serving group: one block per SM, like its split, so that it starts beside another
             // group's search once that leaves a block's room on each SM, not a whole free device)
-            CK(W.vchg.ensure(domain_coop_bytes(nverts, arcs)), "alloc domain flags");
-            CK(W.cand.ensure((size_t)std::max(slots, 1ll) * 3 * 4), "alloc candidate lists");
             CK(upload(W.deoff, edge_off, st), "upload edge offsets");
             coop = launch_domain_coop(W.fjobs.as<JobDesc>(), W.vert_off.as<long long>(), W.deoff.as<int>(), nf, nverts,
                                       arcs, any_fc ? 1 : 0, longest, W.vchg.p, W.cand.as<int>(), slots, serving ? 1 : 0,

@@ -38,3 +38,30 @@ def test_target_without_room_for_label_runs(fresh, monkeypatch, directed):
         for kernel in (0, 1):
             rc, rows = fresh.count_batch([tid] * len(pids), pids, algo=algo, kernel=kernel)
             assert [counters(r) for r in rows] == want, (algo, kernel)
+
+
+# the largest block that a call below cannot do without, the list of what the split leaves: 36.7 MB
+ROOM = 37_500_000
+
+
+def test_few_pairs_without_room_for_the_domain_slots(fresh, monkeypatch):
+    """12 bytes for every vertex that may carry a pattern vertex's label, here 43 MB: the sweeps,
+    which list the candidates there are, take the call."""
+    n = 20_000
+    g = _graph(11, n, 4 * n, 1)
+    pats = [_pattern(s, g, 3) for s in range(3)]
+    tid, pids = fresh.load_target(g), [fresh.load_pattern(p) for p in pats] * 20
+    assert 12 * n * 3 * len(pids) > ROOM
+    for algo in (1, 3):
+        want = [tuple(oracle.run(g, p, algo)[k] for k in KEYS) for p in pats] * 20
+        launches = {}
+        for room in (ROOM, None):
+            if room:
+                monkeypatch.setenv("SGE_BLOCK_MAX", str(room))
+            else:
+                monkeypatch.delenv("SGE_BLOCK_MAX")
+            rc, rows = fresh.count_batch([tid] * len(pids), pids, algo=algo, tuned=False, frontier_kib=1024)
+            assert [counters(r) for r in rows] == want, (algo, room)
+            launches[room] = int(rows["launches"][0])
+        if algo == 1:   # (the second variant finds the slots' block there)
+            assert launches[ROOM] > launches[None]
