@@ -1796,16 +1796,20 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         SplitAsync async;
         std::memset(&async, 0, sizeof(async));
         if (to_the_end && !o.no_donation && ckpt_frames == nullptr) {
-            async.narrow = resident_warps;
-            async.ctl = wtot + async_at;
-            async.qcap = ASYNC_QUEUE;
-            CK(split_queue_ready(W.aentry, (size_t)ASYNC_QUEUE * 8, W.aleft,
-                                 (size_t)(ASYNC_QUEUE + 64 * wcap + async.narrow) * 8, W.aepoch,
-                                 [&](void *p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st); }),
-               "split queue");
-            async.epoch = W.aepoch;
-            async.entries = W.aentry.as<unsigned long long>();
-            async.left = W.aleft.as<const int32_t *>();
+            const cudaError_t e = split_queue_ready(W.aentry, (size_t)ASYNC_QUEUE * 8, W.aleft,
+                                                    (size_t)(ASYNC_QUEUE + 64 * wcap + resident_warps) * 8, W.aepoch,
+                                                    [&](void *p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st); });
+            if (e == cudaErrorMemoryAllocation) {
+                (void)cudaGetLastError();   // no room: level by level to the end
+            } else {
+                CK(e, "split queue");
+                async.narrow = resident_warps;
+                async.ctl = wtot + async_at;
+                async.qcap = ASYNC_QUEUE;
+                async.epoch = W.aepoch;
+                async.entries = W.aentry.as<unsigned long long>();
+                async.left = W.aleft.as<const int32_t *>();
+            }
         }
         if (!W.ev2) {
             CK(cudaEventCreate(&W.ev2), "event");

@@ -65,3 +65,22 @@ def test_few_pairs_without_room_for_the_domain_slots(fresh, monkeypatch):
             launches[room] = int(rows["launches"][0])
         if algo == 1:   # (the second variant finds the slots' block there)
             assert launches[ROOM] > launches[None]
+
+
+def test_split_without_room_for_its_queue(fresh, monkeypatch):
+    """The levels then go on to the end one by one; the call after it has the queue again."""
+    from test_gpu_split_async import _broom, _pattern as _handle
+    handles = [2, 17, 60, 125]
+    g = _broom(handles, 30)
+    starts = np.cumsum([0] + [h + 90 for h in handles[:-1]])
+    pats = [_handle(g, h, int(s)) for h, s in zip(handles, starts)]
+    tid, pids = fresh.load_target(g), [fresh.load_pattern(p) for p in pats]
+    want = [tuple(oracle.run(g, p, 0)[k] for k in KEYS) for p in pats] * 5
+    for room in (ROOM // 2, None, ROOM // 2, None):   # (18.7 MB: the entries fit, the list does not)
+        if room:
+            monkeypatch.setenv("SGE_BLOCK_MAX", str(room))
+        else:
+            monkeypatch.delenv("SGE_BLOCK_MAX")
+        for kib in (1024, 16):
+            rc, rows = fresh.count_batch([tid] * 20, pids * 5, kernel=1, frontier_kib=kib)
+            assert [counters(r) for r in rows] == want, (room, kib)
