@@ -52,7 +52,8 @@ constexpr int POOL_CELLS = 1 << 15;
 // 59.7 / 38.6 / 25.6 / 18.6 / 17.2 / 18.7, paths of 5 on a sparse one from 20,000 frames
 // 20.6 / 16.1 / 12.5 / 10.9 / 10.8 / 11.7.
 constexpr int CSR_DONATE_ITERS = 16;
-constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call
+constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call ...
+constexpr int ASYNC_INTS_PER_ENTRY = 64;         // ... and no more than one per this many ints of its arena
 constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
 constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
@@ -1796,8 +1797,9 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         SplitAsync async;
         std::memset(&async, 0, sizeof(async));
         if (to_the_end && !o.no_donation && ckpt_frames == nullptr) {
-            const cudaError_t e = split_queue_ready(W.aentry, (size_t)ASYNC_QUEUE * 8, W.aleft,
-                                                    (size_t)(ASYNC_QUEUE + 64 * wcap + resident_warps) * 8, W.aepoch,
+            const long long qcap = std::min(ASYNC_QUEUE, std::max(1ll, cap_ints / ASYNC_INTS_PER_ENTRY));
+            const cudaError_t e = split_queue_ready(W.aentry, (size_t)qcap * 8, W.aleft,
+                                                    (size_t)(qcap + 64 * wcap + resident_warps) * 8, W.aepoch,
                                                     [&](void *p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st); });
             if (e == cudaErrorMemoryAllocation) {
                 (void)cudaGetLastError();   // no room: level by level to the end
@@ -1805,7 +1807,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                 CK(e, "split queue");
                 async.narrow = resident_warps;
                 async.ctl = wtot + async_at;
-                async.qcap = ASYNC_QUEUE;
+                async.qcap = qcap;
                 async.epoch = W.aepoch;
                 async.entries = W.aentry.as<unsigned long long>();
                 async.left = W.aleft.as<const int32_t *>();
@@ -1850,6 +1852,13 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             if (trace_on()) {
                 std::fprintf(stderr, "[sge] device split: %d levels, %lld frames at %.3f ms\n", depth, F,
                              now_ms() - t_start);
+                if (listed) {
+                    unsigned long long pushed = 0, top = 0;
+                    CK(cudaMemcpy(&pushed, static_cast<char *>(async.ctl) + 128, 8, cudaMemcpyDeviceToHost), "read trace");
+                    CK(cudaMemcpy(&top, static_cast<char *>(async.ctl) + 3 * 128, 8, cudaMemcpyDeviceToHost), "read trace");
+                    std::fprintf(stderr, "[sge]   without barriers: %llu frames queued (room for %lld), %llu of %lld ints\n",
+                                 pushed, async.qcap, top, cap_ints);
+                }
                 if (!ordered) {
                     // per level: end time, children, longest candidate list of one frame
                     std::vector<long long> tr((size_t)2 * KMAX), lv((size_t)std::max(depth, 1));
