@@ -42,6 +42,7 @@ constexpr int HUB_MIN_DEGREE = 24;               // larger targets: bitset rows 
 constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device memory
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
 constexpr long long LIST_FIRST_ROWS = 1 << 16;   // matches a listing call has room for at first
+constexpr size_t LIST_KEEP_BYTES = size_t(256) << 20;   // sorting scratch a workspace keeps from call to call
 constexpr int LEAN_MIN_PAIRS = 4096;             // plain RI batches from this many pairs: records built on the device
 constexpr int POOL_CELLS = 1 << 15;
 // Iterations of the CSR search from one look for idle warps to the next.  A look reads two words
@@ -892,6 +893,21 @@ float span_ms(unsigned long long inv_start, unsigned long long end) {
     if (inv_start == 0 || end == 0) return 0.f;
     const unsigned long long start = ~inv_start;
     return end > start ? (float)((double)(end - start) * 1e-6) : 0.f;
+}
+
+// Rows of k ints in ascending order.
+void sort_rows(std::vector<int32_t> &rows, int k) {
+    const size_t n = rows.size() / (size_t)k;
+    std::vector<size_t> order(n);
+    for (size_t i = 0; i < n; ++i) order[i] = i * (size_t)k;
+    std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+        return std::lexicographical_compare(rows.begin() + (long)a, rows.begin() + (long)a + k, rows.begin() + (long)b,
+                                            rows.begin() + (long)b + k);
+    });
+    std::vector<int32_t> sorted(rows.size());
+    for (size_t i = 0; i < n; ++i)
+        std::copy_n(rows.begin() + (long)order[i], k, sorted.begin() + (long)(i * (size_t)k));
+    rows.swap(sorted);
 }
 
 // Run a homogeneous group of pairs (same directedness) through the whole
@@ -2144,14 +2160,27 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
         if (rows > match_cap) return SGE_OK;   // (the caller comes again with room for them)
         match_rows->resize((size_t)rows * k);
         if (rows > 0) {
+            const size_t bytes = (size_t)rows * k * 4;
+            cudaError_t e = W.msort.ensure(match_sort_bytes(rows));
+            if (e == cudaSuccess) e = W.mout.ensure(bytes);
+            const bool device_sort = e == cudaSuccess;
+            if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();   // no room: sorted on the host
+            else CK(e, "alloc match order");
             int sorting = 0;
-            CK(W.msort.ensure(match_sort_bytes(rows)), "alloc match order");
-            CK(W.mout.ensure((size_t)rows * k * 4), "alloc sorted matches");
-            CK(launch_match_sort(W.mbuf.as<int32_t>(), rows, k, W.msort.p, W.mout.as<int32_t>(), &sorting, st), "sort matches");
-            out[jobs[0].pair].launches += sorting;
-            CK(cudaMemcpyAsync(match_rows->data(), W.mout.p, (size_t)rows * k * 4, cudaMemcpyDeviceToHost, st),
+            if (device_sort) {
+                CK(launch_match_sort(W.mbuf.as<int32_t>(), rows, k, W.msort.p, W.mout.as<int32_t>(), &sorting, st),
+                   "sort matches");
+                out[jobs[0].pair].launches += sorting;
+            }
+            CK(cudaMemcpyAsync(match_rows->data(), (device_sort ? W.mout : W.mbuf).p, bytes, cudaMemcpyDeviceToHost, st),
                "read matches");
             CK(cudaStreamSynchronize(st), "read matches");
+            if (!device_sort) sort_rows(*match_rows, k);
+            // (scratch of an ordinary list stays; a long one's, up to 17 GB, goes back)
+            if (W.msort.cap + W.mout.cap > LIST_KEEP_BYTES) {
+                W.msort.release();
+                W.mout.release();
+            }
         }
     }
     if (status != 0) {

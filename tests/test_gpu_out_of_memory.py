@@ -84,3 +84,27 @@ def test_split_without_room_for_its_queue(fresh, monkeypatch):
         for kib in (1024, 16):
             rc, rows = fresh.count_batch([tid] * 20, pids * 5, kernel=1, frontier_kib=kib)
             assert [counters(r) for r in rows] == want, (room, kib)
+
+
+def test_listing_without_room_to_sort_on_the_device(fresh, monkeypatch):
+    """24 bytes a match to sort, 38.4 MB here, against 8 to list: then the host sorts."""
+    n, m = 50_000, 800_000
+    r = np.random.default_rng(2)
+    key = np.unique(r.integers(0, n, 3 * m) * n + r.integers(0, n, 3 * m))
+    src, dst = key // n, key % n
+    keep = r.permutation(np.flatnonzero(src < dst))[:m]
+    g = Graph(n, src[keep].astype(np.int32), dst[keep].astype(np.int32), np.zeros(n, np.int32), None, False)
+    edge = Graph(2, np.array([0], np.int32), np.array([1], np.int32), np.zeros(2, np.int32), None, False)
+    tid, pid = fresh.load_target(g), fresh.load_pattern(edge)
+    both = np.concatenate([np.stack([g.src, g.dst], 1), np.stack([g.dst, g.src], 1)])
+    want = both[np.lexsort((both[:, 1], both[:, 0]))]
+    launches = {}
+    for room in (ROOM, None, None):
+        if room:
+            monkeypatch.setenv("SGE_BLOCK_MAX", str(room))
+        else:
+            monkeypatch.delenv("SGE_BLOCK_MAX", raising=False)
+        got = fresh.enumerate(tid, pid, frontier_kib=4096)
+        assert got["matches"] == 2 * m and np.array_equal(got["match_list"], want)
+        launches[room] = got["launches"]
+    assert launches[ROOM] < launches[None]
