@@ -3335,6 +3335,7 @@ struct Frame {
     int job, depth, beg, end;
     bool counted;   // FRAME_COUNTED: the range's accepted nodes and states are already counted
     bool in_run;    // FRAME_RUN: the range counts in the node's label run
+    bool queued;    // it came from another warp
 };
 
 // Optional per-warp timing, kept in the warp's own trace record (no registers):
@@ -3490,6 +3491,7 @@ __device__ bool acquire_frame(const SearchCtl &C, int *M, Frame &fr, unsigned lo
     const int dw = src[1];
     fr.job = src[0]; fr.depth = dw & FRAME_DEPTH_MASK; fr.counted = (dw & FRAME_COUNTED) != 0;
     fr.in_run = (dw & FRAME_RUN) != 0;
+    fr.queued = kind == 2;
     fr.beg = src[2]; fr.end = src[3];
     for (int i = lane; i < fr.depth; i += 32) M[i] = src[FRAME_HDR + i];
     __syncwarp();
@@ -3669,6 +3671,10 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
         // candidate list below 2^24 states (longer lists go straight to the 64-bit total)
         unsigned st32 = 0, nd32 = 0, mt32 = 0;
         bool counts0 = true;   // the frame counted its first node's states
+        // a frame of the frontier (or a part of one) that starts on the last level but one has nothing
+        // shallower to give: halves of its range, if that is long, have one level below them (a path of
+        // 3 on a 100,000-vertex network of 2 labels, from depth 1: 25 ms on one hub's frame -> 3.6)
+        const bool last_but_one = d0 + 2 == k && (!fr.queued || fr.beg >= 0);
         // scan the next 32 candidates [cur, ..) of level `l`'s list
         auto scan = [&](int l, const PosV &p, const Cand &S, int cur, int end) {
             int c;
@@ -3759,7 +3765,8 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                 want = __shfl_sync(FULL, want, 0);
                 // donate the shallowest unexplored work: half of an unscanned range, else up to
                 // `gran` pending survivors as new search nodes
-                for (int l = d0; want > 0 && l <= lvl && l + 1 + DONATE_MIN_LEVELS <= k; ++l) {
+                const int levels = last_but_one ? 1 : DONATE_MIN_LEVELS;
+                for (int l = d0; want > 0 && l <= lvl && l + 1 + levels <= k; ++l) {
                     LvCsr &L = lv[l];
                     int rem = L.end - L.cur;
                     if (rem >= 64 && L.kind >= LIST_RUN) {   // past the entries no part may start in
@@ -3780,6 +3787,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_search_csr(const JobDesc *jobs, Se
                         }
                         break;
                     }
+                    if (last_but_one) break;   // (no single nodes)
                     const unsigned m = L.mask;
                     // (the current level keeps one for this warp, which would else be out of work)
                     const int most = min(min(want, C.gran), __popc(m) - (l == lvl ? 1 : 0));

@@ -116,3 +116,36 @@ def test_a_search_from_one_frame_spreads_as_fast_as_a_batched_call():
     finally:
         sge_unload_pattern(E.h, pid)
         sge_unload_target(E.h, tid)
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("hub", [63, 64, 65, 500, 1500])
+def test_a_hub_with_one_level_below_is_shared(hub, directed):
+    """Frames that start on the last position but one: the range of a long one is handed out in
+    halves (nothing was, and one warp searched below a hub alone)."""
+    from paper_1705_09358_gb300 import sge_unload_pattern, sge_unload_target
+    n = hub + 200
+    r = np.random.default_rng(hub)
+    # vertex 0 to `hub` others, which form a dense graph with the rest
+    a, b = r.integers(1, n, 40 * n), r.integers(1, n, 40 * n)
+    key = np.unique((np.minimum(a, b).astype(np.int64) * n + np.maximum(a, b))[a != b])
+    key = np.concatenate([np.arange(1, hub + 1, dtype=np.int64), key])
+    lab = np.zeros(n, np.int32)
+    lab[0] = 1
+    g = Graph(n, (key // n).astype(np.int32), (key % n).astype(np.int32), lab, None, directed)
+    p = Graph(3, np.array([0, 0], np.int32), np.array([1, 2], np.int32), np.array([1, 0, 0], np.int32), None, directed)
+    E = engine()
+    tid, pid = E.load_target(g), E.load_pattern(p)
+    try:
+        for algo in (0, 1):
+            want = tuple(oracle.run(g, p, algo)[key] for key in ("matches", "states", "nodes", "hash"))
+            for copies in (1, 5):
+                given = 0
+                for opts in ({"split_depth": 1}, {"split_depth": 1, "donate_every_iters": 1}, {"state_budget": 1 << 60}):
+                    rc, rows = E.count_batch([tid] * copies, [pid] * copies, algo=algo, kernel=1, tuned=False, **opts)
+                    assert [counters(x) for x in rows] == [want] * copies, (algo, opts)
+                    given += int(rows["donations"][0])
+                assert hub < 500 or given > 0, (algo, copies)
+    finally:
+        sge_unload_pattern(E.h, pid)
+        sge_unload_target(E.h, tid)
