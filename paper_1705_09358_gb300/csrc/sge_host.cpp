@@ -1632,6 +1632,7 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
                     longl = P.par < 0 && ((D.flags & JOB_RIDS) ? (long long)P.ucnt : jobs[q].t->n) > SPLIT_RANGE;
                 }
                 if (longl) D.flags |= JOB_LONG_LISTS;
+                if (T.cached.runs && T.maxrun > SPLIT_RANGE) D.flags |= JOB_LONG_LAST;
             }
             D.ulist = W.ulist.as<int32_t>();
             if (enumerate) {

@@ -46,12 +46,19 @@ constexpr int JOB_FC = 8;            // forward checking of singleton domains
 // AC_ENT_DENSE marks a vertex whose pattern neighbours' domains are all dense (see k_domain_ac_cand)
 constexpr int AC_ENT_DENSE = 1 << 16;
 constexpr int AC_DENSE = 8;           // dense: a domain holding at least 1/AC_DENSE of the target
-constexpr int JOB_LONG_LISTS = 16;   // some position after the first may have more than SPLIT_RANGE candidates
+constexpr int JOB_LONG_LISTS = 16;   // some position after the first may have more candidates than one frame takes
+constexpr int JOB_LONG_LAST = 32;    // the last position may (label runs are cut finer there)
 
 // The breadth-first split writes a child whose candidate list is longer than
 // this as range frames of this many candidates each.
 constexpr int SPLIT_RANGE = 256;
-constexpr int SPLIT_RUN_RANGE = 1024;   // ... or as this many entries of a label run
+// ... or as this many entries of a label run, which all hold the right label and mostly pass:
+// finer parts cost more in child frames and repeated look-ups than they balance (160 queries on a
+// 100,000-vertex network 3.43 ms, with 512 3.52, with 256 3.76).  On the last position a frame has
+// no children, and a level there lasts as long as the warp with most candidates: with barriers
+// SPLIT_RANGE holds there (a path of 3 on a 100,000-vertex network of 2 labels, 100 million states:
+// 4.7 ms with 1,024 there, 3.0 with 256).
+constexpr int SPLIT_RUN_RANGE = 1024;
 
 // One search position i of a job: pattern vertex mu_i and its constraints.
 struct PosInfo {

@@ -2341,23 +2341,25 @@ __global__ void __launch_bounds__(BLOCK) k_split_coop(const JobDesc *jobs, long 
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long *>(S.result + 7), globaltimer());
 }
 
-// Frames a child of `depth` images plus c takes: one, or one per SPLIT_RANGE candidates
-// of its list when that is longer (JOB_LONG_LISTS pairs only).
-template <bool DIR>
-__device__ __forceinline__ int split_child_frames(const JobDesc &J, int depth, int c, const int *M) {
-    if (!(J.flags & JOB_LONG_LISTS)) return 1;
+// Frames a child of `depth` images plus c takes: one, or one per `range` entries of its list when
+// that is longer (JOB_LONG_LISTS pairs; where the next level is a whole one, LEVELS, and the last,
+// JOB_LONG_LAST ones too).
+template <bool DIR, bool LEVELS>
+__device__ __forceinline__ int split_child_frames(const JobDesc &J, int depth, int c, const int *M, int &range) {
+    range = SPLIT_RANGE;
+    const bool fine = LEVELS && depth + 2 == J.k;
+    if (!(J.flags & (fine ? JOB_LONG_LISTS | JOB_LONG_LAST : JOB_LONG_LISTS))) return 1;
     const PosInfo *Q = J.pos + depth + 1;
     const PosV q = load_pos(Q);
     long long len;
-    int range = SPLIT_RANGE;
     if (q.par >= 0) {
         if (J.t.maxdeg != 0 && J.t.maxdeg <= SPLIT_RANGE) return 1;
         const LabelRuns *R = J.t.runs;
         const JobRef v{&J};
         const int li = R ? J.plidx[q.pv] : -1;
         if (R && li < 0) return 1;
-        // the shortest constraint's list, as pick_lane will find it; any short one settles it
-        if (R) range = SPLIT_RUN_RANGE;
+        // the shortest constraint's list, as pick_group will find it; any short one settles it
+        if (R && !fine) range = SPLIT_RUN_RANGE;
         len = 0x7fffffff;
         for (int x = 0; x <= (R ? q.bc : 0); ++x) {
             int pos = q.par, in = DIR ? q.flags & POS_IN_ROW : 0;
@@ -2378,12 +2380,12 @@ __device__ __forceinline__ int split_child_frames(const JobDesc &J, int depth, i
     return (int)((len + range - 1) / range);
 }
 
-// Header words of range q of r of a child frame.
-__device__ __forceinline__ void split_child_header(int32_t *dst, const JobDesc &J, int j, int depth, int r, int q) {
+// Header words of part q of r, of `range` entries each, of a child frame.
+__device__ __forceinline__ void split_child_header(int32_t *dst, const JobDesc &J, int j, int depth, int r, int q,
+                                                   int range) {
     const bool run = r > 1 && J.t.runs != nullptr && J.pos[depth].par >= 0;   // (its range counts in a run)
     dst[0] = j;
     dst[1] = depth | (run ? FRAME_RUN : 0);
-    const int range = run ? SPLIT_RUN_RANGE : SPLIT_RANGE;
     dst[2] = r == 1 ? -1 : q * range;
     dst[3] = r == 1 ? -1 : (q + 1 == r ? 0x7fffffff : (q + 1) * range);
 }
@@ -2426,6 +2428,7 @@ struct SplitWarp {   // one warp's shared memory: the batch's frames, then its w
 // counter.  A reservation that ends past `cap_frames` raises `full` and writes nothing (the
 // level is then abandoned, see k_split_once).
 struct LevelOut {
+    static constexpr bool LEVELS = true;
     const int32_t *fin;
     long long f0;
     int sin;
@@ -2516,7 +2519,8 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, int depth, O &
     }
     // frames per child: one, or one per part of a long list, so that no warp of the next level
     // scans a hub's whole row while the others wait at the barrier
-    const int r = ok && !leaf ? split_child_frames<DIR>(J, depth, c, Mg) : 0;
+    int range = 0;
+    const int r = ok && !leaf ? split_child_frames<DIR, O::LEVELS>(J, depth, c, Mg, range) : 0;
     int incl = r;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -2530,7 +2534,7 @@ __device__ __forceinline__ void split_accept(const JobDesc *jobs, int depth, O &
     const bool coop = depth >= SPLIT_COOP_DEPTH;
     for (int q = 0; q < r; ++q) {
         int32_t *dst = to + (long long)(incl - r + q) * sout;
-        split_child_header(dst, J, W.job[L], depth + 1, r, q);
+        split_child_header(dst, J, W.job[L], depth + 1, r, q, range);
         for (int t = 0; t < depth && !coop; ++t) dst[FRAME_HDR + t] = Mg[t];
         dst[FRAME_HDR + depth] = c;
     }
@@ -2803,6 +2807,7 @@ constexpr int ASYNC_SEGS = 8;       // pieces of the arena one batch's children 
 constexpr unsigned long long ASYNC_OFFSET = (1ull << 40) - 1;
 
 struct AsyncOut {
+    static constexpr bool LEVELS = false;
     const SplitCtl &S;
     int32_t *arena;
     long long chunk;                 // ints taken at once
