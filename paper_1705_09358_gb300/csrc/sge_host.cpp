@@ -895,8 +895,18 @@ float span_ms(unsigned long long inv_start, unsigned long long end) {
     return end > start ? (float)((double)(end - start) * 1e-6) : 0.f;
 }
 
+// Listed matches on their way to the caller: ints that a copy from the device fills (clearing
+// them first took a pass over the list, fresh pages and all).
+template <class T>
+struct Unfilled : std::allocator<T> {
+    template <class U> struct rebind { using other = Unfilled<U>; };
+    template <class U> void construct(U *p) { ::new (static_cast<void *>(p)) U; }
+    template <class U, class... A> void construct(U *p, A &&...a) { ::new (static_cast<void *>(p)) U(std::forward<A>(a)...); }
+};
+using MatchRows = std::vector<int32_t, Unfilled<int32_t>>;
+
 // Rows of k ints in ascending order.
-void sort_rows(std::vector<int32_t> &rows, int k) {
+void sort_rows(MatchRows &rows, int k) {
     const size_t n = rows.size() / (size_t)k;
     std::vector<size_t> order(n);
     for (size_t i = 0; i < n; ++i) order[i] = i * (size_t)k;
@@ -904,7 +914,7 @@ void sort_rows(std::vector<int32_t> &rows, int k) {
         return std::lexicographical_compare(rows.begin() + (long)a, rows.begin() + (long)a + k, rows.begin() + (long)b,
                                             rows.begin() + (long)b + k);
     });
-    std::vector<int32_t> sorted(rows.size());
+    MatchRows sorted(rows.size());
     for (size_t i = 0; i < n; ++i)
         std::copy_n(rows.begin() + (long)order[i], k, sorted.begin() + (long)(i * (size_t)k));
     rows.swap(sorted);
@@ -921,7 +931,7 @@ struct Resume {
 
 sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vector<PairReq> &reqs,
                      const std::vector<int> &idx, const sge_opts &o, sge_result *out, bool enumerate,
-                     std::vector<int32_t> *match_rows, long long match_cap, bool serving,
+                     MatchRows *match_rows, long long match_cap, bool serving,
                      const Resume *resume = nullptr, std::vector<int32_t> *ckpt_frames = nullptr,
                      int *ckpt_kmax = nullptr) {
     const double t_start = now_ms();
@@ -2257,7 +2267,7 @@ sge_status prepare_pairs(sge_ctx *ctx, std::vector<PairReq> &reqs, const sge_opt
 }
 
 sge_status run_pairs(sge_ctx *ctx, Workspace &W, cudaStream_t st, std::vector<PairReq> &reqs,
-                     const sge_opts *opts, sge_result *out, bool enumerate, std::vector<int32_t> *rows,
+                     const sge_opts *opts, sge_result *out, bool enumerate, MatchRows *rows,
                      long long cap, bool serving = false) {
     sge_opts o;
     std::vector<int> und, dir;
@@ -3020,7 +3030,7 @@ sge_status sge_enumerate(sge_ctx *ctx, int32_t target_id, int32_t pattern_id, co
     std::vector<PairReq> reqs{{target_id, pattern_id}};
     // list into a buffer of a usual size; when there are more matches (the run has counted them
     // all the same) again into one that holds them
-    std::vector<int32_t> rows;
+    MatchRows rows;
     long long cap = LIST_FIRST_ROWS;
     sge_status rc = run_pairs(ctx, ctx->ws, ctx->stream, reqs, opts, out, true, &rows, cap);
     if (rc != SGE_OK) return rc;
