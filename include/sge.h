@@ -92,8 +92,11 @@ typedef struct {
                                   of one launch (targets of at most 16384 vertices: word by word;
                                   larger ones: over candidate lists); 0 = auto: on targets of at
                                   most 16384 vertices word-by-word blocks from half as many RI-DS
-                                  pairs as the device has SMs, candidate-list blocks from 32 pairs,
-                                  else sweeps; on larger targets candidate-list blocks always.
+                                  pairs as the device has SMs, from eight per SM a warp per pair
+                                  where patterns have at most 64 and targets at most 512 vertices;
+                                  fewer pairs, and larger targets, the whole device in one
+                                  cooperative launch (up to 8192 pattern vertices a call); beyond,
+                                  candidate-list blocks (small targets below 32 pairs: sweeps).
                                   All reach the same fixpoint. */
     int32_t frontier_kib;      /* size of each of the breadth-first split's two frontier buffers
                                   in KiB (default 524288 = 512 MiB); a split level whose children

@@ -41,9 +41,14 @@ constexpr int BITSET_MAX_N = 16384;              // adjacency bitset kept for n 
 constexpr int HUB_MIN_DEGREE = 24;               // larger targets: bitset rows for vertices of this degree+
 constexpr long long HUB_BYTES = 512ll << 20;     // ... within this much device memory
 constexpr long long FRONTIER_MAX_INTS = 1ll << 27;  // 512 MB per frontier buffer
-constexpr long long LIST_FIRST_ROWS = 1 << 16;   // matches a listing call has room for at first
+// Matches a listing call has room for at first: most lists are shorter (1.5 MB of 6 vertices), and a
+// longer one needs no more passes than the count and the list it took when the count came first.
+constexpr long long LIST_FIRST_ROWS = 1 << 16;
 constexpr size_t LIST_KEEP_BYTES = size_t(256) << 20;   // sorting scratch a workspace keeps from call to call
-constexpr int LEAN_MIN_PAIRS = 4096;             // plain RI batches from this many pairs: records built on the device
+// Plain RI batches from this many pairs have their records built on the device: at 4,096 molecule pairs
+// 0.80 ms a call against 1.08 with host records, at 16,384 1.39 and 2.29 (at 1,024 already 0.67 and
+// 0.79, at 256 0.59 and 0.66: the line could lie lower).
+constexpr int LEAN_MIN_PAIRS = 4096;
 constexpr int POOL_CELLS = 1 << 15;
 // Iterations of the CSR search from one look for idle warps to the next.  A look reads two words
 // that every warp shares, an L2 round trip that the next iteration waits for; without it idle
@@ -55,16 +60,17 @@ constexpr int POOL_CELLS = 1 << 15;
 constexpr int CSR_DONATE_ITERS = 16;
 constexpr long long ASYNC_QUEUE = 1ll << 21;     // frames the split's asynchronous end may queue in one call ...
 constexpr int ASYNC_INTS_PER_ENTRY = 64;         // ... and no more than one per this many ints of its arena
-constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint
+constexpr long long COOP_CANDIDATES = 1ll << 25;  // most candidate slots of the whole-device domain fixpoint (402 MB)
 constexpr long long CAND_MAX = 1ll << 28;   // most listed domain candidates per launch group (1 GiB)
 constexpr int ROOT_CHUNK = 1024;                 // most root candidates per root range frame
 constexpr int BLOCK_FIXPOINT_MAX_N = 16384;      // auto domain mode: in-block fixpoint for targets up to this
 constexpr int LABELS_PER_THREAD = 16384;         // a load's label pass: fewest vertices worth another thread
 constexpr long long LABEL_TABLE_MAX = 1ll << 26; // most (vertex, label) entries of a target's degree table
 constexpr int WARP_FIXPOINT_MIN_JOBS = 8;        // auto domain mode: a warp per pair from this many pairs per SM
-constexpr int LIST_FIXPOINT_MIN_JOBS = 32;      // auto domain mode, small targets: in-block fixpoint over lists from
-                                                 // this many pairs (large targets: always; on the 100k-vertex target it
-                                                 // beat the sweeps from 1 to 32 pairs)
+constexpr int LIST_FIXPOINT_MIN_JOBS = 32;      // auto domain mode, calls that the whole-device fixpoint does not take,
+                                                 // small targets: in-block fixpoint over lists from this many pairs (large
+                                                 // targets: always; on the 100k-vertex target it beat the sweeps from 1 to
+                                                 // 32 pairs)
 
 // Opt-in phase trace on stderr (SGE_TRACE=1): sizes and timings of each launch group.
 // SGE_TRACE: unset or "0" off; "errors" prints only failures; anything else
@@ -1187,9 +1193,9 @@ sge_status run_group(sge_ctx *ctx, Workspace &W, cudaStream_t st, const std::vec
             any_rids = any_rids || jobs[q].algo != SGE_RI;
             any_fc = any_fc || jobs[q].algo == SGE_RIDS_SI_FC;
         }
-        // RI-DS jobs in the batch; with many of them (or on request) the whole
-        // fixpoint of each job runs inside one block of one launch, else under the host loop
-        // below, whose sweeps spread one job's candidates over the whole device
+        // RI-DS jobs in the batch; a few of them take the whole device in one launch; with many (or
+        // on request) the whole fixpoint of each job runs inside one block (or warp) of one launch;
+        // else under the host loop below, whose sweeps spread one job's candidates over the device
         // (on small targets the blocks scan domains word by word; large targets' domains are
         // mostly empty words, so there the blocks walk candidate lists, built first, below)
         // (SGE_DOMAIN_WORDS=1 forces the word sweeps, which otherwise serve only lists beyond CAND_MAX)

@@ -192,7 +192,7 @@ struct SearchCtl {
     int *idle;                  // warps waiting for work
     int *status;                // first error code (0 = ok)
     unsigned long long *donations;
-    int *promised;              // donations decided on but not yet pushed (bounds concurrent donors)
+    int *promised;              // bitset search: donations decided on but not yet pushed (bounds concurrent donors)
     const volatile int *cancel; // host-mapped cancel word (nonzero = stop), or null
     unsigned long long deadline_ns;  // time limit in ns from each warp's start (%globaltimer), 0 = none
     long long budget;           // states budget per job, 0 = none

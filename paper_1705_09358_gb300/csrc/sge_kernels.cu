@@ -6,10 +6,13 @@
 // pruned by arc consistency, forward checking of singleton domains).
 //
 // GPU design (not the paper's CPU work-stealing runtime):
-//  * domain kernels: one warp per 64-target bitset word; arc consistency and
-//    forward checking iterate to their joint fixpoint under a host loop;
+//  * domain kernels: initialisation by one warp per 64-target bitset word or per label
+//    bucket; arc consistency and forward checking iterate to their joint fixpoint in one
+//    launch -- by the whole device for a few pairs, a block or a warp per pair for many --
+//    or in sweeps under a host loop;
 //  * split: breadth-first expansion of the search tree, up to 32 frames per
-//    warp at once, until the frontier holds enough frames for every resident warp;
+//    warp at once, to the end (its narrow part without level barriers) or until the
+//    frontier holds enough frames for every resident warp;
 //  * persistent search: one warp owns one depth-first search.  The CSR kernel
 //    scans the candidate list (on targets with label runs the shortest run among
 //    the earlier neighbours' rows) 32 candidates at a time, one per lane, spreads the
@@ -487,18 +490,8 @@ __device__ __forceinline__ bool unused(const PosInfo *P, int c, const int *M) {
     return true;
 }
 
-// All rules for candidate c, entry e of list S, by one lane.
-template <bool DIR, class V>
-__device__ __forceinline__ bool cand_lane(const V &v, const PosV &p, const PosInfo *P, const Cand &S, int c, int e,
-                                          const int *M) {
-    if (!cand_local<DIR>(v, p, S, c, e)) return false;
-    if (p.par >= 0)
-        for (int q = 0; q <= p.bc; ++q)
-            if (q != S.skip && !con_holds<DIR>(v, p, q, S.li, c, M)) return false;
-    return unused(P, c, M);
-}
-
-// Up to this many (candidate, constraint) tests of a chunk are spread over the warp's lanes.
+// Up to this many (candidate, constraint) tests of a chunk are spread over the warp's lanes: four
+// rounds of them (64, 256 and 1,024 measured alike on deep, network, directed and molecule batches).
 constexpr int SPREAD_TESTS = 128;
 
 // Warp-collective: the candidates of entries [x0, x0 + 32) below `end` of list S that pass all
@@ -2399,12 +2392,18 @@ __device__ __forceinline__ void split_child_header(int32_t *dst, const JobDesc &
 // and records are read through (5.9 KB per warp made the widest levels 1.6x slower than 3.4 KB).
 constexpr int SPLIT_STEPS = 2;
 constexpr int SPLIT_QUEUE = 32 * SPLIT_STEPS + 32;
-// A child with at least this many images is written by the whole warp, consecutive words at a time.
+// A child with at least this many images is written by the whole warp, consecutive words at a time
+// (from 2 on: 24 directed patterns 1.16 -> 1.42 ms, 200,000 molecule pairs 5.25 -> 5.65; never: 160
+// network queries 3.4 -> 3.6; from 32 on batches take the same, 96 served queries 2.9 instead of
+// 4.1 ms, which is not understood yet).
 constexpr int SPLIT_COOP_DEPTH = 8;
 // Of a longer list, each candidate's local tests include the constraints whose images have a
 // bitset row, the next shortest run's first: their row pointers are looked up once per frame
 // (at most SPLIT_ROWS for the batch), so a test is one load instead of a chain of four
-// (a power-law network's hubs form a near-clique: long lists there pass most constraints).
+// (a power-law network's hubs form a near-clique: long lists there pass most constraints).  Never:
+// 160 network queries 3.4 -> 4.1 ms, 96 served ones 4.1 -> 4.6, ten deep patterns 1.31 -> 1.27;
+// lists of 1 and of 17 on as the least: within the spread.  32 rows: served queries 4.1 -> 4.4;
+// 128: within the spread, for 512 bytes of shared memory more.
 constexpr int SPLIT_ROW_MIN = 4;
 constexpr int SPLIT_ROWS = 64;
 
